@@ -89,10 +89,10 @@ extern "C" {
 #define BURR_CUT_DIFF 3u          /* cut search: least (bumped by the cut) - (keys before it) */
 #define BURR_MAX_LAYERS 8
 #define BURR_FLAG_TIMING 1u       /* record per-stage device times (burr_stats) */
-#define BURR_FLAG_TEST_WINDOW 2u  /* testing only: the band treats a pivot 136 or more slots past
-                                     its bucket's first slot as leaving the on-chip window (the
-                                     BURR_ERR_INTERNAL path of a real window overflow, which needs
-                                     a pivot 382 or more slots past its row's start) */
+#define BURR_FLAG_TEST_WINDOW 2u  /* testing only: the band treats a row that is still without a
+                                     pivot 136 or more slots past its bucket's first slot as leaving
+                                     its window (drives the BURR_ERR_INTERNAL path; a row has its
+                                     pivot at most 190 slots past, and the window holds 256) */
 #define BURR_FLAG_TEST_SLACK 4u   /* testing only: a layer sorted in two scatter passes (more than
                                      2^16 buckets) sorts into bins of half their expected size, so
                                      that they overflow and the layer is sorted again exactly (the

@@ -3,126 +3,134 @@
 // ("Back Substitution" of Fig. 7).
 //
 // One warp per partition.  The paper gives one partition to one CPU thread,
-// which eliminates the rows one by one.  Here the 32 lanes of a warp insert a
-// bucket together:
+// which eliminates the rows one by one against a stored band.  Here the warp
+// sweeps the slots of its partition from left to right instead and settles one
+// slot per step:
 //
-//   * The kept set of a bucket does not depend on the order of its rows
-//     inside a threshold band: the threshold is the smallest level t such
-//     that the rows kept so far plus the bucket's rows with offset >= t are
-//     linearly independent, and independence is a property of the set.  The
-//     table does not depend on it either (unique solution with free slots 0).
-//   * So the warp first inserts the whole bucket as one set.  Most buckets
-//     insert without a dependency.  If the set is dependent it is rolled back
-//     and, with 2-bit thresholds, the rows [l1, B), then [l2, B), are tried as
-//     one set each until one inserts, which fixes the threshold exactly as the
-//     row-by-row elimination in descending offset order would.
-//   * With 1+-bit thresholds (exact threshold t in [0, B]) t is the least
-//     value for which the rows at offsets >= t insert.  The first pass over
-//     the bucket carries row tags and drops dependent rows instead of
-//     stopping.  The dropped rows' tags span the set's dependencies, and t
-//     follows from them (insert_tagged).  The rows at offsets >= t are then
-//     inserted again as one set.  Where the tags cannot place a dependency,
-//     t is found by probes instead: a set of rows is independent whenever a
-//     superset is, so each probe inserts the rows of [mid, t_ok) on top of
-//     those already kept and either keeps them (t_ok = mid) or rolls them
-//     back (t_fail = mid).
-//   * A set is inserted as a stream: the 32 lanes eliminate one row each and
-//     take their steps in lockstep.  A step is one 128-bit compare-and-swap
-//     on the ring slot of the row's leading bit, which either claims the
-//     slot if it is empty (row and right-hand side stored in one atomic
-//     write) or returns the stored row and right-hand side to XOR with.  Plain
-//     reads of the next two slots are in flight beside the swap, and the
-//     elimination goes on through those that hold stored rows.  This
-//     is a sequential insertion in claim order: every slot a row eliminated
-//     against was occupied when read and stays so, and a row is stored only
-//     on a slot that was still empty.  Lanes whose row was stored take the
-//     next rows of the set, and the stored slots are listed for a rollback,
-//     by ballot and prefix count; a dependent row ends the set at once.
-//   * Rows are staged per bucket in shared memory in ascending offset order
-//     (a counting sort on the 7-bit offset), so each threshold band is a
-//     contiguous range and rows that run through the dense overflow of the
-//     previous buckets start first.
-//   * The live part of the band, [bucket start, bucket start + 512), sits in a
-//     shared-memory ring per warp; slots left behind are final and are
-//     written to the global band in coalesced runs.
+//   * A row is live from its start slot until it becomes the pivot row of a
+//     slot.  At slot j every live row has its support in [j, j + 63], so at
+//     most 64 of them are independent, and they fit in registers: two rows per
+//     lane, as 64 coefficient bits (bit of slot s at position s mod 64, so
+//     that nothing is shifted from slot to slot), the right-hand side and a
+//     key.
+//   * A step picks, among the live rows with bit j, the one of the highest
+//     priority (one warp maximum over keys), stores it as slot j's row and
+//     XORs it into the others.  No row meets more than one stored row per step
+//     and none waits for another lane's chain of eliminations.
+//   * Priority is the paper's insertion order: rows of earlier buckets first,
+//     then descending offset.  A row is then only ever changed by rows that are
+//     inserted before it, so a row that becomes zero is dependent on them, as
+//     in the row-by-row elimination in descending offset order; with offset o
+//     its bucket's threshold is the least one above o.  The rows at offsets
+//     >= t and the slots they hold are untouched by the rows below t, so
+//     bumping is just dropping the rows below t and emptying their slots:
+//     nothing is rolled back or inserted again, in either threshold mode.
+//   * Rows of bucket b may turn out dependent up to 63 slots into bucket b + 1,
+//     whose rows they have changed by then.  The live rows at the bucket
+//     boundary are therefore kept in shared memory, and bucket b + 1 starts
+//     again from them without the dropped rows (a few percent of the buckets).
+//   * More live rows than registers means more than 64 rows in 64 slots, so a
+//     dependency: the lowest-offset row of the bucket cannot be kept, and the
+//     threshold above it is taken at once.
+//
+// What bounds it: with every warp slot taken, the ALU pipe (integer logic,
+// selects and compares at half rate: 79% busy at 10^9 keys, 43 warp
+// instructions per key); with few partitions, the chain of a step (bit test,
+// warp maximum, shuffle, XOR: ~95 cycles per slot).  Layer-0 band, ms (r = 8
+// unless said), against the streaming insertion that it replaces (32 lanes
+// eliminating one row each against a band in shared memory, a 128-bit
+// compare-and-swap per step, every bucket as long as its longest chain, a
+// dependent bucket inserted again):
+//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 3.2
+//   10^6 keys (16 partitions)                     6.57 -> 4.4
+//   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 7.7
+//   10^8 keys (1504 partitions)                   8.33 -> 6.9;  1+-bit 16.3 -> 10.6
+//   10^9 keys (15034 partitions)                  63.7 -> 50.5
 #include "burr_internal.cuh"
 
 namespace burr {
 
 namespace {
 
-constexpr int kRing = 512;
+constexpr int kRing = 256;              // stored rows kept on chip: a bucket and the one before it
 constexpr uint32_t kRingMask = kRing - 1;
-constexpr int kStage = 256;             // rows of a bucket staged at once
+constexpr int kStage = 192;             // rows of a bucket staged at once (see stage_rows)
 constexpr int kStagePerLane = kStage / 32;
-// Partitions (warps) per CTA.  Small CTAs spread partitions evenly over the
-// SMs (1503 partitions at 10^8 keys fill ~10 of the 12 warp slots per SM) and
-// give a finer tail; 2 measured best against 1 and 4.
-#ifndef BURR_BAND_WARPS
-#define BURR_BAND_WARPS 2
-#endif
-constexpr int kBandWarps = BURR_BAND_WARPS;
 constexpr unsigned kFull = 0xffffffffu;
+// Slots per round of the sweep's loop.  The whole sweep has to stay small: with
+// 16 slots unrolled and the sweep inlined for both halves of a bucket, the
+// warps of an SM, each at its own place in the code, waited on instruction
+// fetches (layer-0 band of 10^9 keys 104.7 ms against 60.9 with 4 slots and
+// one copy); 1, 2, 4, 8 and 16 slots in one copy: 58.7, 55.2, 54.2, 54.5, 56.6.
+#ifndef BURR_BAND_UNROLL
+#define BURR_BAND_UNROLL 8
+#endif
+constexpr uint32_t kUnrollSlots = BURR_BAND_UNROLL;
+// CTAs (partitions) per SM that the kernel's registers allow: 64 registers a
+// thread.  Layer-0 band of 10^9 keys with 16, 14 and 12: 50.5, 53.3, 55.4 ms.
+#ifndef BURR_BAND_CTAS
+#define BURR_BAND_CTAS 16
+#endif
 
-constexpr unsigned long long kYValid = 1ull << 32;   // marks a stored right-hand side
+// Key of a live row: bit 30 = row of an earlier bucket, bits 22..29 = offset + 1,
+// bit 21 = which of the lane's two rows, bits 0..4 = lane (so that a key is a
+// shuffle's source lane as it is); 0 = no row.  Bits 5..20 hold the right-hand
+// side when it has at most 16 bits: the maximum over keys that finds the pivot
+// then brings its right-hand side along.
+constexpr uint32_t kOldKey = 1u << 30;
+constexpr uint32_t kOffsetBit = 22, kRowBit = 21, kValueBit = 5;
+constexpr uint32_t kValueMask = 0xffffu << kValueBit;
+__device__ __forceinline__ uint32_t key_offset(uint32_t key) { return ((key >> kOffsetBit) & 0xffu) - 1u; }
 
-struct alignas(16) RingSlot {
-    unsigned long long c;   // stored coefficient row (bit 0 = pivot), 0 = empty
-    unsigned long long y;   // kYValid | right-hand side (low r bits); 0 = empty
+// A live row: w1:w0 are its 64 coefficient bits relative to the block of slots
+// being swept (rotated right by the block's length after it), so that the
+// block's slots are the low bits of w0.  A row that starts inside the block
+// ignores the slots before its start (whose positions hold its last bits).
+struct Row {
+    uint32_t w0, w1, key, y, gate;   // y: right-hand sides of more than 16 bits
+};
+
+// A stored row of the ring, as it was live at its slot: rotated by the slot's
+// place in its block, which is kept in y (in the key's value bits where y is
+// taken).  key 0 = empty slot.
+struct alignas(16) Pivot {
+    uint32_t w0, w1, key, y;
 };
 
 // A staged equation: one 16-byte read hands it to a lane.
 struct alignas(16) StagedRow {
-    unsigned long long c;   // coefficient row (bit 0 = start slot)
+    uint32_t lo, hi;        // coefficient row (bit 0 = start slot)
     uint32_t y;             // right-hand side
     uint32_t o;             // offset of the start slot in its bucket
 };
 
-// Ring slots read ahead of the swap in each step (see stream_insert), per
-// threshold mode: more read-ahead means fewer steps but more instructions per
-// step, and with many warps per SM competing for issue slots two measured
-// best in both modes (10^8 keys, r=8; 1+-bit: 1, 2, 3, 4 slots gave 27.2,
-// 26.6, 27.5, 27.6 ms per build and query step; 2-bit, layer-0 band of 10^9
-// keys: 68.2, 65.9, 69.0, 80.1 ms).
-#ifndef BURR_BAND_LOOKAHEAD_2BIT
-#define BURR_BAND_LOOKAHEAD_2BIT 2
-#endif
-#ifndef BURR_BAND_LOOKAHEAD_1PLUS
-#define BURR_BAND_LOOKAHEAD_1PLUS 2
-#endif
-template <bool kExact>
-struct Lookahead {
-    static constexpr int value = kExact ? BURR_BAND_LOOKAHEAD_1PLUS : BURR_BAND_LOOKAHEAD_2BIT;
-    static_assert(value >= 0 && value <= 8, "lookahead out of range");
+// What one warp works on: a partition of one structure's layer, and where that
+// structure's data sits in the layer-wide arrays (all bases 0 for a single
+// structure).  It sits in shared memory: it is read once per bucket or less, and
+// held in registers it took 60 of them.
+struct Ctx {
+    LayerDesc L;
+    uint32_t part;
+    uint64_t bucket_base, slot_base, tw_base, out_base;
+    uint64_t own_hi;         // one past the partition's slots
+    uint32_t b0, b1;         // its buckets
+    uint32_t pend;           // end of its equations
+    unsigned long long *bcount;
+    uint32_t *fail;          // base case, batched: per-structure flag
 };
-// Read-ahead of a 2-bit launch whose partitions are all resident at once (a
-// layer of few partitions): the SMs then have issue slots to spare, each warp's
-// chain of steps sets the time, and a third slot saves steps.  Measured with
-// every partition resident: layer-0 band of 10^8 keys 8.54 -> 8.35 ms, of 2^25
-// keys 6.96 -> 6.75 ms; when partitions outnumber the resident warps (10^9
-// keys) the extra registers cost a CTA per SM: 63.7 -> 71.4 ms.
-constexpr int kLookFew = 3;
-constexpr int kMaxOf(int a, int b) { return a > b ? a : b; }
-constexpr int kLookMax = kMaxOf(kMaxOf(Lookahead<false>::value, Lookahead<true>::value), kLookFew);
 
-// Tagged sets (1+-bit thresholds): the kTagRows lowest-offset rows of the set
-// carry one bit each in bits 33.. of the right-hand-side word, and a row's tag
-// travels with every XOR, so a row that reduces to zero names the rows of the
-// set that its dependency runs through.
-constexpr uint32_t kTagRows = 31;
-
-__device__ __forceinline__ unsigned long long row_tag(uint32_t k) {
-    return k < kTagRows ? 1ull << (33u + k) : 0ull;
-}
-
-struct BandWarpSmem {
-    RingSlot ring[kRing + kLookMax];   // live band window (+ read-ahead pad: zero, never written)
-    uint16_t clist[kRing];         // ring indices stored by the current set (rollback)
-    StagedRow rows[kStage];        // staged equations, ascending offset
-    uint32_t first[132];           // first staged index of each offset (+ [128] = count)
-    uint32_t ncommit;              // entries of clist
-    uint32_t nfail;                // rows of a tagged set that reduced to zero
-    uint32_t ftag[kTagRows];       // their tags (the first kTagRows of them)
+struct BandSmem {
+    Pivot ring[kRing];             // stored rows of slots [bucket start - B, bucket start + B)
+    StagedRow rows[2][kStage];     // staged equations of two buckets, ascending offset
+    uint32_t first[2][132];        // first staged index of each offset (+ [128] = count)
+    uint32_t tstage[2];            // threshold the bucket starts from
+    uint32_t tdone;                // final threshold of the bucket before the one being swept
+    // an error was recorded in the first or second half of a bucket: both warps leave at that
+    // half's barrier (one flag per half, or a warp could see the other's next half's flag)
+    uint32_t stop[2];
+    uint32_t sweeper;              // the warp that sweeps
+    Pivot snap[2][32];             // live rows at the bucket's start
+    Ctx x;
 };
 
 template <typename V>
@@ -142,70 +150,21 @@ struct BandArgs {
     BatchView bv;            // sd == nullptr: a single layer described by L
 };
 
-// What one warp works on: a partition of one structure's layer, and where that
-// structure's data sits in the layer-wide arrays (all bases 0 for a single
-// structure).
-struct Ctx {
-    LayerDesc L;
-    uint64_t part;
-    uint64_t bucket_base, slot_base, tw_base, out_base;
-    unsigned long long *bcount;
-    uint32_t *fail;          // base case, batched: per-structure flag
-};
-
-enum { kOk = 0, kDependent = 1, kOverflow = 2 };
-
-// Pivots at or past bucket start + this many slots leave the live window: the
-// ring less the read-ahead, so that the slots a step reads ahead of its pivot
-// are still inside the window and never alias the window's first slots (a
-// smaller window when a test asks for one).
-constexpr uint32_t kWindow = (uint32_t)(kRing - kLookMax);
-__device__ __forceinline__ uint32_t window_of(const LayerDesc &L) {
-    return L.window ? min(L.window, kWindow) : kWindow;
+// Least threshold of the layer's mode at or above o (o <= B).
+__device__ __forceinline__ uint32_t threshold_from(const LayerDesc &L, uint32_t o) {
+    if (L.mode == BURR_THRESH_1PLUS) return o;
+    if (o == 0) return 0;
+    return o <= L.levels[1] ? L.levels[1] : (o <= L.levels[2] ? L.levels[2] : L.levels[3]);
 }
 
-__device__ __forceinline__ void rollback(BandWarpSmem &S, uint32_t ncommit, int lane) {
-    __syncwarp();
-    for (uint32_t i = lane; i < ncommit; i += 32) {
-        const uint32_t ri = S.clist[i];
-        S.ring[ri].c = 0;
-        S.ring[ri].y = 0;
-    }
-    __syncwarp();
-}
-
-// Stage rows [base, base+cnt) (cnt <= kStage) of the bucket starting at slot
-// bB: equations in ascending offset order; S.first[o] = first index with
-// offset >= o.  A call, not inline code: inlined at its call sites, staging
-// kept registers live across the elimination loops (166 registers in the 2-bit
-// kernel, over 240 in the 1+-bit one); as a call both take 128, so 8 CTAs of 2
-// warps fit per SM instead of 6.  Measured: equal at 10^8 keys (all partitions
-// resident either way), layer-0 band 76.9 -> 68.2 ms at 10^9 keys.
-template <typename V>
-__device__ __noinline__ void stage_rows(BandWarpSmem &S, const BandArgs<V> &a, const Ctx &x, uint32_t base, uint32_t cnt,
-                           uint32_t bB, int lane) {
-    const LayerDesc &L = x.L;
-    for (int i = lane; i < 132; i += 32) S.first[i] = 0;
-    __syncwarp();
-    uint64_t c[kStagePerLane];
-    uint32_t y[kStagePerLane], o[kStagePerLane], rank[kStagePerLane];
+// Exclusive scan of first[0..128) in place, first[128] = total.
+__device__ __forceinline__ void scan_first(uint32_t *first, int lane) {
+    uint32_t v[4], loc = 0;
 #pragma unroll
-    for (int j = 0; j < kStagePerLane; ++j) {
-        const uint32_t i = (uint32_t)lane + 32u * j;
-        if (i < cnt) {
-            const uint64_t h = a.keys[base + i];     // the record h of the key
-            const uint32_t s = start_of_h(h, L.range);
-            c[j] = coeff_of_h(h, L.sigma);
-            o[j] = s - bB;
-            y[j] = (uint32_t)a.vals[base + i] & L.vmask;
-            rank[j] = atomicAdd(&S.first[o[j]], 1u);
-        }
+    for (int k = 0; k < 4; ++k) {
+        v[k] = first[4 * lane + k];
+        loc += v[k];
     }
-    __syncwarp();
-    // exclusive scan of the 128 offset counts, 4 per lane
-    uint32_t v0 = S.first[4 * lane], v1 = S.first[4 * lane + 1], v2 = S.first[4 * lane + 2],
-             v3 = S.first[4 * lane + 3];
-    const uint32_t loc = v0 + v1 + v2 + v3;
     uint32_t incl = loc;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -214,348 +173,101 @@ __device__ __noinline__ void stage_rows(BandWarpSmem &S, const BandArgs<V> &a, c
     }
     __syncwarp();
     uint32_t run = incl - loc;
-    S.first[4 * lane] = run;
-    run += v0;
-    S.first[4 * lane + 1] = run;
-    run += v1;
-    S.first[4 * lane + 2] = run;
-    run += v2;
-    S.first[4 * lane + 3] = run;
-    if (lane == 31) S.first[128] = incl;
-    __syncwarp();
 #pragma unroll
-    for (int j = 0; j < kStagePerLane; ++j) {
-        const uint32_t i = (uint32_t)lane + 32u * j;
-        if (i < cnt) {
-            const uint32_t p = S.first[o[j]] + rank[j];
-            S.rows[p] = StagedRow{c[j], y[j], o[j]};
-        }
+    for (int k = 0; k < 4; ++k) {
+        first[4 * lane + k] = run;
+        run += v[k];
     }
+    if (lane == 31) first[128] = incl;
     __syncwarp();
 }
 
-// 128-bit compare-and-swap on a ring slot: if the slot is (0, 0) it becomes
-// (c, y); the previous contents are returned either way.
-__device__ __forceinline__ void slot_cas(unsigned addr, unsigned long long c, unsigned long long y,
-                                         unsigned long long &oc, unsigned long long &oy) {
-    const unsigned long long zero = 0ull;
-    asm volatile("{\n\t.reg .b128 d, b, v;\n\t"
-                 "mov.b128 b, {%2, %2};\n\t"
-                 "mov.b128 v, {%3, %4};\n\t"
-                 "atom.shared.cas.b128 d, [%5], b, v;\n\t"
-                 "mov.b128 {%0, %1}, d;\n\t}"
-                 : "=l"(oc), "=l"(oy)
-                 : "l"(zero), "l"(c), "l"(y), "r"(addr)
-                 : "memory");
-}
-
-// Plain read of a ring slot, as 32-bit words: the row's two halves and the
-// low word of the right-hand side; the right-hand side's high word (the tags
-// of a tagged set) only when kHi (a sink otherwise, so it takes no register).
-// A slot goes from empty to its final contents once per set (one atomic write
-// of row and right-hand side), and a step's reads are issued only after the
-// previous step's swaps have returned (their addresses depend on them), so a
-// read sees a slot either empty (all zero) or with both words of a stored
-// equation that stays.
-template <bool kHi>
-__device__ __forceinline__ void slot_load_words(unsigned addr, uint32_t &clo, uint32_t &chi, uint32_t &ylo,
-                                                uint32_t &yhi) {
-    if (kHi) {
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(clo), "=r"(chi), "=r"(ylo), "=r"(yhi)
-                     : "r"(addr)
-                     : "memory");
-    } else {
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, _}, [%3];" : "=r"(clo), "=r"(chi), "=r"(ylo) : "r"(addr) : "memory");
-        yhi = 0u;
-    }
-}
-
-// Stream staged rows [lo, hi) (index range) into the band; stored ring
-// indices are appended to S.clist (from S.ncommit).  Returns kOk, kDependent
-// or kOverflow; nothing is rolled back here.  Every lane takes one step per
-// iteration; stores, the commit list and the hand-out of the next rows go by
-// ballot and prefix count, with no shared atomics besides the swaps.
-//
-// Lookahead: beside the swap on the slot of its leading bit p, a lane reads
-// the slots p+1 .. p+kLook with plain loads (in flight together with the
-// swap).  When the swap returns a stored row, elimination goes on through
-// those slots without another round trip: a slot read as occupied holds a
-// final equation, so XORing it is the step the swap would have taken; the
-// step ends at the first leading bit whose slot was not read as occupied,
-// and the next swap goes there.  The row is kept as 64 bits from p plus the
-// kLook bits beyond p+63 that the read-ahead rows bring in.
-//
-// kTag: the rows carry tags (see kTagRows), and a row that reduces to zero does
-// not end the set: its tag is listed in S.ftag (count in S.nfail, from 0), the
-// row is dropped and its lane takes the next one.  This is a sequential
-// insertion in claim order that skips the dependent rows, so each dropped row
-// gives one dependency of the set on the band and the rows stored before it,
-// and together they span all of the set's dependencies.  The result is then
-// kDependent if any row was dropped; a ring overflow still ends the set.
-template <int kLook, bool kTag = false>
-__device__ int stream_insert(BandWarpSmem &S, uint32_t lo, uint32_t hi, uint32_t bB, uint32_t wlim, int lane) {
-    if (hi <= lo) return kOk;
-    const unsigned lt = (1u << lane) - 1u;
-    const unsigned ring0 = (unsigned)__cvta_generic_to_shared(&S.ring[0]);
-    uint32_t nc = S.ncommit;
-    // tagged: index of the next row to hand out; untagged: that index less the rows stored
-    uint32_t next = kTag ? lo + 32u : lo + 32u - nc;
-    bool has = lo + (uint32_t)lane < hi;
-    // a lane without a row swaps (0, 0) in, which leaves every slot as it was
-    unsigned long long cur = 0, y = 0;
-    uint32_t pos = bB;
-    if (has) {
-        const StagedRow r = S.rows[lo + (uint32_t)lane];
-        cur = r.c;
-        y = kYValid | r.y;
-        if (kTag) y |= row_tag((uint32_t)lane);
-        pos = bB + r.o;
-    }
-    uint32_t nf = 0;
-    bool pend = false;   // tagged: the lane's row was dropped; it takes the next one
-    int result = kOk;
-    for (;;) {
-        const uint32_t ri = pos & kRingMask;
-        const unsigned addr = ring0 + ri * (unsigned)sizeof(RingSlot);
-        // Read-ahead: the pivot lies below bB + wlim <= bB + kRing - kLook, so the slots read
-        // ahead are inside the window; past the ring's end they are the zero pad, which reads
-        // as empty (the step then ends there, and the next swap goes to the true slot).
-        unsigned long long oc, oy;
-        uint32_t lcl[kLook > 0 ? kLook : 1], lch[kLook > 0 ? kLook : 1], lyl[kLook > 0 ? kLook : 1],
-            lyh[kLook > 0 ? kLook : 1];
-#pragma unroll
-        for (int j = 0; j < kLook; ++j)
-            slot_load_words<kTag>(addr + (unsigned)((j + 1) * sizeof(RingSlot)), lcl[j], lch[j], lyl[j], lyh[j]);
-        slot_cas(addr, cur, y, oc, oy);
-        // an empty slot is all zero and a stored row has its pivot bit set
-        const bool stored = has && ((uint32_t)oc & 1u) == 0u;
-
-        // Hand-out first: the next row's shared read is in flight during the elimination.
-        const bool take = stored || (kTag && pend);
-        // untagged, every stored row frees its lane for the next row: the next row handed out
-        // is row lo + 32 + (rows stored so far), and a lane's commit-list entry gives its index
-        const unsigned sm = __ballot_sync(kFull, stored);
-        const unsigned tm = kTag ? __ballot_sync(kFull, take) : sm;
-        const uint32_t ci = nc + (uint32_t)__popc(sm & lt);
-        const uint32_t nidx = kTag ? next + (uint32_t)__popc(tm & lt) : ci + next;
-        const bool nhas = take && nidx < hi;
-        StagedRow nr = StagedRow{0ull, 0u, 0u};
-        if (nhas) nr = S.rows[nidx];
-        if (stored) S.clist[ci] = (uint16_t)ri;
-        nc += (uint32_t)__popc(sm);
-        if (kTag) next += (uint32_t)__popc(tm);
-
-        // Elimination for lanes whose swap returned a stored row: against that row, then through
-        // the read-ahead slots.  The row is (over : hi32 : lo32), bit j = slot pos + j; bit 0 is
-        // now clear.  Which read-ahead rows are used depends only on the low word, so the
-        // decisions run on 32 bits and the other words are XORed afterwards, all at once.
-        const bool act = has && !stored;
-        uint32_t lo32 = (uint32_t)cur ^ (uint32_t)oc;
-        uint32_t hi32 = (uint32_t)(cur >> 32) ^ (uint32_t)(oc >> 32);
-        uint32_t over = 0;
-        uint32_t y2 = (uint32_t)y ^ (uint32_t)oy;   // right-hand sides fit in 32 bits
-        uint32_t yh = kTag ? (uint32_t)(y >> 32) ^ (uint32_t)(oy >> 32) : 0u;   // tags (bits 1..)
-        // while go is 1, bits 0 .. j-1 are clear, so bit j is the leading bit if set; a stored row
-        // has its pivot bit (bit 0) set.  Decisions as 0/1 words and all-ones masks: measured
-        // 5.7% fewer instructions than with predicates and selects (layer-0 band 65.8 -> 63.9 ms
-        // at 10^9 keys).
-        uint32_t go = 1u;
-        uint32_t um[kLook > 0 ? kLook : 1];   // 0 or all ones: the read-ahead row of slot pos+j is used
-#pragma unroll
-        for (int j = 1; j <= kLook; ++j) {
-            const uint32_t occ = lcl[j - 1] & 1u;
-            const uint32_t bit = (lo32 >> j) & 1u;
-            um[j - 1] = 0u - (go & bit & occ);
-            lo32 ^= (lcl[j - 1] << j) & um[j - 1];
-            go &= (bit ^ 1u) | occ;
-        }
-#pragma unroll
-        for (int j = 1; j <= kLook; ++j) {
-            hi32 ^= __funnelshift_l(lcl[j - 1], lch[j - 1], (unsigned)j) & um[j - 1];
-            over ^= (lch[j - 1] >> (32 - j)) & um[j - 1];
-            y2 ^= lyl[j - 1] & um[j - 1];
-            if (kTag) yh ^= lyh[j - 1] & um[j - 1];
-        }
-        // normalise: shift the leading bit (>= 1 for an active lane) down to bit 0; it is
-        // almost always in the low word
-        int tz = __ffs((int)lo32) - 1;
-        uint32_t n0 = __funnelshift_r(lo32, hi32, (unsigned)tz), n1 = __funnelshift_r(hi32, over, (unsigned)tz);
-        bool zero = false;
-        if (act && lo32 == 0u) {
-            zero = (hi32 | over) == 0u;
-            if (hi32) {
-                tz = 31 + __ffs((int)hi32);
-                n0 = __funnelshift_r(hi32, over, (unsigned)(tz - 32));
-                n1 = over >> (tz - 32);
-            } else {
-                tz = 63 + __ffs((int)over);
-                n0 = over >> ((tz - 64) & 31);
-                n1 = 0;
-            }
-        }
-        const uint32_t npos = pos + (uint32_t)tz;
-        const bool dep = act && zero;
-        const bool ovf = act && !zero && npos - bB >= wlim;
-        if (act) {
-            cur = ((unsigned long long)n1 << 32) | n0;
-            y = kTag ? ((unsigned long long)(yh | 1u) << 32) | y2 : kYValid | y2;
-            pos = npos;
-        }
-        if (take) {
-            has = nhas;
-            cur = nr.c;
-            y = nhas ? kYValid | nr.y : 0ull;
-            if (kTag && nhas) y |= row_tag(nidx - lo);
-            if (nhas) pos = bB + nr.o;
-            pend = false;
-        }
-        const unsigned bm = __ballot_sync(kFull, dep || ovf);
-        unsigned hm = __ballot_sync(kFull, has);
-        if (bm) {
-            const unsigned om = __ballot_sync(kFull, ovf);
-            if (!kTag || om) {
-                result = om ? kOverflow : kDependent;
-                break;
-            }
-            // tagged: list the dropped rows' tags; their lanes swap (0, 0) once and then take the
-            // next rows
-            const uint32_t dr = (uint32_t)__popc(bm & lt);
-            if (dep) {
-                if (nf + dr < kTagRows) S.ftag[nf + dr] = yh >> 1;
-                has = false;
-                cur = 0;
-                y = 0;
-                pend = true;
-            }
-            nf += (uint32_t)__popc(bm);
-            hm = __ballot_sync(kFull, has || (pend && next < hi));
-        }
-        if (!hm) break;
-    }
-    __syncwarp();
-    if (lane == 0) {
-        S.ncommit = nc;
-        if (kTag) S.nfail = nf;
-    }
-    __syncwarp();
-    if (kTag && result == kOk && nf) result = kDependent;
-    return result;
-}
-
-// Insert the rows of bucket [rs, re) whose offset lies in [olo, ohi) as one
-// set; on a dependency or overflow every row this call stored is removed.
-// kL: slots read ahead per step.
-template <typename V, bool kExact, int kL = Lookahead<kExact>::value>
-__device__ int insert_set(BandWarpSmem &S, const BandArgs<V> &a, const Ctx &x, uint32_t rs, uint32_t re,
-                          uint32_t bB, uint32_t olo, uint32_t ohi, uint32_t &staged_base, int lane) {
-    if (lane == 0) S.ncommit = 0;
-    __syncwarp();
-    for (uint32_t base = rs; base < re; base += kStage) {
-        const uint32_t cnt = min((uint32_t)kStage, re - base);
-        if (staged_base != base) {
-            stage_rows(S, a, x, base, cnt, bB, lane);
-            staged_base = base;
-        }
-        const int rc = stream_insert<kL>(S, S.first[olo], S.first[ohi], bB, window_of(x.L), lane);
-        if (rc != kOk) {
-            rollback(S, S.ncommit, lane);
-            if (rc == kOverflow && lane == 0) atomicOr(a.err, kErrRingOverflow);
-            return rc;
-        }
-    }
-    return kOk;
-}
-
-constexpr uint32_t kTagUnknown = 0xffffffffu;
-
-// 1+-bit threshold of a bucket whose rows fit one stage, from one tagged pass
-// over its rows at offsets >= forced.  The set's dependencies form a space D
-// spanned by the dropped rows' dependency vectors (one per dropped row).  The
-// rows at offsets >= t insert iff no nonzero vector of D lies inside them, so
-// the least such t is one above the largest, over D, of the lowest offset a
-// vector contains.  Row i of the set (ascending offset) is tag bit i for
-// i < kTagRows, every later row sits at an offset at least as high, and a tag
-// is the vector's restriction to the tagged rows: after a reduction of the
-// tags to distinct lowest bits, the largest lowest bit b gives t = offset of
-// row b + 1.  A tag that reduces to zero means a dependency among untagged
-// rows only, which the tags cannot place: kTagUnknown.
-// Returns forced if the set inserts (its rows stay in the band), else t with
-// nothing of the set left in the band, kTagUnknown (same), or B + 1 on a ring
-// overflow.
+// Stage the rows of bucket [rs, re) (start slot bB) at offsets >= the returned
+// threshold, in ascending offset order; first[o] = first index with offset
+// >= o.  The rows at offsets >= o span 63 + B - o slots, so where there are
+// more of them the threshold is above o; the rows left after that (at most
+// 63 + B) always fit the stage.  Otherwise returns `forced` and stages every
+// row (the sweep skips those below the threshold).  A call, not inline code:
+// its registers would stay live across the sweep.
 template <typename V>
-__device__ uint32_t insert_tagged(BandWarpSmem &S, const BandArgs<V> &a, const Ctx &x, uint32_t rs, uint32_t re,
-                                  uint32_t bB, uint32_t forced, uint32_t &staged, int lane) {
-    if (staged != rs) {
-        stage_rows(S, a, x, rs, re - rs, bB, lane);
-        staged = rs;
-    }
-    if (lane == 0) S.ncommit = 0;
+__device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, const BandArgs<V> &a, const LayerDesc &L,
+                                            uint32_t rs, uint32_t re, uint32_t bB, uint32_t forced, int lane) {
+    const uint32_t cnt = re - rs;
+    for (int i = lane; i < 132; i += 32) first[i] = 0;
     __syncwarp();
-    const uint32_t lo = S.first[forced];
-    const int rc = stream_insert<Lookahead<true>::value, true>(S, lo, S.first[x.L.B], bB, window_of(x.L), lane);
-    const uint32_t nc = S.ncommit;
-    if (rc == kOk) {
-        for (uint32_t i = lane; i < nc; i += 32) S.ring[S.clist[i]].y &= kYValid | 0xffffffffull;   // drop the tags
+    if (cnt <= (uint32_t)kStage) {
+        uint64_t c[kStagePerLane];
+        uint32_t y[kStagePerLane], at[kStagePerLane];   // at: offset, and rank among its rows from bit 8
+#pragma unroll
+        for (int j = 0; j < kStagePerLane; ++j) {
+            const uint32_t i = (uint32_t)lane + 32u * j;
+            if (i < cnt) {
+                const uint64_t h = a.keys[rs + i];     // the record h of the key
+                c[j] = coeff_of_h(h, L.sigma);
+                const uint32_t o = start_of_h(h, L.range) - bB;
+                y[j] = (uint32_t)a.vals[rs + i] & L.vmask;
+                at[j] = o | atomicAdd(&first[o], 1u) << 8;
+            }
+        }
+        __syncwarp();
+        scan_first(first, lane);
+#pragma unroll
+        for (int j = 0; j < kStagePerLane; ++j) {
+            const uint32_t i = (uint32_t)lane + 32u * j;
+            if (i < cnt) {
+                const uint32_t o = at[j] & 0xffu;
+                rows[first[o] + (at[j] >> 8)] = StagedRow{(uint32_t)c[j], (uint32_t)(c[j] >> 32), y[j], o};
+            }
+        }
         __syncwarp();
         return forced;
     }
-    rollback(S, nc, lane);
-    if (rc == kOverflow) {
-        if (lane == 0) atomicOr(a.err, kErrRingOverflow);
-        return x.L.B + 1u;
+    // more rows than can be kept: count, find the threshold, stage the rows above it
+    for (uint32_t i = rs + lane; i < re; i += 32) atomicAdd(&first[start_of_h(a.keys[i], L.range) - bB], 1u);
+    __syncwarp();
+    scan_first(first, lane);
+    uint32_t over = 0;   // one above the largest offset o with more than 63 + B - o rows at offsets >= o
+    for (uint32_t o = lane; o < L.B; o += 32)
+        if (cnt - first[o] > 63u + L.B - o) over = o + 1;
+    over = __reduce_max_sync(kFull, over);
+    const uint32_t t = max(forced, threshold_from(L, over));
+    __syncwarp();
+    for (int i = lane; i < 132; i += 32) first[i] = 0;
+    __syncwarp();
+    for (uint32_t i = rs + lane; i < re; i += 32) {
+        const uint32_t o = start_of_h(a.keys[i], L.range) - bB;
+        if (o >= t) atomicAdd(&first[o], 1u);
     }
-    const uint32_t nf = S.nfail;
-    if (nf > kTagRows) return kTagUnknown;
-    uint32_t v = (uint32_t)lane < nf ? S.ftag[lane] : 0u;
-    bool piv = false;
-    int top = -1;
-    for (int b = 0; b < (int)kTagRows; ++b) {
-        const unsigned cand = __ballot_sync(kFull, !piv && ((v >> b) & 1u));
-        if (!cand) continue;
-        const int p = __ffs((int)cand) - 1;
-        const uint32_t pv = __shfl_sync(kFull, v, p);
-        if (lane == p) piv = true;
-        else if ((cand >> lane) & 1u) v ^= pv;
-        top = b;
+    __syncwarp();
+    scan_first(first, lane);
+    // place the rows: the cursor of offset o is first[o] itself, which then ends where offset
+    // o + 1 starts
+    for (uint32_t i = rs + lane; i < re; i += 32) {
+        const uint64_t h = a.keys[i];
+        const uint32_t o = start_of_h(h, L.range) - bB;
+        if (o >= t) {
+            const uint64_t c = coeff_of_h(h, L.sigma);
+            const uint32_t p = atomicAdd(&first[o], 1u);
+            rows[p] = StagedRow{(uint32_t)c, (uint32_t)(c >> 32), (uint32_t)a.vals[i] & L.vmask, o};
+        }
     }
-    if (__ballot_sync(kFull, (uint32_t)lane < nf && !piv) || top < 0) return kTagUnknown;
-    return S.rows[lo + (uint32_t)top].o + 1u;
-}
-
-// Offsets above the failing threshold tried first (8, 12, 16 and 24 measured;
-// 8 and 16 tied at 10^8 keys when every failing bucket was searched by probes).
-constexpr uint32_t kFirstProbe = 16;
-
-// 1+-bit threshold of a bucket whose rows at offsets >= forced are dependent,
-// by probes (where the tagged pass cannot decide it): the least t for which
-// the rows at offsets >= t insert, those rows left inserted.  Rows at offsets
-// >= t_fail are dependent, those >= t_ok are kept; exact thresholds are mostly
-// small (a few rows at the lowest offsets), so the first probe keeps all but
-// the lowest 16 offsets and bisection follows.  Returns B + 1 on a ring
-// overflow.
-template <typename V>
-__device__ __forceinline__ uint32_t exact_threshold(BandWarpSmem &S, const BandArgs<V> &a, const Ctx &x, uint32_t rs,
-                                                 uint32_t re, uint32_t bB, uint32_t forced, uint32_t &staged,
-                                                 int lane) {
-    uint32_t t_fail = forced, t_ok = x.L.B;
-    bool first = true;
-    while (t_ok - t_fail > 1) {
-        const uint32_t mid = (first && t_fail + kFirstProbe < t_ok) ? t_fail + kFirstProbe : (t_fail + t_ok) >> 1;
-        first = false;
-        const int rc = insert_set<V, true>(S, a, x, rs, re, bB, mid, t_ok, staged, lane);
-        if (rc == kOverflow) return x.L.B + 1u;
-        if (rc == kOk) t_ok = mid;
-        else t_fail = mid;
-    }
-    return t_ok;
+    __syncwarp();
+    uint32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = first[4 * lane + k];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) first[4 * lane + k + 1] = v[k];
+    if (lane == 0) first[0] = 0;
+    __syncwarp();
+    return t;
 }
 
 // Rows of the bucket below threshold t leave for the next layer (as keys: the
 // next layer hashes them with its own seed).
 template <typename V>
-__device__ void emit_bumped(const BandArgs<V> &a, const Ctx &x, uint32_t rs, uint32_t re, uint32_t bB,
-                            uint32_t t, int lane) {
+__device__ __noinline__ void emit_bumped(const BandArgs<V> &a, const Ctx &x, uint32_t rs, uint32_t re, uint32_t bB,
+                                         uint32_t t, int lane) {
     for (uint32_t base = rs; base < re; base += 32) {
         const uint32_t idx = base + lane;
         bool bump = false;
@@ -582,175 +294,377 @@ __device__ void emit_bumped(const BandArgs<V> &a, const Ctx &x, uint32_t rs, uin
     }
 }
 
-// Write ring slots [from, to) to the global band and clear them.
+// Write the ring's slots [from, to) to the global band.
 template <typename V>
-__device__ __forceinline__ void flush(BandWarpSmem &S, const BandArgs<V> &a, const Ctx &x, uint64_t from,
+__device__ __forceinline__ void flush(BandSmem &S, const BandArgs<V> &a, const Ctx &x, uint64_t from,
                                       uint64_t to, int lane) {
     __syncwarp();
     for (uint64_t s = from + lane; s < to; s += 32) {
-        const uint32_t ri = (uint32_t)s & kRingMask;
-        a.Cg[x.slot_base + s] = S.ring[ri].c;
-        a.Yg[x.slot_base + s] = (V)(S.ring[ri].y & 0xffffffffull);
-        S.ring[ri].c = 0;
-        S.ring[ri].y = 0;
+        const Pivot e = S.ring[(uint32_t)s & kRingMask];
+        const uint32_t v = (e.key & kValueMask) >> kValueBit;
+        const uint32_t q = sizeof(V) <= 2 ? e.y : v;
+        const uint32_t lo = __funnelshift_r(e.w0, e.w1, q), hi = __funnelshift_r(e.w1, e.w0, q);
+        a.Cg[x.slot_base + s] = e.key ? ((uint64_t)hi << 32) | lo : 0ull;
+        a.Yg[x.slot_base + s] = e.key ? (V)(sizeof(V) <= 2 ? v : e.y) : (V)0;
     }
     __syncwarp();
 }
 
-// kExact: 1+-bit thresholds (exact per bucket) instead of 2-bit codes; a
-// template parameter so that each mode gets its own register allocation.  kL:
-// slots read ahead per step (see kLookFew).
-template <typename V, bool kExact, int kL = Lookahead<kExact>::value>
-// All 1504 layer-0 partitions of 10^8 keys are resident at once when the
-// kernel takes at most 170 registers (six CTAs of two warps per SM).  Measured
-// with staging inline: at 186 registers (5 CTAs per SM) the layer-0 band took
-// 15.5 ms instead of 9.7; with a 128-register cap (spills inside the
-// elimination loop) 13.4 ms.  With staging as a call it takes 128 without
-// such spills (see stage_rows).  The 2-bit kernel for values wider than a
-// byte at two slots of read-ahead gets an explicit bound of 8 CTAs per SM:
-// without it ptxas gave it 139 registers (7 CTAs per SM; r = 16 at 10^9 keys:
-// layer-0 band 67.4 -> 72.7 ms); the other instantiations keep the bound on
-// threads alone (0 below), under which the one-byte kernel measured fastest.
-__global__ void __launch_bounds__(32 * kBandWarps, (sizeof(V) > 1 && !kExact && kL == 2) ? 8 : 0)
-    k_band(BandArgs<V> a) {
-    __shared__ BandWarpSmem smem[kBandWarps];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint64_t gp = (uint64_t)blockIdx.x * kBandWarps + warp;
-    Ctx x;
+// The live row of staged row r, relative to the block that starts at offset o.
+template <bool kPacked>
+__device__ __forceinline__ void load_row(Row &R, const StagedRow &r, uint32_t o, uint32_t id) {
+    const uint32_t q = r.o - o;              // < 32
+    R.w0 = __funnelshift_l(r.hi, r.lo, q);   // the row rotated left by its start's position
+    R.w1 = __funnelshift_l(r.lo, r.hi, q);
+    R.y = kPacked ? 0u : r.y;
+    R.gate = kFull << q;
+    R.key = ((r.o + 1u) << kOffsetBit) | id | (kPacked ? r.y << kValueBit : 0u);
+}
+
+// The slots from the w-th on become the low bits of w0 (w <= 32).
+__device__ __forceinline__ void rotate_row(Row &R, uint32_t w) {
+    const uint32_t w0 = R.w0;
+    R.w0 = __funnelshift_rc(w0, R.w1, w);
+    R.w1 = __funnelshift_rc(R.w1, w0, w);
+}
+
+// Drop a live row of this bucket (old: of the one before) below threshold t.
+__device__ __forceinline__ void drop_row(Row &R, bool old, uint32_t t) {
+    if (R.key && (R.key >= kOldKey) == old && key_offset(R.key) < t) R.w0 = R.w1 = R.key = 0;
+}
+
+// Empty the ring's slots [from, from + n) held by rows of their own bucket below t.
+__device__ __forceinline__ void drop_slots(BandSmem &S, uint32_t from, uint32_t n, uint32_t t, int lane) {
+    __syncwarp();
+    for (uint32_t i = lane; i < n; i += 32) {
+        Pivot &e = S.ring[(from + i) & kRingMask];
+        if (e.key && e.key < kOldKey && key_offset(e.key) < t) e.key = 0;
+    }
+    __syncwarp();
+}
+
+
+// One slot: the live row of the highest key with bit `mask` is stored at `e`
+// (place c of the block) and XORed into every other such row.  Without such a
+// row every lane writes key 0 (an empty slot) and nothing changes.
+//
+// What a step costs (measured on the GB300, cycles of an SM quarter per warp
+// instruction): LOP3, SEL, ISETP 2 each, max 1, warp maximum 2, shuffle 4,
+// ballot 4, popc and find-first-bit 8, a 16-byte exchange through shared memory
+// about 20.  So the pivot's lane comes out of the maximum itself (its low
+// bits) instead of a ballot and a find-first, and the pivot travels by three
+// shuffles.
+template <bool kPacked>
+__device__ __forceinline__ void sweep_slot(Row &A, Row &B, uint32_t mask, unsigned slot, uint32_t c) {
+    const uint32_t xa = A.w0 & A.gate & mask, xb = B.w0 & B.gate & mask;
+    const uint32_t ka = xa ? A.key : 0u, kb = xb ? B.key : 0u;
+    const bool second = kb > ka;
+    const uint32_t s0 = second ? B.w0 : A.w0, s1 = second ? B.w1 : A.w1, sk = max(ka, kb),
+                   sy = kPacked ? 0u : (second ? B.y : A.y);
+    const uint32_t ek = kPacked || sk == 0u ? sk : sk | c << kValueBit, ey = kPacked ? c : sy;
+    const uint32_t K = __reduce_max_sync(kFull, sk);
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %5, %6;\n\t@p st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}" ::"r"(slot),
+                 "r"(s0), "r"(s1), "r"(ek), "r"(ey), "r"(sk), "r"(K));
+    const uint32_t p0 = __shfl_sync(kFull, s0, (int)K), p1 = __shfl_sync(kFull, s1, (int)K);
+    const uint32_t py = kPacked ? K & kValueMask : __shfl_sync(kFull, sy, (int)K);
+    uint32_t &ya = kPacked ? A.key : A.y, &yb = kPacked ? B.key : B.y;
+    // predicated by hand: written as conditionals each XOR became a select besides
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p xor.b32 %0, %0, %4;\n\t@p xor.b32 %1, %1, %5;\n\t"
+        "@p xor.b32 %2, %2, %6;\n\t}"
+        : "+r"(A.w0), "+r"(A.w1), "+r"(ya)
+        : "r"(xa), "r"(p0), "r"(p1), "r"(py));
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p xor.b32 %0, %0, %4;\n\t@p xor.b32 %1, %1, %5;\n\t"
+        "@p xor.b32 %2, %2, %6;\n\t}"
+        : "+r"(B.w0), "+r"(B.w1), "+r"(yb)
+        : "r"(xb), "r"(p0), "r"(p1), "r"(py));
+}
+
+// The two warps of a partition meet.
+__device__ __forceinline__ void pair_sync() { asm volatile("bar.sync 0, 64;" ::: "memory"); }
+
+// The sweeping warp's state over its partition.
+struct Sweep {
+    Row A{0, 0, 0, 0, kFull}, B{0, 0, 0, 0, kFull};
+    uint32_t o = 0;        // next offset of the bucket
+    uint32_t t = 0;        // its threshold so far
+    uint32_t it = 0;       // staged index of its first row at or above t
+    uint32_t tprev = 0;    // the previous bucket's threshold
+    uint32_t fa = kFull, fb = kFull;   // lanes whose row A, B is free
+    __device__ __forceinline__ uint32_t nfree() const { return (uint32_t)(__popc(fa) + __popc(fb)); }
+    __device__ __forceinline__ void find_free() {
+        fa = __ballot_sync(kFull, A.key == 0);
+        fb = __ballot_sync(kFull, B.key == 0);
+    }
+};
+
+// Sweep offsets [W.o, lim) of the bucket at slot bB.  Returns false if the
+// build has to end (the error is recorded).
+template <typename V>
+__device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Sweep &W, uint32_t lim, uint32_t bB,
+                                         const StagedRow *rows, const uint32_t *first, uint32_t tstart, int lane) {
+    constexpr bool kPacked = sizeof(V) <= 2;
+    const LayerDesc &L = S.x.L;
+    const uint32_t lt = (1u << lane) - 1u;
+    Row &A = W.A, &B = W.B;
+    auto unsolvable = [&]() {
+        if (lane == 0) atomicOr(S.x.fail ? S.x.fail : a.err, kErrUnsolvable);
+        return false;
+    };
+    uint32_t nfree = W.nfree();
+    while (W.o < lim) {
+        const uint32_t o = W.o;
+        // the longest block of slots (up to 32) whose new rows fit the free registers
+        const uint32_t i0 = max(first[o], W.it);
+        const uint32_t upto = max(first[min(o + 1u + (uint32_t)lane, lim)], i0) - i0;   // rows that start in slots o .. o + lane
+        uint32_t w = (uint32_t)__popc(__ballot_sync(kFull, upto <= nfree && o + (uint32_t)lane < lim));
+        if (w == 0) {
+            // more than 64 rows in 64 slots: the lowest-offset row of the bucket goes
+            if (L.fallback) return unsolvable();
+            uint32_t low = o;
+            if (A.key && A.key < kOldKey) low = min(low, key_offset(A.key));
+            if (B.key && B.key < kOldKey) low = min(low, key_offset(B.key));
+            W.t = threshold_from(L, __reduce_min_sync(kFull, low) + 1u);
+            W.it = first[W.t];
+            drop_row(A, false, W.t);
+            drop_row(B, false, W.t);
+            drop_slots(S, bB, o, W.t, lane);
+            W.find_free();
+            nfree = W.nfree();
+            continue;
+        }
+        if (w > kUnrollSlots) w &= ~(kUnrollSlots - 1u);   // whole rounds of the unrolled loop
+        const uint32_t cnt = __shfl_sync(kFull, upto, (int)w - 1);
+        if (L.window && o < 64 && o + L.B >= L.window && __any_sync(kFull, max(A.key, B.key) >= kOldKey)) {
+            // testing only: a row would be stored past the window that the test asked for
+            if (lane == 0) atomicOr(a.err, kErrRingOverflow);
+            return false;
+        }
+        if (cnt == 0 && nfree == 64) {   // no live row: empty slots
+            if ((uint32_t)lane < w) S.ring[(bB + o + (uint32_t)lane) & kRingMask].key = 0;
+            W.o += w;
+            continue;
+        }
+        A.gate = B.gate = kFull;
+        const uint32_t ra = (uint32_t)__popc(W.fa & lt), rb = (uint32_t)(__popc(W.fa) + __popc(W.fb & lt));
+        if (A.key == 0 && ra < cnt) load_row<kPacked>(A, rows[i0 + ra], o, (uint32_t)lane);
+        if (B.key == 0 && rb < cnt) load_row<kPacked>(B, rows[i0 + rb], o, 1u << kRowBit | (uint32_t)lane);
+        const Pivot *e = &S.ring[(bB + o) & kRingMask];
+        const unsigned slot = (unsigned)__cvta_generic_to_shared(e);
+        uint32_t c = 0;
+#pragma unroll 1
+        for (; c + kUnrollSlots <= w; c += kUnrollSlots) {
+            const uint32_t mask = 1u << c;
+#pragma unroll
+            for (uint32_t k = 0; k < kUnrollSlots; ++k)
+                sweep_slot<kPacked>(A, B, mask << k, slot + (c + k) * (unsigned)sizeof(Pivot), c + k);
+        }
+#pragma unroll 1
+        for (; c < w; ++c) sweep_slot<kPacked>(A, B, 1u << c, slot + c * (unsigned)sizeof(Pivot), c);
+        rotate_row(A, w);
+        rotate_row(B, w);
+        asm volatile("" ::: "memory");   // the slots' stores
+        __syncwarp();
+        // free registers: a live row that is zero was stored in this block, or it is dependent
+        const bool za = (A.w0 | A.w1) == 0u, zb = (B.w0 | B.w1) == 0u;
+        const uint32_t K = (uint32_t)lane < w ? e[lane].key : 0u;
+        W.fa = __ballot_sync(kFull, za);
+        W.fb = __ballot_sync(kFull, zb);
+        const uint32_t np = (uint32_t)__popc(__ballot_sync(kFull, K != 0));
+        const uint32_t expect = nfree - cnt + np;
+        nfree = W.nfree();
+        W.o += w;
+        if (nfree == expect) {
+            if (za) A.key = 0;
+            if (zb) B.key = 0;
+            continue;
+        }
+        for (uint32_t k = 0; k < w; ++k) {   // the rows that were stored are free
+            const uint32_t x = __shfl_sync(kFull, K, (int)k);
+            if (x && ((x ^ A.key) & ~kValueMask) == 0u) A.key = 0;
+            if (x && ((x ^ B.key) & ~kValueMask) == 0u) B.key = 0;
+        }
+        const uint32_t D = __reduce_max_sync(kFull, max(za ? A.key : 0u, zb ? B.key : 0u));
+        if (L.fallback) return unsolvable();
+        if (D == 0 || (D >= kOldKey && o >= 64)) {   // not expected
+            if (lane == 0) atomicOr(a.err, kErrRingOverflow);
+            return false;
+        }
+        if (D < kOldKey) {
+            W.t = threshold_from(L, key_offset(D) + 1u);
+            drop_row(A, false, W.t);
+            drop_row(B, false, W.t);
+            drop_slots(S, bB, o + w, W.t, lane);
+        } else {
+            // the bucket before: bump its rows below the threshold above this row, and start this
+            // bucket again without them
+            W.tprev = threshold_from(L, key_offset(D) + 1u);
+            Pivot s = S.snap[0][lane];
+            A = Row{s.w0, s.w1, s.key, s.y, kFull};
+            s = S.snap[1][lane];
+            B = Row{s.w0, s.w1, s.key, s.y, kFull};
+            drop_row(A, true, W.tprev);
+            drop_row(B, true, W.tprev);
+            S.snap[0][lane] = Pivot{A.w0, A.w1, A.key, A.y};
+            S.snap[1][lane] = Pivot{B.w0, B.w1, B.key, B.y};
+            drop_slots(S, bB - L.B, L.B, W.tprev, lane);
+            W.t = tstart;
+            W.o = 0;
+        }
+        W.it = first[W.t];
+        W.find_free();
+        nfree = W.nfree();
+    }
+    return true;
+}
+
+// One CTA of two warps per partition.  One warp sweeps.  The other stages the next
+// bucket's rows during the first 64 slots of a bucket, and during the rest
+// writes out the bucket before, whose threshold and slots are final by then:
+// done by the sweeping warp itself these were a quarter of its time per
+// bucket.  Which warp sweeps alternates with the hardware warp slot: slots are
+// dealt to the four SM quarters in turn, and with warp 0 sweeping everywhere
+// the sweeps of an SM shared two of its quarters (layer-0 band of 10^8 keys
+// 16.4 ms).
+template <typename V>
+__global__ void __launch_bounds__(64, BURR_BAND_CTAS)
+k_band(BandArgs<V> a) {
+    __shared__ BandSmem S;
+    const int lane = threadIdx.x & 31;
+    Ctx &x = S.x;
+    uint64_t gp = blockIdx.x;
     if (a.bv.sd) {
         if (gp >= a.bv.nparts) return;
         if (a.bv.part_order) gp = a.bv.part_order[gp];   // longest partitions first
-        const uint32_t si = a.bv.part_struct[gp];
-        const StructDesc &D = a.bv.sd[si];
-        x.L = D.L;
-        x.part = gp - D.part_base;
-        x.bucket_base = D.bucket_base;
-        x.slot_base = D.slot_base;
-        x.tw_base = D.tw_base;
-        x.out_base = D.out_base;
-        x.bcount = a.bcount + si;
-        x.fail = a.bv.fail ? a.bv.fail + si : nullptr;
+        if (threadIdx.x == 0) {
+            const uint32_t si = a.bv.part_struct[gp];
+            const StructDesc &D = a.bv.sd[si];
+            x.L = D.L;
+            x.part = (uint32_t)(gp - D.part_base);
+            x.bucket_base = D.bucket_base;
+            x.slot_base = D.slot_base;
+            x.tw_base = D.tw_base;
+            x.out_base = D.out_base;
+            x.bcount = a.bcount + si;
+            x.fail = a.bv.fail ? a.bv.fail + si : nullptr;
+        }
     } else {
         gp += a.L.part_lo;
         if (gp >= part_end(a.L)) return;
-        x.L = a.L;
-        x.part = gp;
-        x.bucket_base = x.slot_base = x.tw_base = x.out_base = 0;
-        x.bcount = a.bcount;
-        x.fail = nullptr;
+        if (threadIdx.x == 0) {
+            x.L = a.L;
+            x.part = (uint32_t)gp;
+            x.bucket_base = x.slot_base = x.tw_base = x.out_base = 0;
+            x.bcount = a.bcount;
+            x.fail = nullptr;
+        }
     }
     const LayerDesc &L = x.L;
-    const uint64_t part = x.part;
-    BandWarpSmem &S = smem[warp];
-
-    const uint64_t b0 = part_bucket(L, part);
-    const uint64_t b1 = part_bucket(L, part + 1);
-    const uint64_t own_lo = part_own_lo(L, part);
-    const uint64_t own_hi = part_own_hi(L, part);
-
-    for (int i = lane; i < kRing + kLookMax; i += 32) {   // the ring and its pad
-        S.ring[i].c = 0;
-        S.ring[i].y = 0;
+    if (threadIdx.x == 0) {
+        x.b0 = (uint32_t)part_bucket(L, x.part);
+        x.b1 = (uint32_t)part_bucket(L, x.part + 1);
+        x.own_hi = part_own_hi(L, x.part);
+        x.pend = a.bstart[x.bucket_base + x.b1];
+        S.stop[0] = S.stop[1] = 0;
+        uint32_t slot;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+        S.sweeper = (slot >> 2) & 1u;
     }
-    __syncwarp();
+    __syncthreads();
+    const uint32_t b0 = x.b0, b1 = x.b1, Bs = L.B;
 
-    uint32_t lv[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) lv[i] = L.levels[i];
-    const uint32_t fcode = L.forced_code;
-    const uint32_t flevel = lv[fcode & 3];
+    if ((threadIdx.x >> 5) == S.sweeper) {
+        Sweep W;
+        pair_sync();   // the first bucket is staged
+        // the last round, past the partition's buckets, only finishes the rows of the last one
+        for (uint32_t b = b0; b <= b1; ++b) {
+            const uint32_t q = b & 1u, bB = b * Bs;   // (low 32 bits of the start slot)
+            const uint32_t tstart = S.tstage[q];
+            if (W.A.key) W.A.key |= kOldKey;
+            if (W.B.key) W.B.key |= kOldKey;
+            S.snap[0][lane] = Pivot{W.A.w0, W.A.w1, W.A.key, W.A.y};
+            S.snap[1][lane] = Pivot{W.B.w0, W.B.w1, W.B.key, W.B.y};
+            W.tprev = W.t;
+            W.t = tstart;
+            W.it = S.first[q][tstart];
+            W.o = 0;
+#pragma unroll 1
+            for (uint32_t half = 0; half < 2; ++half) {
+                const uint32_t lim = half == 0 ? 64u : (b < b1 ? Bs : 64u);
+                const bool ok = sweep_to(S, a, W, lim, bB, S.rows[q], S.first[q], tstart, lane);
+                if (lane == 0) {
+                    S.tdone = W.tprev;
+                    if (!ok) S.stop[half] = 1;
+                }
+                pair_sync();
+                if (S.stop[half]) return;
+            }
+        }
+        return;
+    }
 
-    uint64_t flushed = own_lo;
-    uint64_t tword = 0, twi = b0 >> 5;
-    // bucket bounds are read one bucket ahead, and the next bucket's equations are
-    // prefetched into L2, so that staging does not wait on DRAM
-    const uint32_t *bst = a.bstart + x.bucket_base;
-    const uint32_t pend = bst[b1];   // end of the partition's equations
-    uint32_t nrs = b0 < b1 ? bst[b0] : 0, nre = b0 < b1 ? bst[b0 + 1] : 0;
-    for (uint64_t b = b0; b < b1; ++b) {
-        const uint64_t bB = b * L.B;
-        const uint32_t rs = nrs, re = nre;
-        nrs = re;
-        nre = b + 2 <= b1 ? bst[b + 2] : re;
+    uint64_t flushed = part_own_lo(L, x.part);
+    uint64_t tword = 0;
+    uint32_t rs = a.bstart[x.bucket_base + b0];   // first equation of the next bucket to stage
+    auto stage = [&](uint32_t b) {
+        const uint32_t q = b & 1u, re = a.bstart[x.bucket_base + b + 1];
+        uint32_t t = 0;
+        if (x.part > 0 && b == b0 && !L.fallback)
+            t = L.mode == BURR_THRESH_1PLUS ? kW : L.levels[L.forced_code & 3];   // after a cut
+        // the next bucket's equations are prefetched into L2
         if (lane < 16) {
             const uint32_t k = re + (uint32_t)lane * (128u / sizeof(uint64_t));
-            if (k < pend) prefetch_l2(a.keys + k);
+            if (k < x.pend) prefetch_l2(a.keys + k);
         } else if (lane < 24) {
             const uint32_t k = re + (uint32_t)(lane - 16) * (128u / sizeof(V));
-            if (k < pend) prefetch_l2(a.vals + k);
+            if (k < x.pend) prefetch_l2(a.vals + k);
         }
-        if (bB > flushed) {
-            flush(S, a, x, flushed, bB, lane);
-            flushed = bB;
+        const uint32_t ts = stage_rows(S.rows[q], S.first[q], a, L, rs, re, b * Bs, t, lane);
+        if (lane == 0) S.tstage[q] = ts;
+        rs = re;
+        if (ts > t && L.fallback) {
+            if (lane == 0) {
+                atomicOr(x.fail ? x.fail : a.err, kErrUnsolvable);
+                S.stop[0] = 1;
+            }
         }
-        const bool cut = (part > 0 && b == b0 && !L.fallback);
-        const uint32_t forced = cut ? (kExact ? (uint32_t)kW : flevel) : 0;
-        uint32_t code = cut ? fcode : 0;
-        uint32_t texact = forced;
-        if (re > rs) {
-            uint32_t staged = 0xffffffffu;
-            bool search = false;   // 1+-bit: find the threshold by probes
-            if (kExact && !L.fallback && re - rs <= (uint32_t)kStage) {
-                // one tagged pass gives the threshold; the search only where the tags do not decide
-                texact = insert_tagged(S, a, x, rs, re, (uint32_t)bB, forced, staged, lane);
-                if (texact == L.B + 1u) return;   // ring overflow (recorded)
-                if (texact != kTagUnknown && texact > forced) {
-                    const int rc = insert_set<V, kExact, kL>(S, a, x, rs, re, (uint32_t)bB, texact, L.B, staged, lane);
-                    if (rc == kOverflow) return;
-                    if (rc != kOk) texact = kTagUnknown;   // not expected: the rows at offsets >= t are independent
-                }
-                search = texact == kTagUnknown;
-            } else if (const int rc = insert_set<V, kExact, kL>(S, a, x, rs, re, (uint32_t)bB, forced, L.B, staged, lane);
-                       rc != kOk) {
-                if (rc == kOverflow) return;
-                if (L.fallback) {
-                    if (lane == 0) atomicOr(x.fail ? x.fail : a.err, kErrUnsolvable);
-                    return;
-                }
-                if (kExact) {
-                    search = true;
+    };
+    stage(b0);
+    pair_sync();
+    for (uint32_t b = b0; b <= b1; ++b) {
+        if (b + 1 < b1) {
+            stage(b + 1);
+        } else {                       // nothing more: no rows
+            for (int i = lane; i < 132; i += 32) S.first[(b + 1) & 1u][i] = 0;
+            if (lane == 0) S.tstage[(b + 1) & 1u] = 0;
+        }
+        pair_sync();
+        if (S.stop[0]) return;
+        if (b > b0) {
+            const uint32_t bp = b - 1, t = S.tdone;
+            const uint64_t end = min((uint64_t)b * Bs, x.own_hi);
+            if (end > flushed) {
+                flush(S, a, x, flushed, end, lane);
+                flushed = end;
+            }
+            if (!L.fallback) {
+                if (t > 0) emit_bumped(a, x, a.bstart[x.bucket_base + bp], a.bstart[x.bucket_base + b], bp * Bs, t, lane);
+                if (L.mode == BURR_THRESH_1PLUS) {
+                    if (lane == 0) a.texact[x.bucket_base + bp] = (uint8_t)t;
                 } else {
-                    // the set [forced, B) was just found dependent: the threshold is the least
-                    // level above `forced` whose rows [level, B) insert, each candidate tried as
-                    // one set (rolled back if dependent).  Nearly always the first one inserts,
-                    // so this is one stream; inserting the bands [64, 128) and [32, 64) one
-                    // after the other took two.
-                    code = 3;
-                    for (int k = 1; k <= 2; ++k) {
-                        if (lv[k] <= forced) continue;
-                        const int rc2 = insert_set<V, kExact, kL>(S, a, x, rs, re, (uint32_t)bB, lv[k], L.B, staged, lane);
-                        if (rc2 == kOverflow) return;
-                        if (rc2 == kOk) {
-                            code = (uint32_t)k;
-                            break;
-                        }
+                    const uint32_t code = t == 0 ? 0u : (t <= L.levels[1] ? 1u : (t <= L.levels[2] ? 2u : 3u));
+                    tword |= (uint64_t)code << (2 * (bp & 31));
+                    if ((b & 31u) == 0 || b == b1) {
+                        if (lane == 0 && tword)
+                            atomicOr((unsigned long long *)&a.thresh[x.tw_base + (bp >> 5)], (unsigned long long)tword);
+                        tword = 0;
                     }
                 }
             }
-            if (kExact && search) {
-                texact = exact_threshold(S, a, x, rs, re, (uint32_t)bB, forced, staged, lane);
-                if (texact > L.B) return;   // ring overflow (recorded)
-            }
-            const uint32_t t = kExact ? texact : lv[code];
-            if (!L.fallback && t > 0) emit_bumped(a, x, rs, re, (uint32_t)bB, t, lane);
         }
-        if (kExact && !L.fallback) {
-            if (lane == 0) a.texact[x.bucket_base + b] = (uint8_t)texact;
-            continue;
-        }
-        if (!L.fallback) {
-            if ((b >> 5) != twi) {
-                if (lane == 0 && tword)
-                    atomicOr((unsigned long long *)&a.thresh[x.tw_base + twi], (unsigned long long)tword);
-                tword = 0;
-                twi = b >> 5;
-            }
-            tword |= (uint64_t)code << (2 * (b & 31));
-        }
+        pair_sync();
+        if (S.stop[1]) return;
     }
-    if (!L.fallback && lane == 0 && tword)
-        atomicOr((unsigned long long *)&a.thresh[x.tw_base + twi], (unsigned long long)tword);
-    flush(S, a, x, flushed, own_hi, lane);
+    if (x.own_hi > flushed) flush(S, a, x, flushed, x.own_hi, lane);
 }
 
 // Back-substitution, right to left over the partition's owned slots, one
@@ -946,28 +860,9 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
     a.bcount = bcount;
     a.err = err;
     const uint64_t parts = bv ? bv->nparts : part_end(L) - L.part_lo;
-    const unsigned grid = (unsigned)((parts + kBandWarps - 1) / kBandWarps);
-    // the threshold mode is one for the whole launch (a batch shares its parameters)
-    cudaError_t e;
-    if (L.mode == BURR_THRESH_1PLUS && !L.fallback) {
-        if ((e = prefer_shared(k_band<V, true>)) != cudaSuccess) return e;
-        k_band<V, true><<<grid, 32 * kBandWarps, 0, st>>>(a);
-        return cudaGetLastError();
-    }
-    // 2-bit: the deeper read-ahead where every CTA of the launch is resident at once
-    if ((e = prefer_shared(k_band<V, false, kLookFew>)) != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_band<V, false, kLookFew>, 32 * kBandWarps, 0)) !=
-        cudaSuccess)
-        return e;
-    if ((uint64_t)grid <= (uint64_t)sms * (uint64_t)per_sm) {
-        k_band<V, false, kLookFew><<<grid, 32 * kBandWarps, 0, st>>>(a);
-    } else {
-        if ((e = prefer_shared(k_band<V, false>)) != cudaSuccess) return e;
-        k_band<V, false><<<grid, 32 * kBandWarps, 0, st>>>(a);
-    }
+    const cudaError_t e = prefer_shared(k_band<V>);
+    if (e != cudaSuccess) return e;
+    k_band<V><<<(unsigned)parts, 64, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -15,7 +15,7 @@ constexpr uint32_t kW = 64;                       // ribbon width (Sec. 2)
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;
 
 // error bits written by kernels into the build's device error word
-constexpr uint32_t kErrRingOverflow = 1u;         // a pivot left the on-chip window
+constexpr uint32_t kErrRingOverflow = 1u;         // a pivot left the band's window (only a test's window can be too small)
 constexpr uint32_t kErrUnsolvable = 2u;           // base case: an equation was dependent
 constexpr uint32_t kErrSortSlack = 4u;            // a sort bin of fixed capacity overflowed (sort again exactly)
 
@@ -96,7 +96,7 @@ struct LayerDesc {
     uint32_t forced_code;
     uint32_t vmask;      // (1 << r) - 1
     uint32_t mode;       // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
-    uint32_t window;     // pivots at or past bucket start + window leave the band's window (0 = the whole ring)
+    uint32_t window;     // testing: live rows this many slots past their bucket's start are an error (0 = no check)
     uint32_t test_slack; // 1: the fixed-capacity sort bins get half their expected size (testing the exact redo)
     uint32_t part_lo;    // band and back-substitution launches cover partitions [part_lo, part_hi)
     uint32_t part_hi;    // (0: up to K); a shard of a sharded build owns such a range

@@ -1,0 +1,44 @@
+"""The band sweep where it can go wrong: more rows than registers (loads far
+above one), more rows in a bucket than are staged at once, buckets of one
+block's worth of slots, values that travel inside the row keys (up to 16 bits)
+and beside them (17 and more), in both threshold modes.  Whole exports against
+the serial oracle, bit for bit."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2411_12365_gb300 import inputs as I
+from tests.export_format import describe_difference
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2411_12365_gb300 import burr  # noqa: E402
+
+B64 = dict(bucket_slots=64, levels=(0, 16, 40, 64))
+CASES = [
+    (20_011, 8, 0.5, {}),                          # sparse: empty blocks
+    (20_011, 16, 1.45, {}), (20_011, 17, 1.5, {}),   # around 192 rows per bucket
+    (30_000, 32, 3.0, {}), (30_000, 1, 12.0, {}),  # most rows bumped, layer after layer
+    (15_013, 8, 1.015, B64), (15_013, 24, 2.5, B64),
+    (127, 8, 1.015, {}), (130, 16, 1.015, {}), (64, 32, 1.0, {}),
+    (40_000, 8, 1.015, dict(partition_slots=128, min_partition_slots=0)),   # a cut at every bucket
+]
+
+
+@pytest.mark.parametrize("mode", [burr.THRESH_2BIT, burr.THRESH_1PLUS])
+@pytest.mark.parametrize("n,r,alpha,kw", CASES)
+def test_sweep_matches_oracle(n, r, alpha, kw, mode):
+    keys = I.keys_torch(n, "cuda", seed=n + r)
+    vals = I.values_torch(keys, r)
+    got = burr.build(keys, vals, r, threshold_mode=mode, load_factor=alpha, **kw).export()
+    v = vals.cpu().numpy()
+    names = {"bucket_slots": "B"}
+    ref = O.build(keys.cpu().numpy().view(np.uint64), v.view(f"u{v.dtype.itemsize}").astype(np.uint32), r=r,
+                  threshold_mode=mode, alpha=alpha, **{names.get(k, k): x for k, x in kw.items()})
+    assert ref.ok
+    want = ref.export()
+    assert got == want, describe_difference(got, want)
