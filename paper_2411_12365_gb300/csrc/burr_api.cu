@@ -504,6 +504,19 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
         CK(cudaMemsetAsync(blkseg, 0, dir_blocks(cap_nb) * 4, st), "clear threshold blocks");
     }
 
+    // scratch of the segmented band (launches of few partitions)
+    void *seg = nullptr;
+    size_t seg_bytes = 0;
+    auto band_scratch = [&](const LayerDesc &L) -> cudaError_t {
+        const size_t need = band_scratch_bytes(L);
+        if (need <= seg_bytes) return cudaSuccess;
+        if (seg) ar.release(seg);
+        seg_bytes = 0;
+        const cudaError_t e = ar.alloc(&seg, need);
+        if (e == cudaSuccess) seg_bytes = need;
+        return e;
+    };
+
     // A bumping layer's back-substitution is queued on the side stream only
     // after the next layer's sort: it fills every SM for milliseconds, and the
     // sort, queued behind it, used to wait that long (layer 1 of a 10^9-key
@@ -574,6 +587,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             CK(ar.alloc(&ygs[set], S.m * vb), "alloc band values");
             cgcap[set] = S.m;
         }
+        CK(band_scratch(L), "alloc band scratch");
         // the band of layer l overwrites the set that layer l-3 solved: wait for it
         CK(side.reuse(set), "order");
         // sorted with fixed-capacity bins where they fit the scratch; if a bin overflowed
@@ -647,7 +661,8 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
                 h->launches += 2;
             } else {
                 CK(launch_band(L, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cgs[set], ygs[set],
-                               S.thresh, tex, (uint64_t *)bk[which], bv[which], bcount, err, st), "band");
+                               S.thresh, tex, (uint64_t *)bk[which], bv[which], bcount, err, st, nullptr, seg), "band");
+                h->launches += band_kernel_count(L) - 1;
             }
             tev[l][2] = tm.mark();
             if (onep) CK(launch_thresh_flags(tex, dseg, blkseg, (uint32_t)nd, S.flags, tcounts, S.dir, st), "flags");
@@ -720,12 +735,13 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             CK(dev_alloc((void **)&F.z, (F.m / 64) * r * 8, st), "alloc table");
             CK(cudaMemsetAsync(ctr, 0, 64, st), "clear counters");
             const LayerDesc L = make_desc(p, r, cur_n, F.m, F.sigma, 1, true, F.m);
+            CK(band_scratch(L), "alloc band scratch");
             const int t0 = tm.mark();
             CK(launch_sort(L, vb, cur_k, cur_v, (uint64_t *)sk, sv, (uint32_t *)bst, ss, err, st), "sort");
             const int t1 = tm.mark();
             CK(launch_band(L, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cgs[set], ygs[set],
-                           nullptr, nullptr, nullptr, nullptr, bcount, err, st), "band");
-            h->launches += sort_kernel_count(L) + 1;
+                           nullptr, nullptr, nullptr, nullptr, bcount, err, st, nullptr, seg), "band");
+            h->launches += sort_kernel_count(L) + band_kernel_count(L);
             uint32_t he = 0;
             CK(cudaMemcpyAsync(&he, err, 4, cudaMemcpyDeviceToHost, st), "read error word");
             CK(cudaStreamSynchronize(st), "base case");
@@ -792,6 +808,8 @@ struct BatchTables {
     std::vector<uint32_t> part_order;   // partitions by decreasing length (the band's launch order)
     std::vector<uint64_t> tile_lo;
     std::vector<uint32_t> who;   // active index -> structure index
+    uint32_t max_len = 0;        // buckets of the longest partition
+    bool fallback = false;
     uint64_t nbuckets = 0, ngroups = 0, nparts = 0, slots = 0, tw = 0, zw = 0, nkeys = 0;
 };
 
@@ -870,6 +888,9 @@ int batch_tables(const burr_params &p, const std::vector<uint32_t> &r, const std
             len[T.sd[i].part_base + k] = x;
             lmax = std::max(lmax, x);
         }
+    // (cut search moves a cut by less than a partition)
+    T.max_len = lmax + (p.cut_search != BURR_CUT_NONE && !fb ? (uint32_t)(Pl / p.bucket_slots) : 0u);
+    T.fallback = fb;
     std::vector<uint32_t> at(lmax + 2, 0);
     for (const uint32_t x : len) ++at[lmax - x + 1];   // decreasing length
     for (uint32_t x = 1; x <= lmax + 1; ++x) at[x] += at[x - 1];
@@ -933,6 +954,8 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
     void *scratch = nullptr, *bst = nullptr;
     void *cgs[kBandSets] = {}, *ygs[kBandSets] = {};
     uint64_t cap_scratch = 0, cap_nb = 0, cgcap[kBandSets] = {};
+    void *seg = nullptr;        // of the segmented band (launches of few partitions)
+    size_t seg_bytes = 0;
     auto ensure_band = [&](int set, uint64_t slots) -> int {
         if (slots > cgcap[set]) {
             CK(side.reuse(set), "order");   // its previous user's back-substitution is done
@@ -1003,6 +1026,16 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         v.ntiles = (uint32_t)T.tile_struct.size();
         v.nbuckets = T.nbuckets;
         v.nkeys = T.nkeys;
+        v.max_len = T.max_len;
+        v.mode = p.threshold_mode;
+        v.fallback = T.fallback;
+        const size_t need = band_scratch_bytes(LayerDesc(), &v);
+        if (need > seg_bytes) {
+            if (seg) ar.release(seg);
+            seg_bytes = 0;
+            CK(ar.alloc(&seg, need), "alloc band scratch");
+            seg_bytes = need;
+        }
         return BURR_OK;
     };
     auto table_alloc = [&](size_t bytes, auto **d) -> cudaError_t {
@@ -1109,7 +1142,8 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
             for (auto *h : hs) h->launches += 2;
         } else {
             CK(launch_band(none, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cg, yg, th, tex,
-                           (uint64_t *)bk[w], bv2[w], bcount, err, st, &v), "band");
+                           (uint64_t *)bk[w], bv2[w], bcount, err, st, &v, seg), "band");
+            for (auto *h : hs) h->launches += band_kernel_count(none, &v) - 1;
         }
         const int t2 = tm.mark();
         ThreshSeg *dsegs = nullptr;
@@ -1194,7 +1228,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         CK(cudaMemsetAsync(ctr, 0, (size_t)S * 12 + 64, st), "clear counters");
         CK(launch_sort_batch(v, vb, cur_k, cur_v, (uint64_t *)sk, sv, (uint32_t *)bst, scratch, st), "sort");
         CK(launch_band(none, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cg, yg, nullptr, nullptr,
-                       (uint64_t *)bk[wfb], bv2[wfb], bcount, err, st, &v), "band");
+                       (uint64_t *)bk[wfb], bv2[wfb], bcount, err, st, &v, seg), "band");
         CK(launch_backsub(none, vb, (const uint64_t *)cg, yg, z, st, &v), "backsub");
         for (auto *h : hs) h->launches += 6;
         std::vector<uint32_t> f(left.size());

@@ -46,6 +46,8 @@
 //   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 7.7
 //   10^8 keys (1504 partitions)                   8.33 -> 6.9;  1+-bit 16.3 -> 10.6
 //   10^9 keys (15034 partitions)                  63.7 -> 50.5
+#include <algorithm>
+
 #include "burr_internal.cuh"
 
 namespace burr {
@@ -125,10 +127,12 @@ struct BandSmem {
     uint32_t first[2][132];        // first staged index of each offset (+ [128] = count)
     uint32_t tstage[2];            // threshold the bucket starts from
     uint32_t tdone;                // final threshold of the bucket before the one being swept
-    // an error was recorded in the first or second half of a bucket: both warps leave at that
-    // half's barrier (one flag per half, or a warp could see the other's next half's flag)
+    // why both warps leave at the barrier of the first or second half of a bucket (kRunError or
+    // kRunCoupled; one word per half, or a warp could see the other's next half's reason)
     uint32_t stop[2];
+    uint32_t at;                   // bucket where the last run ended
     uint32_t sweeper;              // the warp that sweeps
+    uint32_t failed;               // the build has failed already
     Pivot snap[2][32];             // live rows at the bucket's start
     Ctx x;
 };
@@ -148,13 +152,26 @@ struct BandArgs {
     unsigned long long *bcount;
     uint32_t *err;
     BatchView bv;            // sd == nullptr: a single layer described by L
+    // segmented launches (see k_band_seg)
+    uint32_t seg;            // buckets per segment
+    uint32_t nseg;           // segments of the longest partition
+    uint64_t *omask;         // per bucket: slots of its first 64 held by rows of the bucket before
+    struct Pivot *state[2];  // per segment: live rows at its end, as the last even and odd pass left them
+    uint32_t *moved[2];      // per segment: the last odd (even) pass left other rows than the passes before
 };
+
+enum { kRunDone = 0, kRunError = 1, kRunCoupled = 2 };
 
 // Least threshold of the layer's mode at or above o (o <= B).
 __device__ __forceinline__ uint32_t threshold_from(const LayerDesc &L, uint32_t o) {
     if (L.mode == BURR_THRESH_1PLUS) return o;
     if (o == 0) return 0;
     return o <= L.levels[1] ? L.levels[1] : (o <= L.levels[2] ? L.levels[2] : L.levels[3]);
+}
+
+// 2-bit code of threshold t.
+__device__ __forceinline__ uint32_t code_of(const LayerDesc &L, uint32_t t) {
+    return t == 0 ? 0u : (t <= L.levels[1] ? 1u : (t <= L.levels[2] ? 2u : 3u));
 }
 
 // Exclusive scan of first[0..128) in place, first[128] = total.
@@ -517,23 +534,20 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
     return true;
 }
 
-// One CTA of two warps per partition.  One warp sweeps.  The other stages the next
-// bucket's rows during the first 64 slots of a bucket, and during the rest
-// writes out the bucket before, whose threshold and slots are final by then:
-// done by the sweeping warp itself these were a quarter of its time per
-// bucket.  Which warp sweeps alternates with the hardware warp slot: slots are
-// dealt to the four SM quarters in turn, and with warp 0 sweeping everywhere
-// the sweeps of an SM shared two of its quarters (layer-0 band of 10^8 keys
-// 16.4 ms).
+// What one warp pair works on: buckets [b0, b1) of its partition.
+struct Run {
+    uint32_t b0, b1;
+    const Pivot *in = nullptr;   // live rows at b0 (64 of them); none: no live rows
+    Pivot *out = nullptr;        // live rows at b1 go here
+    bool compare = false;        // stop where the stored run over these buckets is met
+};
+
+// The partition (or segment's partition) of launch index gp; false if there is none.
 template <typename V>
-__global__ void __launch_bounds__(64, BURR_BAND_CTAS)
-k_band(BandArgs<V> a) {
-    __shared__ BandSmem S;
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ bool load_ctx(BandSmem &S, const BandArgs<V> &a, uint64_t gp) {
     Ctx &x = S.x;
-    uint64_t gp = blockIdx.x;
     if (a.bv.sd) {
-        if (gp >= a.bv.nparts) return;
+        if (gp >= a.bv.nparts) return false;
         if (a.bv.part_order) gp = a.bv.part_order[gp];   // longest partitions first
         if (threadIdx.x == 0) {
             const uint32_t si = a.bv.part_struct[gp];
@@ -549,7 +563,7 @@ k_band(BandArgs<V> a) {
         }
     } else {
         gp += a.L.part_lo;
-        if (gp >= part_end(a.L)) return;
+        if (gp >= part_end(a.L)) return false;
         if (threadIdx.x == 0) {
             x.L = a.L;
             x.part = (uint32_t)gp;
@@ -558,24 +572,89 @@ k_band(BandArgs<V> a) {
             x.fail = nullptr;
         }
     }
-    const LayerDesc &L = x.L;
     if (threadIdx.x == 0) {
-        x.b0 = (uint32_t)part_bucket(L, x.part);
-        x.b1 = (uint32_t)part_bucket(L, x.part + 1);
-        x.own_hi = part_own_hi(L, x.part);
+        x.b0 = (uint32_t)part_bucket(x.L, x.part);
+        x.b1 = (uint32_t)part_bucket(x.L, x.part + 1);
+        x.own_hi = part_own_hi(x.L, x.part);
         x.pend = a.bstart[x.bucket_base + x.b1];
-        S.stop[0] = S.stop[1] = 0;
         uint32_t slot;
         asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
         S.sweeper = (slot >> 2) & 1u;
+        // read once for the CTA: other CTAs may be setting it
+        S.failed = (*a.err & (kErrRingOverflow | kErrUnsolvable)) || (x.fail && *x.fail);
     }
     __syncthreads();
-    const uint32_t b0 = x.b0, b1 = x.b1, Bs = L.B;
+    return true;
+}
+
+// Whether the rows that buckets before bucket b left live at its start (slot
+// bB) span the same space, right-hand sides included, as those of the stored
+// run.  Each run's pivots of these rows, which lie in the bucket's first 64
+// slots, are an echelon basis of its space; `mine` and `theirs` are their slots.
+template <typename V>
+__device__ __forceinline__ bool same_space(BandSmem &S, const BandArgs<V> &a, uint64_t slot, uint32_t bB, uint64_t mine,
+                                           uint64_t theirs, int lane) {
+    if (mine != theirs) return false;
+    uint64_t *c = reinterpret_cast<uint64_t *>(&S.snap[0][0]);        // the snapshot is not needed any more
+    uint32_t *y = reinterpret_cast<uint32_t *>(c + 64);
+    __syncwarp();
+    for (int i = lane; i < 64; i += 32) {   // (the partition's slots reach at least 64 past its last bucket's start)
+        const bool has = (theirs >> i) & 1ull;
+        c[i] = has ? a.Cg[slot + i] << i : 0ull;
+        y[i] = has ? (uint32_t)a.Yg[slot + i] : 0u;
+    }
+    __syncwarp();
+    bool same = true;
+    for (int i = lane; i < 64; i += 32) {
+        if (!((mine >> i) & 1ull)) continue;
+        const Pivot e = S.ring[(bB + (uint32_t)i) & kRingMask];
+        const uint32_t v = (e.key & kValueMask) >> kValueBit, q = sizeof(V) <= 2 ? e.y : v;
+        uint64_t w = ((uint64_t)__funnelshift_r(e.w1, e.w0, q) << 32 | __funnelshift_r(e.w0, e.w1, q)) << i;
+        uint32_t z = sizeof(V) <= 2 ? v : e.y;
+        for (int n = 0; w && n < 64; ++n) {   // each step clears the lowest bit, or there is no row for it
+            const int p = __ffsll((long long)w) - 1;
+            if (!c[p]) break;
+            w ^= c[p];
+            z ^= y[p];
+        }
+        same &= w == 0 && z == 0;
+    }
+    same = __all_sync(kFull, same);
+    __syncwarp();
+    return same;
+}
+
+// Band the buckets of a run.  One warp of the pair sweeps.  The other stages
+// the next bucket's rows during the first 64 slots of a bucket, and during the
+// rest writes out the bucket before, whose threshold and slots are final by
+// then: done by the sweeping warp itself these were a quarter of its time per
+// bucket.  Which warp sweeps alternates with the hardware warp slot: slots are
+// dealt to the four SM quarters in turn, and with warp 0 sweeping everywhere
+// the sweeps of an SM shared two of its quarters (layer-0 band of 10^8 keys
+// 16.4 ms).
+//
+// kSeg: thresholds go to texact in either mode and no row is emitted
+// (k_band_finish does both), and what a later run needs to meet this one is kept.
+template <typename V, bool kSeg>
+__device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &a, const Run &R, int lane) {
+    const Ctx &x = S.x;
+    const LayerDesc &L = x.L;
+    const uint32_t b0 = R.b0, b1 = R.b1, Bs = L.B;
+    if (kSeg) pair_sync();               // the run before is done with the ring
+    if (threadIdx.x == 0) S.stop[0] = S.stop[1] = 0;
+    pair_sync();
 
     if ((threadIdx.x >> 5) == S.sweeper) {
         Sweep W;
+        if (kSeg && R.in) {
+            Pivot s = R.in[lane];
+            W.A = Row{s.w0, s.w1, s.key, s.y, kFull};
+            s = R.in[32 + lane];
+            W.B = Row{s.w0, s.w1, s.key, s.y, kFull};
+            W.find_free();
+        }
         pair_sync();   // the first bucket is staged
-        // the last round, past the partition's buckets, only finishes the rows of the last one
+        // the last round, past the run's buckets, only finishes the rows of the last one
         for (uint32_t b = b0; b <= b1; ++b) {
             const uint32_t q = b & 1u, bB = b * Bs;   // (low 32 bits of the start slot)
             const uint32_t tstart = S.tstage[q];
@@ -590,25 +669,40 @@ k_band(BandArgs<V> a) {
 #pragma unroll 1
             for (uint32_t half = 0; half < 2; ++half) {
                 const uint32_t lim = half == 0 ? 64u : (b < b1 ? Bs : 64u);
-                const bool ok = sweep_to(S, a, W, lim, bB, S.rows[q], S.first[q], tstart, lane);
+                uint32_t why = sweep_to(S, a, W, lim, bB, S.rows[q], S.first[q], tstart, lane) ? kRunDone : kRunError;
+                if (kSeg && half == 0 && why == kRunDone) {
+                    if (b < b1) {
+                        const uint32_t k0 = S.ring[(bB + lane) & kRingMask].key, k1 = S.ring[(bB + 32 + lane) & kRingMask].key;
+                        const uint64_t mine = (uint64_t)__ballot_sync(kFull, k1 >= kOldKey) << 32 |
+                                              __ballot_sync(kFull, k0 >= kOldKey);
+                        uint64_t *om = a.omask + x.bucket_base + b;
+                        if (R.compare && same_space(S, a, x.slot_base + (uint64_t)b * Bs, bB, mine, *om, lane)) why = kRunCoupled;
+                        else if (lane == 0) *om = mine;
+                    } else if (R.out) {
+                        R.out[lane] = S.snap[0][lane];
+                        R.out[32 + lane] = S.snap[1][lane];
+                    }
+                }
                 if (lane == 0) {
                     S.tdone = W.tprev;
-                    if (!ok) S.stop[half] = 1;
+                    S.at = b;
+                    if (why) S.stop[half] = why;
                 }
                 pair_sync();
-                if (S.stop[half]) return;
+                if (S.stop[half]) return S.stop[half];
             }
         }
-        return;
+        return kRunDone;
     }
 
-    uint64_t flushed = part_own_lo(L, x.part);
+    uint64_t flushed = b0 == x.b0 ? part_own_lo(L, x.part) : (uint64_t)b0 * Bs;
+    const uint64_t own_hi = b1 == x.b1 ? x.own_hi : (uint64_t)b1 * Bs;
     uint64_t tword = 0;
     uint32_t rs = a.bstart[x.bucket_base + b0];   // first equation of the next bucket to stage
     auto stage = [&](uint32_t b) {
         const uint32_t q = b & 1u, re = a.bstart[x.bucket_base + b + 1];
         uint32_t t = 0;
-        if (x.part > 0 && b == b0 && !L.fallback)
+        if (x.part > 0 && b == x.b0 && !L.fallback)
             t = L.mode == BURR_THRESH_1PLUS ? kW : L.levels[L.forced_code & 3];   // after a cut
         // the next bucket's equations are prefetched into L2
         if (lane < 16) {
@@ -624,7 +718,7 @@ k_band(BandArgs<V> a) {
         if (ts > t && L.fallback) {
             if (lane == 0) {
                 atomicOr(x.fail ? x.fail : a.err, kErrUnsolvable);
-                S.stop[0] = 1;
+                S.stop[0] = kRunError;
             }
         }
     };
@@ -638,21 +732,21 @@ k_band(BandArgs<V> a) {
             if (lane == 0) S.tstage[(b + 1) & 1u] = 0;
         }
         pair_sync();
-        if (S.stop[0]) return;
+        const uint32_t why = S.stop[0];
+        if (why == kRunError) return why;
         if (b > b0) {
             const uint32_t bp = b - 1, t = S.tdone;
-            const uint64_t end = min((uint64_t)b * Bs, x.own_hi);
+            const uint64_t end = min((uint64_t)b * Bs, own_hi);
             if (end > flushed) {
                 flush(S, a, x, flushed, end, lane);
                 flushed = end;
             }
             if (!L.fallback) {
-                if (t > 0) emit_bumped(a, x, a.bstart[x.bucket_base + bp], a.bstart[x.bucket_base + b], bp * Bs, t, lane);
-                if (L.mode == BURR_THRESH_1PLUS) {
+                if (!kSeg && t > 0) emit_bumped(a, x, a.bstart[x.bucket_base + bp], a.bstart[x.bucket_base + b], bp * Bs, t, lane);
+                if (kSeg || L.mode == BURR_THRESH_1PLUS) {
                     if (lane == 0) a.texact[x.bucket_base + bp] = (uint8_t)t;
                 } else {
-                    const uint32_t code = t == 0 ? 0u : (t <= L.levels[1] ? 1u : (t <= L.levels[2] ? 2u : 3u));
-                    tword |= (uint64_t)code << (2 * (bp & 31));
+                    tword |= (uint64_t)code_of(L, t) << (2 * (bp & 31));
                     if ((b & 31u) == 0 || b == b1) {
                         if (lane == 0 && tword)
                             atomicOr((unsigned long long *)&a.thresh[x.tw_base + (bp >> 5)], (unsigned long long)tword);
@@ -661,10 +755,113 @@ k_band(BandArgs<V> a) {
                 }
             }
         }
+        if (why) return why;           // the stored run goes on from here
         pair_sync();
-        if (S.stop[1]) return;
+        if (S.stop[1]) return S.stop[1];
     }
-    if (x.own_hi > flushed) flush(S, a, x, flushed, x.own_hi, lane);
+    if (own_hi > flushed) flush(S, a, x, flushed, own_hi, lane);
+    return kRunDone;
+}
+
+// One partition per CTA, from its first bucket to its last.
+template <typename V>
+__global__ void __launch_bounds__(64, BURR_BAND_CTAS)
+k_band(BandArgs<V> a) {
+    __shared__ BandSmem S;
+    if (!load_ctx(S, a, blockIdx.x)) return;
+    Run R{S.x.b0, S.x.b1};
+    run_buckets<V, false>(S, a, R, (int)(threadIdx.x & 31));
+}
+
+// Few partitions: each is banded in segments of a.seg buckets at the same time.
+//
+// A bucket's result depends on the buckets before it only through the rows
+// they leave live at its start, as a space (of equations, right-hand sides
+// included): thresholds are a property of sets, and any basis gives the same
+// solution.  Runs that start from different live rows soon leave the same
+// space (here: two runs from no live rows and from the true ones, over random
+// start buckets of a layer at load 1.015, 2-bit thresholds: after 15 buckets in
+// the median, 23 on average, 53 / 115 / 179 in 90 / 99 / 100% of 409 starts;
+// 1+-bit thresholds 34 / 58 on average).  So
+//   pass 0: every segment is banded from no live rows, and its live rows at the
+//           end are kept;
+//   pass 1: every segment but a partition's first is banded again from the rows
+//           that pass 0 left before it, up to the bucket where it meets its own
+//           stored run; a segment that never does leaves other rows than before;
+//   pass 2..: the same for the segments behind those;
+//   last:   one CTA per partition goes on behind what is left of them, in
+//           order, each time until the stored run is met (rare, but then as
+//           long as it takes).
+// In the end every bucket's stored threshold and slots follow from true live
+// rows, so the result does not depend on the segments.  k_band_finish then
+// emits the bumped rows.
+template <typename V>
+__global__ void __launch_bounds__(64, BURR_BAND_CTAS)
+k_band_seg(BandArgs<V> a, uint32_t nparts, uint32_t pass, bool last) {
+    __shared__ BandSmem S;
+    const uint32_t gp = last ? blockIdx.x : blockIdx.x % nparts, i = last ? 0 : blockIdx.x / nparts;
+    const uint64_t base = (uint64_t)gp * a.nseg;      // the partition's first segment
+    const uint64_t g = base + i;
+    const uint32_t now = pass & 1u, then = now ^ 1u;
+    // (a partition's first segment starts from true rows; what a segment behind a partition's end
+    // finds here does not matter)
+    if (!last && pass > 0 && (i == 0 || (pass > 1 && (i == 1 || !a.moved[then][g - 1])))) {
+        if (threadIdx.x == 0) a.moved[now][g] = 0;
+        return;
+    }
+    if (!load_ctx(S, a, gp) || (pass > 0 && S.failed)) return;   // after a failure the stored runs are incomplete
+    const int lane = (int)(threadIdx.x & 31);
+    const uint32_t b0 = S.x.b0, b1 = S.x.b1, n = (b1 - b0 + a.seg - 1) / a.seg;
+    if (!last) {
+        if (i >= n) return;
+        Run R{b0 + i * a.seg, min(b0 + (i + 1) * a.seg, b1)};
+        if (i + 1 < n) R.out = a.state[now] + g * 64;
+        if (pass > 0) {
+            R.in = a.state[then] + (g - 1) * 64;
+            R.compare = true;
+        }
+        const uint32_t why = run_buckets<V, true>(S, a, R, lane);
+        if (threadIdx.x == 0) a.moved[now][g] = why == kRunDone;
+        return;
+    }
+    for (uint32_t j = 2; j < n;) {
+        if (!a.moved[then][base + j - 1]) {
+            ++j;
+            continue;
+        }
+        Run R{b0 + j * a.seg, b1};
+        R.in = a.state[then] + (base + j - 1) * 64;
+        R.compare = true;
+        if (run_buckets<V, true>(S, a, R, lane) != kRunCoupled) return;
+        j = (S.at - b0) / a.seg + 1;
+    }
+}
+
+// After a segmented launch: emit the bumped rows of every bucket and pack the
+// 2-bit codes.  One CTA per 32 buckets of a partition (aligned to the code words).
+template <typename V>
+__global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t nparts) {
+    __shared__ BandSmem S;
+    if (!load_ctx(S, a, blockIdx.x % nparts) || S.failed) return;
+    const Ctx &x = S.x;
+    const int lane = (int)(threadIdx.x & 31);
+    const uint32_t warp = threadIdx.x >> 5;
+    const uint32_t w = (x.b0 >> 5) + blockIdx.x / nparts, b = w * 32u + (uint32_t)lane;
+    if (w * 32u >= x.b1) return;
+    const uint32_t t = b >= x.b0 && b < x.b1 ? a.texact[x.bucket_base + b] : 0u;
+    if (warp == 0 && x.L.mode != BURR_THRESH_1PLUS) {
+        const uint64_t c = (uint64_t)code_of(x.L, t) << (2 * lane);
+        const uint32_t lo = __reduce_or_sync(kFull, (uint32_t)c), hi = __reduce_or_sync(kFull, (uint32_t)(c >> 32));
+        if (lane == 0 && (lo | hi))
+            atomicOr((unsigned long long *)&a.thresh[x.tw_base + w], (unsigned long long)((uint64_t)hi << 32 | lo));
+    }
+    uint32_t left = __ballot_sync(kFull, t > 0);
+    for (uint32_t k = 0; left; ++k, left &= left - 1) {   // the bumping buckets, dealt to the warps in turn
+        if ((k & 3u) != warp) continue;
+        const int j = __ffs((int)left) - 1;
+        const uint32_t bj = w * 32u + (uint32_t)j, tj = __shfl_sync(kFull, t, j);
+        emit_bumped(a, x, a.bstart[x.bucket_base + bj], a.bstart[x.bucket_base + bj + 1], bj * x.L.B, tj, lane);
+    }
 }
 
 // Back-substitution, right to left over the partition's owned slots, one
@@ -841,10 +1038,58 @@ k_backsub_multi(LayerDesc L0, const uint64_t *__restrict__ Cg, const V *__restri
     }
 }
 
+// Segments of a launch: buckets per segment (0: whole partitions) and segments
+// of the longest partition.  A launch of few partitions is bound by their
+// chains (8.2 us per bucket, 512 buckets in a default partition) while most of
+// the chip idles.  Segments of 32 buckets are passed 2-6 times until the last
+// one has met its stored run; measured, layer-0 band in ms, whole partitions
+// against segments: 5*10^4 keys (1 partition) 3.2 / 0.80, 10^6 (16) 4.45 / 1.44,
+// 10^7 (151) 4.6 / 2.34, 3*10^7 (451, segments of 128) 4.7 / 3.5.  Segments of
+// 16 and 24 buckets at 10^6 keys: 1.49 / 1.49.  The passes bring about 23
+// buckets' work per segment, so a launch that fills the chip as it is keeps
+// whole partitions: the segment length grows until segments and partitions fit
+// the 2432 resident CTAs (16 per SM) together (a cap of 1216 / 3700: 2.79 / 2.85
+// at 10^7 keys; 10^8 keys, 1504 partitions, in segments of 128: 7.8 against 6.8).
+// Exact thresholds keep whole partitions: right-hand sides of different
+// bumped rows survive for 58 buckets on average there, and segments gave 5.0-5.6
+// against 5.6 ms at 10^6 keys and 8.1-8.6 against 7.7 at 10^7.
+constexpr uint64_t kSegCap = 2432, kSegMin = 32;
+constexpr uint32_t kSegPasses = 7;
+struct SegPlan {
+    uint32_t seg = 0, nseg = 0;
+    uint64_t parts = 0, buckets = 0;
+};
+SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
+    SegPlan p;
+    uint64_t total, longest;
+    if (bv) {
+        p.parts = bv->nparts;
+        total = bv->nbuckets;
+        longest = bv->max_len;
+        p.buckets = bv->nbuckets;
+    } else {
+        p.parts = part_end(L) - L.part_lo;
+        // partitions of P slots, the last one with the remainder; searched cuts move by less than P
+        longest = L.K <= 1 ? L.nb : std::max<uint64_t>(L.P / L.B, L.nb - (L.K - 1) * (L.P / L.B)) + (L.cuts ? L.P / L.B : 0);
+        total = std::min<uint64_t>(L.nb, p.parts * longest);
+        p.buckets = L.nb;
+    }
+    const uint32_t mode = bv ? bv->mode : L.mode;
+    const bool fallback = bv ? bv->fallback : L.fallback != 0;
+    if (mode == BURR_THRESH_1PLUS && !fallback) return p;
+    uint64_t seg = kSegMin;
+    while (p.parts + total / seg > kSegCap && seg * 2 <= longest) seg *= 2;
+    if (p.parts + total / seg > kSegCap || seg * 2 > longest) return p;
+    p.seg = (uint32_t)seg;
+    p.nseg = (uint32_t)((longest + seg - 1) / seg);
+    return p;
+}
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
 template <typename V>
 cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, const uint32_t *bstart,
                       uint64_t *Cg, V *Yg, uint64_t *thresh, uint8_t *texact, uint64_t *bkeys, V *bvals,
-                      unsigned long long *bcount, uint32_t *err, cudaStream_t st, const BatchView *bv) {
+                      unsigned long long *bcount, uint32_t *err, cudaStream_t st, const BatchView *bv, void *scratch) {
     BandArgs<V> a;
     if (bv) a.bv = *bv;
     a.L = L;
@@ -859,30 +1104,67 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
     a.bvals = bvals;
     a.bcount = bcount;
     a.err = err;
-    const uint64_t parts = bv ? bv->nparts : part_end(L) - L.part_lo;
-    const cudaError_t e = prefer_shared(k_band<V>);
-    if (e != cudaSuccess) return e;
-    k_band<V><<<(unsigned)parts, 64, 0, st>>>(a);
+    const SegPlan p = seg_plan(L, bv);
+    if (!scratch || !p.seg) {
+        const cudaError_t e = prefer_shared(k_band<V>);
+        if (e != cudaSuccess) return e;
+        k_band<V><<<(unsigned)p.parts, 64, 0, st>>>(a);
+        return cudaGetLastError();
+    }
+    char *q = (char *)scratch;
+    a.seg = p.seg;
+    a.nseg = p.nseg;
+    a.omask = (uint64_t *)q;
+    q += align256(p.buckets * 8);
+    for (int i = 0; i < 2; ++i) {
+        a.state[i] = (Pivot *)q;
+        q += align256(p.parts * p.nseg * 64 * sizeof(Pivot));
+    }
+    for (int i = 0; i < 2; ++i) {
+        a.moved[i] = (uint32_t *)q;
+        q += align256(p.parts * p.nseg * 4);
+    }
+    if (!a.texact) a.texact = (uint8_t *)q;
+    const uint32_t parts = (uint32_t)p.parts;
+    const bool fallback = bv ? bv->fallback : L.fallback != 0;
+    cudaError_t e;
+    if ((e = prefer_shared(k_band_seg<V>)) != cudaSuccess || (e = prefer_shared(k_band_finish<V>)) != cudaSuccess) return e;
+    for (uint32_t pass = 0; pass < kSegPasses; ++pass) k_band_seg<V><<<parts * p.nseg, 64, 0, st>>>(a, parts, pass, false);
+    k_band_seg<V><<<parts, 64, 0, st>>>(a, parts, kSegPasses, true);
+    // a partition's buckets may start inside a code word
+    if (!fallback) k_band_finish<V><<<parts * (p.nseg * p.seg / 32 + 2), 128, 0, st>>>(a, parts);
     return cudaGetLastError();
 }
 
 }  // namespace
 
+size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv) {
+    if (bv ? bv->nparts == 0 : part_end(L) <= L.part_lo) return 0;
+    const SegPlan p = seg_plan(L, bv);
+    if (!p.seg) return 0;
+    return align256(p.buckets * 8) + align256(p.buckets) + 2 * align256(p.parts * p.nseg * 64 * sizeof(Pivot)) +
+           2 * align256(p.parts * p.nseg * 4);
+}
+
+uint32_t band_kernel_count(const LayerDesc &L, const BatchView *bv) {
+    return band_scratch_bytes(L, bv) == 0 ? 1u : kSegPasses + ((bv ? bv->fallback : L.fallback != 0) ? 1u : 2u);
+}
+
 cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *keys, const void *vals,
                         const uint32_t *bucket_start, uint64_t *Cg, void *Yg, uint64_t *thresh, uint8_t *texact,
                         uint64_t *bumped_keys, void *bumped_vals, unsigned long long *bumped_count,
-                        uint32_t *err, cudaStream_t st, const BatchView *bv) {
+                        uint32_t *err, cudaStream_t st, const BatchView *bv, void *scratch) {
     if (bv ? bv->nparts == 0 : part_end(L) <= L.part_lo) return cudaSuccess;
     switch (vbytes) {
     case 1:
         return band_impl<uint8_t>(L, keys, (const uint8_t *)vals, bucket_start, Cg, (uint8_t *)Yg, thresh, texact,
-                                  bumped_keys, (uint8_t *)bumped_vals, bumped_count, err, st, bv);
+                                  bumped_keys, (uint8_t *)bumped_vals, bumped_count, err, st, bv, scratch);
     case 2:
         return band_impl<uint16_t>(L, keys, (const uint16_t *)vals, bucket_start, Cg, (uint16_t *)Yg, thresh, texact,
-                                   bumped_keys, (uint16_t *)bumped_vals, bumped_count, err, st, bv);
+                                   bumped_keys, (uint16_t *)bumped_vals, bumped_count, err, st, bv, scratch);
     default:
         return band_impl<uint32_t>(L, keys, (const uint32_t *)vals, bucket_start, Cg, (uint32_t *)Yg, thresh, texact,
-                                   bumped_keys, (uint32_t *)bumped_vals, bumped_count, err, st, bv);
+                                   bumped_keys, (uint32_t *)bumped_vals, bumped_count, err, st, bv, scratch);
     }
 }
 

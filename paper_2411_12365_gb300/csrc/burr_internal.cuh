@@ -145,6 +145,9 @@ struct BatchView {
     uint32_t nstruct = 0, nparts = 0, ngroups = 0, ntiles = 0;
     uint64_t nbuckets = 0;                  // global buckets
     uint64_t nkeys = 0;                     // keys of the layer (sum over structures)
+    uint32_t max_len = 0;                   // buckets of the longest partition
+    uint32_t mode = 0;                      // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
+    bool fallback = false;                  // a base case
 };
 
 // Scratch bytes of launch_sort for n keys in a layer of m slots.
@@ -177,10 +180,16 @@ cudaError_t launch_sort_slack_end(const LayerDesc &L, uint32_t vbytes, uint64_t 
 // Band + bump (or base case), writing the band of every partition to Cg/Yg.
 // With a batch view (bv != nullptr) L is ignored: every partition of every
 // structure of the view is processed, bumped_count is per structure.
+// scratch: band_scratch_bytes(L, bv) bytes of device memory where that is not
+// 0 (launches of few partitions, banded in segments); without it every
+// partition is banded from end to end by one CTA.
+size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv = nullptr);
+// Kernels that launch enqueues with its scratch.
+uint32_t band_kernel_count(const LayerDesc &L, const BatchView *bv = nullptr);
 cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *keys, const void *vals,
                         const uint32_t *bucket_start, uint64_t *Cg, void *Yg, uint64_t *thresh, uint8_t *texact,
                         uint64_t *bumped_keys, void *bumped_vals, unsigned long long *bumped_count,
-                        uint32_t *err, cudaStream_t st, const BatchView *bv = nullptr);
+                        uint32_t *err, cudaStream_t st, const BatchView *bv = nullptr, void *scratch = nullptr);
 
 // Back-substitution of every partition: Z from the band.
 // max_ctas_per_sm > 0 caps the grid at that many CTAs per SM (the warps then

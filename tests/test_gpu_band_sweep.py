@@ -1,5 +1,5 @@
 """The band sweep where it can go wrong: more rows than registers (loads far
-above one), more rows in a bucket than are staged at once, buckets of one
+above one), partitions banded in segments, more rows in a bucket than are staged at once, buckets of one
 block's worth of slots, values that travel inside the row keys (up to 16 bits)
 and beside them (17 and more), in both threshold modes.  Whole exports against
 the serial oracle, bit for bit."""
@@ -26,6 +26,12 @@ CASES = [
     (15_013, 8, 1.015, B64), (15_013, 24, 2.5, B64),
     (127, 8, 1.015, {}), (130, 16, 1.015, {}), (64, 32, 1.0, {}),
     (40_000, 8, 1.015, dict(partition_slots=128, min_partition_slots=0)),   # a cut at every bucket
+    # few long partitions, banded in segments: just too short, one bucket past two segments, odd
+    # lengths, both value layouts, searched cuts, loads where segments seldom or never meet again
+    (8_030, 8, 1.015, {}), (8_290, 8, 1.015, {}), (300_011, 24, 1.015, {}), (270_007, 16, 1.015, {}),
+    (400_003, 5, 1.015, dict(partition_slots=16384, cut_search=burr.CUT_DIFF)),
+    (150_000, 8, 0.97, {}), (150_000, 9, 1.1, {}), (200_000, 32, 1.6, {}), (120_000, 8, 0.9, dict(layers=0)),
+    (260_003, 7, 1.02, dict(partition_slots=40_960, lower_partition_slots=8192)), (90_001, 8, 1.015, B64),
 ]
 
 
