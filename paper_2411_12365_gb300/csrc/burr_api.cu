@@ -534,7 +534,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
         cudaError_t e = side.order(st, side.side, kOrderSlot);
         if (e != cudaSuccess) return e;
         tev[pending.l][3] = tm.mark_on(side.side);
-        e = launch_backsub(pending.L, vb, (const uint64_t *)cgs[pending.set], ygs[pending.set], pending.z, side.side,
+        e = launch_backsub(pending.L, vb, (uint64_t *)cgs[pending.set], ygs[pending.set], pending.z, side.side,
                            nullptr, kBacksubCtasPerSm);
         if (e != cudaSuccess) return e;
         tev[pending.l][4] = tm.mark_on(side.side);
@@ -652,7 +652,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
                                S.thresh, tex, (uint64_t *)bk[which], bv[which], bcount, err, side.band2), "band");
                 CK(side.order(st, side.side, kOrderSlot), "order");
                 tev[l][5] = tm.mark_on(side.side);
-                CK(launch_backsub(La, vb, (const uint64_t *)cgs[set], ygs[set], S.z, side.side, nullptr,
+                CK(launch_backsub(La, vb, (uint64_t *)cgs[set], ygs[set], S.z, side.side, nullptr,
                                   kBacksubCtasPerSm),
                    "backsub");
                 tev[l][6] = tm.mark_on(side.side);
@@ -667,7 +667,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             tev[l][2] = tm.mark();
             if (onep) CK(launch_thresh_flags(tex, dseg, blkseg, (uint32_t)nd, S.flags, tcounts, S.dir, st), "flags");
             pending = PendingBacksub{true, l, set, Lpend, S.z};
-            h->launches += (slack ? 6 : sort_kernel_count(L)) + 2 + (onep ? 2 : 0);
+            h->launches += (slack ? 6 : sort_kernel_count(L)) + 1 + backsub_kernel_count(Lpend) + (onep ? 2 : 0);
             CK(cudaMemcpyAsync(hc, ctr, 16, cudaMemcpyDeviceToHost, st), "read counters");
             if (onep) CK(cudaMemcpyAsync(&nflag, S.dir + nd, 4, cudaMemcpyDeviceToHost, st), "read threshold count");
             CK(cudaStreamSynchronize(st), "layer");
@@ -748,8 +748,8 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             if (he & ~kErrUnsolvable) return fail(BURR_ERR_INTERNAL, "base case: device error 0x%x", he);
             if (he & kErrUnsolvable) continue;
             const int t2 = tm.mark();
-            CK(launch_backsub(L, vb, (const uint64_t *)cgs[set], ygs[set], F.z, st), "backsub");
-            h->launches += 1;
+            CK(launch_backsub(L, vb, (uint64_t *)cgs[set], ygs[set], F.z, st), "backsub");
+            h->launches += backsub_kernel_count(L);
             const int t3 = tm.mark();
             solved = true;
             h->fb_attempt = a;
@@ -997,7 +997,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         cudaError_t e = side.order(st, side.side, kOrderSlot);
         if (e != cudaSuccess) return e;
         bsm[pending.l][2] = tm.mark_on(side.side);
-        e = launch_backsub(LayerDesc(), vb, (const uint64_t *)cgs[pending.set], ygs[pending.set], pending.z, side.side,
+        e = launch_backsub(LayerDesc(), vb, (uint64_t *)cgs[pending.set], ygs[pending.set], pending.z, side.side,
                            &pending.v);
         if (e != cudaSuccess) return e;
         bsm[pending.l][3] = tm.mark_on(side.side);
@@ -1026,6 +1026,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         v.ntiles = (uint32_t)T.tile_struct.size();
         v.nbuckets = T.nbuckets;
         v.nkeys = T.nkeys;
+        v.slots = T.slots;
         v.max_len = T.max_len;
         v.mode = p.threshold_mode;
         v.fallback = T.fallback;
@@ -1127,6 +1128,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         if (K1 > 0 && K1 < v.nparts && v.part_order) {
             BatchView va = v;
             va.nparts = K1;
+            va.slots = vrest.slots = 0;   // parts of the layer's slots
             vrest.part_order = v.part_order + K1;
             vrest.nparts = v.nparts - K1;
             CK(side.order(st, side.band2, kSplitSlot), "order");
@@ -1136,7 +1138,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
                            (uint64_t *)bk[w], bv2[w], bcount, err, side.band2, &vrest), "band");
             CK(side.order(st, side.side, kOrderSlot), "order");
             bsm[l][0] = tm.mark_on(side.side);
-            CK(launch_backsub(none, vb, (const uint64_t *)cg, yg, z, side.side, &va), "backsub");
+            CK(launch_backsub(none, vb, (uint64_t *)cg, yg, z, side.side, &va), "backsub");
             bsm[l][1] = tm.mark_on(side.side);
             CK(side.order(side.band2, st, kSplitEndSlot), "order");
             for (auto *h : hs) h->launches += 2;
@@ -1159,7 +1161,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         pending.set = set;
         pending.v = vrest;
         pending.z = z;
-        for (auto *h : hs) h->launches += 6;
+        for (auto *h : hs) h->launches += 5 + backsub_kernel_count(none, &vrest);
         std::vector<unsigned long long> cnt(who.size());
         std::vector<uint32_t> hdir(onep ? blkseg.size() + 1 : 0);
         uint32_t e = 0;
@@ -1229,8 +1231,8 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         CK(launch_sort_batch(v, vb, cur_k, cur_v, (uint64_t *)sk, sv, (uint32_t *)bst, scratch, st), "sort");
         CK(launch_band(none, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cg, yg, nullptr, nullptr,
                        (uint64_t *)bk[wfb], bv2[wfb], bcount, err, st, &v, seg), "band");
-        CK(launch_backsub(none, vb, (const uint64_t *)cg, yg, z, st, &v), "backsub");
-        for (auto *h : hs) h->launches += 6;
+        CK(launch_backsub(none, vb, (uint64_t *)cg, yg, z, st, &v), "backsub");
+        for (auto *h : hs) h->launches += 5 + backsub_kernel_count(none, &v);
         std::vector<uint32_t> f(left.size());
         uint32_t e = 0;
         CK(cudaMemcpyAsync(f.data(), ffail, f.size() * 4, cudaMemcpyDeviceToHost, st), "read flags");
@@ -1954,7 +1956,7 @@ int burr_shard_build_layer(const uint64_t *keys, const void *values, uint64_t n,
     CK(launch_band(L, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cg, yg, thresh, nullptr,
                    bumped_keys, bumped_values, bcount, err, st),
        "band");
-    CK(launch_backsub(L, vb, (const uint64_t *)cg, yg, z, st), "backsub");
+    CK(launch_backsub(L, vb, (uint64_t *)cg, yg, z, st), "backsub");
     unsigned long long hc[2] = {0, 0};
     CK(cudaMemcpyAsync(hc, ctr, 16, cudaMemcpyDeviceToHost, st), "read counters");
     CK(cudaStreamSynchronize(st), "shard layer");
@@ -2012,7 +2014,7 @@ int burr_shard_build_base(const uint64_t *keys, const void *values, uint64_t n, 
         if (he & ~kErrUnsolvable) return fail(BURR_ERR_INTERNAL, "base case: device error 0x%x", he);
         if (he & kErrUnsolvable) continue;
         CK(cudaMemsetAsync(z, 0, z_words * 8, st), "clear table");
-        CK(launch_backsub(L, vb, (const uint64_t *)cg, yg, z, st), "backsub");
+        CK(launch_backsub(L, vb, (uint64_t *)cg, yg, z, st), "backsub");
         CK(cudaStreamSynchronize(st), "base case");
         *m_out = m;
         *seed_index_out = p.layers + a;

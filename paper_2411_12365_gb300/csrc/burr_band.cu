@@ -1,6 +1,5 @@
 // burr_band.cu -- insertion with bumping ("Insertion" of Fig. 7; Sec. 2
-// "Bumping" and Sec. 3 "Bumping at thread boundaries") and back-substitution
-// ("Back Substitution" of Fig. 7).
+// "Bumping" and Sec. 3 "Bumping at thread boundaries").
 //
 // One warp per partition.  The paper gives one partition to one CPU thread,
 // which eliminates the rows one by one against a stored band.  Here the warp
@@ -864,180 +863,6 @@ __global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t npa
     }
 }
 
-// Back-substitution, right to left over the partition's owned slots, one
-// window per value bit: Z[i] = Y[i] ^ parity((C[i] >> 1) & Z[i+1 .. i+63]),
-// Z[i] = 0 on empty slots (C = Y = 0 there).  The 64-bit register T holds Z of
-// the 64 slots right of the current group (bit j = slot i+1+j); after a block
-// of 64 slots it is exactly that block's table word for this bit plane.
-//
-// Four slots are solved per step so that the dependent chain is short: with
-// c'_s = C[s] >> 1, the four parities against T are independent,
-//   A_d = Y[i-d] ^ parity((c'_{i-d} >> d) & T),  d = 0..3,
-// and the slots of the group then correct each other through the low bits of
-// their own rows:
-//   z_i = A_0,  z_{i-1} = A_1 ^ c'_{i-1}[0] z_i,
-//   z_{i-2} = A_2 ^ c'_{i-2}[0] z_{i-1} ^ c'_{i-2}[1] z_i,
-//   z_{i-3} = A_3 ^ c'_{i-3}[0] z_{i-2} ^ c'_{i-3}[1] z_{i-1} ^ c'_{i-3}[2] z_i,
-//   T <- (T << 4) | z_i z_{i-1} z_{i-2} z_{i-3}.
-constexpr int kBsWarps = 4;
-
-__device__ __forceinline__ uint32_t parity64(uint64_t x) {
-    return (uint32_t)__popc((uint32_t)x ^ (uint32_t)(x >> 32)) & 1u;
-}
-
-// Back-substitution with several partitions per warp: a partition needs only
-// R lanes (R = r for one-byte values, one bit plane per lane; r / 2 or r / 4
-// rounded up with 2 or 4 planes per lane for wider values), so a warp solves
-// G = min(32 / R, kBsGroups) partitions side by side, lanes [q*R, q*R + R) on
-// partition q.  For a batch, whose structures may differ in r, R comes from
-// the widest value type (8 lanes); lanes past a structure's r sit out.  Each group runs the four-slot steps above; sharing each instruction
-// among G partitions cuts the issue load G-fold, which matters because the
-// solve runs beside the next layer's sort and band.  Partitions of one warp may
-// differ in length: each walks its own blocks from the right, and a finished
-// group idles until the longest one is done.
-constexpr int kBsGroups = 8;
-
-//
-// kG (1, 2, 4 or 8) bounds G at compile time, so that the per-group registers
-// of a launch with few groups (G = 4 at r = 8) are not those of eight.  A warp
-// job is one set of G partitions; the grid may hold fewer warps than jobs
-// (a cap on the CTAs per SM leaves room beside it for the next layer's
-// kernels), and then every warp walks the jobs with the grid's stride.
-//
-// kPL bit planes per lane (1, 2 or 4; for r up to 8, 16, 32): lane k of a
-// group solves planes k*kPL .. k*kPL + kPL - 1, each with its own window T, and
-// the rows' reads, shifts and low bits serve all of them.  At r = 16 a group
-// then needs 8 lanes instead of 16, so a warp takes 4 partitions instead of 2.
-template <typename V, int kG, int kPL>
-__global__ void __launch_bounds__(32 * kBsWarps, kG >= 8 ? 4 : 1)
-k_backsub_multi(LayerDesc L0, const uint64_t *__restrict__ Cg, const V *__restrict__ Yg, uint64_t *__restrict__ Z0,
-                BatchView bv, uint32_t R, uint32_t G, uint64_t njobs) {
-    __shared__ __align__(16) uint64_t sc[kBsWarps][kG][64];
-    __shared__ __align__(16) uint32_t sy[kBsWarps][kG][64];
-    __shared__ uint64_t sbase[kBsWarps][kG];  // first slot of the group's structure in the layer arrays
-    __shared__ uint64_t shi[kBsWarps][kG];    // one past the last block of the group's partition
-    __shared__ uint32_t slen[kBsWarps][kG];   // its number of blocks
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t q = (uint32_t)lane / R, k = (uint32_t)lane % R;
-    for (uint64_t job = (uint64_t)blockIdx.x * kBsWarps + warp; job < njobs;
-         job += (uint64_t)gridDim.x * kBsWarps) {
-    uint64_t gp = job * G + q + (bv.sd ? 0 : L0.part_lo);
-    const uint64_t nparts = bv.sd ? bv.nparts : part_end(L0);
-    uint64_t bhi = 0, base = 0;
-    uint32_t len = 0, r = 0;
-    uint64_t *Z = Z0;
-    if (q < G && gp < nparts) {
-        LayerDesc L;
-        uint64_t part;
-        if (bv.sd) {
-            if (bv.part_order) gp = bv.part_order[gp];   // partitions of similar length share a warp
-            const StructDesc &D = bv.sd[bv.part_struct[gp]];
-            L = D.L;
-            part = gp - D.part_base;
-            base = D.slot_base;
-            Z += D.z_base;
-        } else {
-            L = L0;
-            part = gp;
-        }
-        const uint64_t lo = part_own_lo(L, part) >> 6, hi = part_own_hi(L, part) >> 6;
-        if (hi > lo) {
-            bhi = hi;
-            len = (uint32_t)(hi - lo);
-        }
-        r = L.r;
-    }
-    if (q < G && k == 0) {
-        sbase[warp][q] = base;
-        shi[warp][q] = bhi;
-        slen[warp][q] = len;
-    }
-    const uint32_t maxlen = __reduce_max_sync(0xffffffffu, len);
-    __syncwarp();
-    if (maxlen == 0) continue;
-    uint64_t gh[kG], gb[kG];
-    uint32_t gl[kG];
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        gh[g] = (uint32_t)g < G ? shi[warp][g] : 0;
-        gb[g] = (uint32_t)g < G ? sbase[warp][g] : 0;
-        gl[g] = (uint32_t)g < G ? slen[warp][g] : 0;
-    }
-    // software pipeline: registers hold every group's next block while this one is solved
-    uint64_t nc0[kG], nc1[kG];
-    uint32_t ny0[kG], ny1[kG];
-#pragma unroll
-    for (int g = 0; g < kG; ++g) {
-        nc0[g] = nc1[g] = 0;
-        ny0[g] = ny1[g] = 0;
-        if (gl[g] > 0) {
-            const uint64_t s0 = gb[g] + ((gh[g] - 1) << 6);
-            nc0[g] = Cg[s0 + lane];
-            nc1[g] = Cg[s0 + lane + 32];
-            ny0[g] = Yg[s0 + lane];
-            ny1[g] = Yg[s0 + lane + 32];
-        }
-    }
-    const bool solve = k * kPL < r;
-    uint64_t T[kPL];
-#pragma unroll
-    for (int pl = 0; pl < kPL; ++pl) T[pl] = 0;
-    for (uint32_t t = 0; t < maxlen; ++t) {
-        __syncwarp();
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-            if (t < gl[g]) {
-                sc[warp][g][lane] = nc0[g] >> 1;
-                sc[warp][g][lane + 32] = nc1[g] >> 1;
-                sy[warp][g][lane] = ny0[g];
-                sy[warp][g][lane + 32] = ny1[g];
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int g = 0; g < kG; ++g) {
-            if (t + 1 < gl[g]) {
-                const uint64_t s0 = gb[g] + ((gh[g] - 2 - t) << 6);
-                nc0[g] = Cg[s0 + lane];
-                nc1[g] = Cg[s0 + lane + 32];
-                ny0[g] = Yg[s0 + lane];
-                ny1[g] = Yg[s0 + lane + 32];
-            }
-        }
-        if (solve && t < len) {
-            const uint64_t *c = sc[warp][q];
-            const uint32_t *yv = sy[warp][q];
-#pragma unroll 4
-            for (int g = 15; g >= 0; --g) {
-                // slots 4g .. 4g+3 in three 16-byte shared reads
-                const ulonglong2 clo = *reinterpret_cast<const ulonglong2 *>(c + 4 * g);
-                const ulonglong2 chi = *reinterpret_cast<const ulonglong2 *>(c + 4 * g + 2);
-                const uint4 yq = *reinterpret_cast<const uint4 *>(yv + 4 * g);
-                const uint64_t c0 = chi.y, c1 = chi.x >> 1, c2 = clo.y >> 2, c3 = clo.x >> 3;
-                const uint32_t l1 = (uint32_t)chi.x, l2 = (uint32_t)clo.y, l3 = (uint32_t)clo.x;
-#pragma unroll
-                for (int pl = 0; pl < kPL; ++pl) {
-                    const uint32_t b = k * kPL + (uint32_t)pl;   // this plane's value bit
-                    const uint32_t a0 = ((yq.w >> b) & 1u) ^ parity64(c0 & T[pl]);
-                    const uint32_t a1 = ((yq.z >> b) & 1u) ^ parity64(c1 & T[pl]);
-                    const uint32_t a2 = ((yq.y >> b) & 1u) ^ parity64(c2 & T[pl]);
-                    const uint32_t a3 = ((yq.x >> b) & 1u) ^ parity64(c3 & T[pl]);
-                    const uint32_t z0 = a0;
-                    const uint32_t z1 = a1 ^ (l1 & z0);
-                    const uint32_t z2 = a2 ^ ((l2 >> 1) & z0) ^ (l2 & z1);
-                    const uint32_t z3 = a3 ^ ((l3 >> 2) & z0) ^ ((l3 >> 1) & z1) ^ (l3 & z2);
-                    T[pl] = (T[pl] << 4) | (uint64_t)(((z0 << 3) | (z1 << 2) | (z2 << 1) | z3) & 15u);
-                }
-            }
-#pragma unroll
-            for (int pl = 0; pl < kPL; ++pl)
-                if (k * kPL + (uint32_t)pl < r) Z[(bhi - 1 - t) * r + k * kPL + pl] = T[pl];
-        }
-    }
-    __syncwarp();   // the warp's shared arrays are reused by its next job
-    }
-}
-
 // Segments of a launch: buckets per segment (0: whole partitions) and segments
 // of the longest partition.  A launch of few partitions is bound by their
 // chains (8.2 us per bucket, 512 buckets in a default partition) while most of
@@ -1165,58 +990,6 @@ cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *key
     default:
         return band_impl<uint32_t>(L, keys, (const uint32_t *)vals, bucket_start, Cg, (uint32_t *)Yg, thresh, texact,
                                    bumped_keys, (uint32_t *)bumped_vals, bumped_count, err, st, bv, scratch);
-    }
-}
-
-template <typename V, int kG, int kPL>
-cudaError_t backsub_launch(const LayerDesc &L, const uint64_t *Cg, const V *Yg, uint64_t *Z, cudaStream_t st,
-                           const BatchView &v, uint32_t R, uint32_t G, uint64_t njobs, unsigned grid) {
-    const cudaError_t e = prefer_shared(k_backsub_multi<V, kG, kPL>);
-    if (e != cudaSuccess) return e;
-    k_backsub_multi<V, kG, kPL><<<grid, 32 * kBsWarps, 0, st>>>(L, Cg, Yg, Z, v, R, G, njobs);
-    return cudaGetLastError();
-}
-
-// Planes per lane: one for values of a byte (r <= 8 lanes already fit four
-// groups in a warp), else as many as the value's bytes.
-template <typename V>
-constexpr int planes_per_lane() {
-    return sizeof(V) == 1 ? 1 : (int)sizeof(V);
-}
-
-template <typename V>
-cudaError_t backsub_impl(const LayerDesc &L, const uint64_t *Cg, const V *Yg, uint64_t *Z, cudaStream_t st,
-                         const BatchView &v, uint32_t R, uint32_t G, uint64_t njobs, unsigned grid) {
-    constexpr int PL = planes_per_lane<V>();
-    if (G <= 1) return backsub_launch<V, 1, PL>(L, Cg, Yg, Z, st, v, R, G, njobs, grid);
-    if (G <= 2) return backsub_launch<V, 2, PL>(L, Cg, Yg, Z, st, v, R, G, njobs, grid);
-    if (G <= 4) return backsub_launch<V, 4, PL>(L, Cg, Yg, Z, st, v, R, G, njobs, grid);
-    return backsub_launch<V, kBsGroups, PL>(L, Cg, Yg, Z, st, v, R, G, njobs, grid);
-}
-
-cudaError_t launch_backsub(const LayerDesc &L, uint32_t vbytes, const uint64_t *Cg, const void *Yg,
-                           uint64_t *Z, cudaStream_t st, const BatchView *bv, uint32_t max_ctas_per_sm) {
-    const uint64_t parts = bv ? bv->nparts : (part_end(L) > L.part_lo ? part_end(L) - L.part_lo : 0);
-    if (parts == 0) return cudaSuccess;
-    // several partitions per warp; a batch's structures may differ in r (up to 8 bits per value
-    // byte); R lanes per partition, each solving one bit plane for one-byte values, else as many
-    // planes as the value has bytes
-    const uint32_t pl = vbytes == 1 ? 1u : vbytes;
-    const uint32_t R = bv ? 8u * vbytes / pl : (L.r + pl - 1) / pl;
-    const uint32_t G = std::min<uint32_t>(32u / R, (uint32_t)kBsGroups);
-    const uint64_t njobs = (parts + G - 1) / G;
-    uint64_t grid = (njobs + kBsWarps - 1) / kBsWarps;
-    if (max_ctas_per_sm) {
-        int dev = 0, sms = 152;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        grid = std::min<uint64_t>(grid, (uint64_t)sms * max_ctas_per_sm);
-    }
-    const BatchView v = bv ? *bv : BatchView();
-    switch (vbytes) {
-    case 1: return backsub_impl<uint8_t>(L, Cg, (const uint8_t *)Yg, Z, st, v, R, G, njobs, (unsigned)grid);
-    case 2: return backsub_impl<uint16_t>(L, Cg, (const uint16_t *)Yg, Z, st, v, R, G, njobs, (unsigned)grid);
-    default: return backsub_impl<uint32_t>(L, Cg, (const uint32_t *)Yg, Z, st, v, R, G, njobs, (unsigned)grid);
     }
 }
 

@@ -145,6 +145,7 @@ struct BatchView {
     uint32_t nstruct = 0, nparts = 0, ngroups = 0, ntiles = 0;
     uint64_t nbuckets = 0;                  // global buckets
     uint64_t nkeys = 0;                     // keys of the layer (sum over structures)
+    uint64_t slots = 0;                     // slots of the layer (sum over structures; 0: only some of its partitions)
     uint32_t max_len = 0;                   // buckets of the longest partition
     uint32_t mode = 0;                      // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
     bool fallback = false;                  // a base case
@@ -195,9 +196,11 @@ cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *key
 // max_ctas_per_sm > 0 caps the grid at that many CTAs per SM (the warps then
 // walk the partitions with the grid's stride), which leaves room beside the
 // back-substitution for the kernels of the next layer.
-cudaError_t launch_backsub(const LayerDesc &L, uint32_t vbytes, const uint64_t *Cg, const void *Yg,
-                           uint64_t *Z, cudaStream_t st, const BatchView *bv = nullptr,
-                           uint32_t max_ctas_per_sm = 0);
+// The band is scratch to it: its rows may be overwritten.
+cudaError_t launch_backsub(const LayerDesc &L, uint32_t vbytes, uint64_t *Cg, void *Yg, uint64_t *Z, cudaStream_t st,
+                           const BatchView *bv = nullptr, uint32_t max_ctas_per_sm = 0);
+// Kernels that launch enqueues.
+uint32_t backsub_kernel_count(const LayerDesc &L, const BatchView *bv = nullptr);
 
 // Batched sort: every structure's keys of the layer grouped by global bucket
 // (as records h of each structure's layer).
