@@ -236,6 +236,9 @@ struct LayerStore {
     uint64_t *z = nullptr;        // (m/64)*r words
 };
 
+// Bytes allocated for a table of so many words: a query reads it in 32-byte loads
+// and may read up to the end of its last one.
+uint64_t table_alloc_bytes(uint64_t words) { return (words * 8 + 31) & ~31ull; }
 uint64_t flag_words(uint64_t nb) { return (nb + 63) / 64; }
 uint64_t dir_blocks(uint64_t nb) { return (nb + 511) / 512; }
 
@@ -568,7 +571,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             CK(dev_alloc((void **)&S.thresh, std::max<uint64_t>(tw, 1) * 8, st), "alloc thresholds");
             CK(cudaMemsetAsync(S.thresh, 0, tw * 8, st), "clear thresholds");
         }
-        CK(dev_alloc((void **)&S.z, std::max<uint64_t>((S.m / 64) * r, 1) * 8, st), "alloc table");
+        CK(dev_alloc((void **)&S.z, table_alloc_bytes(std::max<uint64_t>((S.m / 64) * r, 1)), st), "alloc table");
         if (!bk[which]) {
             CK(ar.alloc(&bk[which], cur_n * 8), "alloc bumped keys");
             CK(ar.alloc(&bv[which], cur_n * vb), "alloc bumped values");
@@ -732,7 +735,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
                 CK(ar.alloc(&ss, ss_bytes), "alloc sort scratch");
             }
             CK(side.reuse(set), "order");
-            CK(dev_alloc((void **)&F.z, (F.m / 64) * r * 8, st), "alloc table");
+            CK(dev_alloc((void **)&F.z, table_alloc_bytes((F.m / 64) * r), st), "alloc table");
             CK(cudaMemsetAsync(ctr, 0, 64, st), "clear counters");
             const LayerDesc L = make_desc(p, r, cur_n, F.m, F.sigma, 1, true, F.m);
             CK(band_scratch(L), "alloc band scratch");
@@ -1629,7 +1632,7 @@ struct Reader {
 };
 
 int upload_table(void **d, const void *src, uint64_t bytes, cudaStream_t st) {
-    CK(dev_alloc(d, std::max<uint64_t>(bytes, 8), st), "alloc imported table");
+    CK(dev_alloc(d, table_alloc_bytes(std::max<uint64_t>((bytes + 7) / 8, 1)), st), "alloc imported table");
     if (bytes) CK(cudaMemcpyAsync(*d, src, bytes, cudaMemcpyHostToDevice, st), "copy imported table");
     return BURR_OK;
 }

@@ -3,6 +3,8 @@
 // was bumped and is looked up in the next layer; the threshold is a 2-bit
 // level code or, with 1+-bit thresholds, 0 unless the bucket's flag is set)
 // and the standalone hash stage.
+#include <type_traits>
+
 #include "burr_internal.cuh"
 
 namespace burr {
@@ -44,66 +46,110 @@ __device__ __forceinline__ uint32_t eval_window(const uint64_t *__restrict__ z, 
     return v;
 }
 
-// The 2r table words around slot s (blocks s/64 and s/64 + 1), loaded before
-// the threshold is known so that both reads are in flight together; R is the
-// value width fixed at compile time.  The second block is needed only when the
-// window is not block-aligned, and a window that starts at the last block
-// (s = m - 64) has no second block inside the table: it is not read then.
-template <int R>
-struct Window {
-    uint64_t w0[R], w1[R];
-};
-
-// 32-byte read-only global load (four table words).
+// 32-byte read-only global load (four table words).  kKeep: the line stays in
+// L1.  A random window of a large table is not met again there, and allocated it
+// drives the thresholds out (192 KB of 2-bit codes per 10^8 keys), which are:
+// without, 10^8 keys of r = 8 took 1.81 -> 1.64 ms, 5*10^6 of r = 16 (10^7 stored)
+// 230 -> 184 us; a table that mostly fits L1 is faster kept (10^6 stored keys, r =
+// 3, 10^7 queried: 110 against 120 us).
+template <bool kKeep>
 __device__ __forceinline__ void ldg_v4(const uint64_t *p, uint64_t &a, uint64_t &b, uint64_t &c, uint64_t &d) {
-    asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+    if (kKeep) asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+    else asm("ld.global.nc.L1::no_allocate.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
 }
 
-// kWide: the table starts on 32 bytes and R is a multiple of 4, so each block
-// of R words is read in R/4 32-byte loads (checked by the launcher).  Narrow
-// reads of random windows cost one L1 wavefront per word and warp lane.
-template <int R, bool kWide>
+// The 2R table words around slot s (blocks s/64 and s/64 + 1), loaded before
+// the threshold is known so that both reads are in flight together; R is the
+// value width fixed at compile time.  The words are contiguous, so they are read
+// in aligned 32-byte loads whatever R is (every table starts on 32 bytes and is
+// allocated to a multiple of 32, see the launcher) and moved down by the place
+// of the first word: narrow reads cost one L1 request per word and lane, and
+// those bound the kernel (10^8 keys, r = 4: 1.76 ms with 8-byte loads).  The
+// second block is needed only when the window is not block-aligned, and a window
+// that starts at the last block (s = m - 64) has no second block inside the
+// table: nothing past the needed words' last load is read.
+template <int R>
+struct Window {
+    static constexpr int kMaxShift = R % 4 == 0 ? 0 : (R % 2 == 0 ? 2 : 3);
+    static constexpr int kLoads = (2 * R + kMaxShift + 3) / 4;
+    uint64_t w[4 * kLoads];
+};
+
+template <int R, bool kKeep>
 __device__ __forceinline__ void load_window(const uint64_t *__restrict__ z, uint32_t s, Window<R> &w) {
-    const uint64_t *p = z + (uint64_t)(s >> 6) * R;
-    const bool two = (s & 63u) != 0u;
-    if constexpr (kWide) {
-        static_assert(R % 4 == 0, "wide window loads need R % 4 == 0");
+    if (R == 1) {   // two words: narrow reads of the same sector are cheaper than the move
+        const bool two = (s & 63u) != 0u;
+        w.w[0] = __ldg(z + (s >> 6));
+        w.w[1] = two ? __ldg(z + (s >> 6) + 1) : 0ull;
+        return;
+    }
+    const uint64_t at = (uint64_t)(s >> 6) * R;
+    const uint32_t shift = (uint32_t)at & 3u & (uint32_t)Window<R>::kMaxShift;
+    const uint32_t need = shift + ((s & 63u) ? 2u * R : (uint32_t)R);
+    const uint64_t *p = z + (at & ~3ull);
 #pragma unroll
-        for (int k = 0; k < R; k += 4) ldg_v4(p + k, w.w0[k], w.w0[k + 1], w.w0[k + 2], w.w0[k + 3]);
+    for (int k = 0; k < Window<R>::kLoads; ++k) {
+        if (4 * k < R || 4u * k < need) ldg_v4<kKeep>(p + 4 * k, w.w[4 * k], w.w[4 * k + 1], w.w[4 * k + 2], w.w[4 * k + 3]);
+        else w.w[4 * k] = w.w[4 * k + 1] = w.w[4 * k + 2] = w.w[4 * k + 3] = 0;
+    }
+    if (Window<R>::kMaxShift & 1) {
 #pragma unroll
-        for (int k = 0; k < R; ++k) w.w1[k] = 0;
-        if (two) {
+        for (int k = 0; k + 1 < 4 * Window<R>::kLoads; ++k) w.w[k] = (shift & 1u) ? w.w[k + 1] : w.w[k];
+    }
+    if (Window<R>::kMaxShift & 2) {
 #pragma unroll
-            for (int k = 0; k < R; k += 4) ldg_v4(p + R + k, w.w1[k], w.w1[k + 1], w.w1[k + 2], w.w1[k + 3]);
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            w.w0[k] = __ldg(p + k);
-            w.w1[k] = two ? __ldg(p + R + k) : 0ull;
-        }
+        for (int k = 0; k + 2 < 4 * Window<R>::kLoads; ++k) w.w[k] = (shift & 2u) ? w.w[k + 2] : w.w[k];
     }
 }
 
 template <int R>
 __device__ __forceinline__ uint32_t eval_loaded(const Window<R> &w, uint32_t s, uint64_t c) {
     uint64_t cA, cB;
-    row_masks(c, s & 63u, cA, cB);   // w1 is zero when the window is block-aligned
+    row_masks(c, s & 63u, cA, cB);   // cB is zero when the window is block-aligned
     uint32_t v = 0;
 #pragma unroll
-    for (int k = 0; k < R; ++k) v |= parity64q((w.w0[k] & cA) ^ (w.w1[k] & cB)) << k;
+    for (int k = 0; k < R; ++k) v |= parity64q((w.w[k] & cA) ^ (w.w[R + k] & cB)) << k;
+    return v;
+}
+
+// Values of more than 16 bits, a multiple of 4: the window of eight (four)
+// planes at a time.
+template <int R, bool kKeep>
+__device__ __forceinline__ uint32_t eval_planes(const uint64_t *__restrict__ z, uint32_t s, uint64_t c) {
+    const uint64_t *p = z + (uint64_t)(s >> 6) * R;
+    uint64_t cA, cB;
+    row_masks(c, s & 63u, cA, cB);
+    const bool two = (s & 63u) != 0u;
+    uint32_t v = 0;
+#pragma unroll
+    for (int k = 0; k < R; k += 4) {
+        uint64_t a[4], b[4] = {0, 0, 0, 0};
+        ldg_v4<kKeep>(p + k, a[0], a[1], a[2], a[3]);
+        if (two) ldg_v4<kKeep>(p + R + k, b[0], b[1], b[2], b[3]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v |= parity64q((a[j] & cA) ^ (b[j] & cB)) << (k + j);
+    }
     return v;
 }
 
 // Threshold t of bucket b of bumping layer l: keys with offset < t are bumped.
+// The mode is fixed at compile time: the other mode's registers cost occupancy.
+template <bool kExact>
 __device__ __forceinline__ uint32_t threshold_of(const QueryDesc &Q, uint32_t l, uint32_t b) {
-    if (Q.mode == BURR_THRESH_1PLUS) {
+    if (kExact) {
         // flag bit; a flagged bucket's threshold sits at its rank
         const uint64_t *fl = Q.flags[l];
         const uint64_t w = __ldg(fl + (b >> 6));
         if (!((w >> (b & 63u)) & 1ull)) return 0;
         uint32_t rank = __ldg(Q.dir[l] + (b >> 9));
-        for (uint32_t k = (b >> 9) << 3; k < (b >> 6); ++k) rank += (uint32_t)__popcll(__ldg(fl + k));
+        const uint32_t before = (b >> 6) & 7u;   // the block's flag words before this one
+        fl += (b >> 9) << 3;
+        // all loads first (a loop to `before` waited for each word)
+        uint64_t x[7];
+#pragma unroll
+        for (uint32_t k = 0; k < 7; ++k) x[k] = k < before ? __ldg(fl + k) : 0ull;
+#pragma unroll
+        for (uint32_t k = 0; k < 7; ++k) rank += (uint32_t)__popcll(x[k]);
         rank += (uint32_t)__popcll(w & ((1ull << (b & 63u)) - 1ull));
         return __ldg(Q.tbytes[l] + rank);
     }
@@ -111,13 +157,12 @@ __device__ __forceinline__ uint32_t threshold_of(const QueryDesc &Q, uint32_t l,
 }
 
 // Query kernel for a value width R known at compile time: the table window
-// of a layer is loaded together with its threshold, and the thread's next key
-// is read while this key's table reads are in flight.  Measured (ms per query
-// of n keys, half members): 10^9 keys r = 8 72.5 either way, 10^8 keys r = 16
-// 4.45 -> 4.20, r = 1 0.79 either way.  Two keys per thread (their layer-0
-// reads in flight together, 98 registers) gave 70.7 at 10^9 but 4.69 and 0.89
-// at 10^8 (r = 16, r = 1).
-template <typename V, int R, bool kWide>
+// of a layer is loaded together with its threshold (values of up to 16 bits),
+// and the thread's next key is read while this key's table reads are in flight.
+// Two keys per thread (their layer-0 reads in flight together, 98 registers)
+// gave 70.7 ms against 72.5 at 10^9 keys (r = 8) but 4.69 against 4.20 and 0.89
+// against 0.79 at 10^8 (r = 16, r = 1).
+template <typename V, int R, bool kKeep, bool kExact>
 __global__ void __launch_bounds__(kQThreads)
 k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -128,26 +173,97 @@ k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, u
         const uint64_t key = key_next;
         if (i + stride < n) key_next = keys[i + stride];
         uint32_t v = 0;
-        uint32_t l = 0;
-        for (; l < Q.layers; ++l) {
+        for (uint32_t l = 0; l <= Q.layers; ++l) {               // [layers] = base case
             const uint64_t m = Q.m[l];
             if (m == 0) break;
             const uint64_t h = mix64(key ^ Q.sigma[l]);
             const uint32_t s = (uint32_t)__umul64hi(h, m - kW + 1);
-            Window<R> w;
-            load_window<R, kWide>(Q.z[l], s, w);
-            if ((s & (Q.B - 1)) < threshold_of(Q, l, s >> log2B)) continue;   // bumped: next layer
-            v = eval_loaded<R>(w, s, mix64(h + Q.sigma[l]) | 1ull);
+            if constexpr (R <= 16) {
+                Window<R> w;
+                load_window<R, kKeep>(Q.z[l], s, w);
+                if (l < Q.layers && (s & (Q.B - 1)) < threshold_of<kExact>(Q, l, s >> log2B)) continue;   // bumped: next layer
+                v = eval_loaded<R>(w, s, mix64(h + Q.sigma[l]) | 1ull);
+            } else {
+                if (l < Q.layers && (s & (Q.B - 1)) < threshold_of<kExact>(Q, l, s >> log2B)) continue;
+                v = eval_planes<R, kKeep>(Q.z[l], s, mix64(h + Q.sigma[l]) | 1ull);
+            }
             break;
         }
-        if (l == Q.layers && Q.m[l] != 0) {                    // base case
-            const uint64_t h = mix64(key ^ Q.sigma[l]);
-            const uint32_t s = (uint32_t)__umul64hi(h, Q.m[l] - kW + 1);
-            Window<R> w;
-            load_window<R, kWide>(Q.z[l], s, w);
-            v = eval_loaded<R>(w, s, mix64(h + Q.sigma[l]) | 1ull);
-        }
         out[i] = (V)v;
+    }
+}
+
+// Widths of 8, 16 and 32 bits: a block of R words is R / 4 32-byte sectors, which
+// G = R / 4 neighbouring lanes read together, for the keys of the group in turn;
+// each lane evaluates four planes of all G keys, and the group exchanges the
+// results.  A load is then one request per key and block instead of one per
+// sector: the requests of an SM to L2 bound the kernel (84% of their peak, 22%
+// of the returning sectors', 10^8 keys of r = 8).  The bumped keys (2 in 100)
+// go on lane by lane in the deeper layers.  Measured against one lane per key:
+// r = 8, 10^8 keys of a 100 MB table 1.71 -> 1.58 ms, 2*10^7 of a 1 MB table 445 ->
+// 290 us (1+-bit); r = 16, 5*10^6 of 20 MB 182 -> 118 us, 1+-bit 261 -> 130; r = 32,
+// 2*10^7 of 40 MB 1070 -> 717 us.
+template <typename V, int R, bool kExact>
+__global__ void __launch_bounds__(kQThreads)
+k_query_group(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
+    constexpr int G = R / 4, kAtOnce = G < 4 ? G : 4;   // keys of the group whose reads are in flight together
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint32_t log2B = 31 - __clz(Q.B);
+    const int lane = threadIdx.x & 31, q = lane & (G - 1), first = lane & ~(G - 1);
+    const uint64_t m0 = Q.m[0], sigma0 = Q.sigma[0];
+    const uint64_t *__restrict__ z0 = Q.z[0] + 4 * q;
+    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint64_t key_next = i < n ? keys[i] : 0ull;
+    // a whole warp at a time: lanes past the end take part with key 0
+    for (; i - (uint64_t)lane < n; i += stride) {
+        const uint64_t key = key_next;
+        if (i + stride < n) key_next = keys[i + stride];
+        const uint64_t h = mix64(key ^ sigma0);
+        const uint32_t s = (uint32_t)__umul64hi(h, m0 - kW + 1);
+        const bool bumped = (s & (Q.B - 1)) < threshold_of<kExact>(Q, 0, s >> log2B);
+        const uint64_t c = mix64(h + sigma0) | 1ull;
+        uint32_t part = 0;   // planes 4q .. 4q + 3 of the group's keys, key t at bits 4t
+#pragma unroll
+        for (int t0 = 0; t0 < G; t0 += kAtOnce) {
+            uint64_t a[kAtOnce][4], b[kAtOnce][4];
+            uint32_t st[kAtOnce];
+#pragma unroll
+            for (int t = 0; t < kAtOnce; ++t) {
+                st[t] = __shfl_sync(0xffffffffu, s, first + t0 + t);
+                const uint64_t *p = z0 + (uint64_t)(st[t] >> 6) * R;
+                ldg_v4<false>(p, a[t][0], a[t][1], a[t][2], a[t][3]);
+                b[t][0] = b[t][1] = b[t][2] = b[t][3] = 0;
+                if (st[t] & 63u) ldg_v4<false>(p + R, b[t][0], b[t][1], b[t][2], b[t][3]);
+            }
+#pragma unroll
+            for (int t = 0; t < kAtOnce; ++t) {
+                const uint64_t ct = (uint64_t)__shfl_sync(0xffffffffu, (uint32_t)(c >> 32), first + t0 + t) << 32 |
+                                    __shfl_sync(0xffffffffu, (uint32_t)c, first + t0 + t);
+                uint64_t cA, cB;
+                row_masks(ct, st[t] & 63u, cA, cB);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) part |= parity64q((a[t][k] & cA) ^ (b[t][k] & cB)) << (4 * (t0 + t) + k);
+            }
+        }
+        uint32_t v = ((part >> (4 * q)) & 15u) << (4 * q);
+#pragma unroll
+        for (int d = 1; d < G; ++d) {
+            const uint32_t x = __shfl_xor_sync(0xffffffffu, part, d);
+            v |= ((x >> (4 * q)) & 15u) << (4 * (q ^ d));
+        }
+        if (bumped) {
+            v = 0;
+            for (uint32_t l = 1; l <= Q.layers; ++l) {           // [layers] = base case
+                const uint64_t m = Q.m[l];
+                if (m == 0) break;
+                const uint64_t hl = mix64(key ^ Q.sigma[l]);
+                const uint32_t sl = (uint32_t)__umul64hi(hl, m - kW + 1);
+                if (l < Q.layers && (sl & (Q.B - 1)) < threshold_of<kExact>(Q, l, sl >> log2B)) continue;
+                v = eval_planes<R, false>(Q.z[l], sl, mix64(hl + Q.sigma[l]) | 1ull);
+                break;
+            }
+        }
+        if (i < n) out[i] = (V)v;
     }
 }
 
@@ -167,7 +283,7 @@ k_query(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uin
             const uint32_t s = (uint32_t)__umul64hi(h, m - kW + 1);
             const uint32_t b = s >> log2B;
             const uint32_t off = s & (Q.B - 1);
-            const uint32_t t = threshold_of(Q, l, b);
+            const uint32_t t = Q.mode == BURR_THRESH_1PLUS ? threshold_of<true>(Q, l, b) : threshold_of<false>(Q, l, b);
             if (off < t) continue;                             // bumped: next layer
             v = eval_window(Q.z[l], Q.r, s, mix64(h + Q.sigma[l]) | 1ull);
             break;
@@ -195,29 +311,52 @@ __global__ void k_hash(const uint64_t *__restrict__ keys, uint64_t n, uint64_t s
 
 }  // namespace
 
+namespace {
+
+// The kernel of width Q.r, if there is one; false otherwise (wider values of
+// which the planes don't come in fours).
+template <int R>
+void query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
+    using V = std::conditional_t<(R <= 8), uint8_t, std::conditional_t<(R <= 16), uint16_t, uint32_t>>;
+    // a table of at most 1 MB (layer 0 holds nearly all of it) mostly stays in L1 or is met again there
+    const bool keep = (Q.m[0] / 64) * R * 8 <= (1ull << 20), exact = Q.mode == BURR_THRESH_1PLUS;
+    if constexpr (R == 8 || R == 16 || R == 32) {
+        if (Q.layers > 0 && Q.m[0] != 0) {   // (without bumping layers there is no layer 0 with thresholds)
+            if (exact) k_query_group<V, R, true><<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n);
+            else k_query_group<V, R, false><<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n);
+            return;
+        }
+    }
+    auto go = [&](auto *kernel) { kernel<<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n); };
+    if (exact) keep ? go(k_query_r<V, R, true, true>) : go(k_query_r<V, R, false, true>);
+    else keep ? go(k_query_r<V, R, true, false>) : go(k_query_r<V, R, false, false>);
+}
+
+bool launch_query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
+    switch (Q.r) {
+#define BURR_QUERY_R(R) \
+    case R: query_r<R>(Q, keys, out, n, grid, st); return true;
+        BURR_QUERY_R(1) BURR_QUERY_R(2) BURR_QUERY_R(3) BURR_QUERY_R(4) BURR_QUERY_R(5) BURR_QUERY_R(6)
+        BURR_QUERY_R(7) BURR_QUERY_R(8) BURR_QUERY_R(9) BURR_QUERY_R(10) BURR_QUERY_R(11) BURR_QUERY_R(12)
+        BURR_QUERY_R(13) BURR_QUERY_R(14) BURR_QUERY_R(15) BURR_QUERY_R(16) BURR_QUERY_R(20) BURR_QUERY_R(24)
+        BURR_QUERY_R(28) BURR_QUERY_R(32)
+#undef BURR_QUERY_R
+    default: return false;
+    }
+}
+
+}  // namespace
+
 cudaError_t launch_query(const QueryDesc &Q, uint32_t vbytes, const uint64_t *keys, void *out, uint64_t n,
                          cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     const unsigned grid = grid_for(n, kQThreads, 152u * 64u);
-    // common widths: the window is loaded together with the threshold, in 32-byte reads when
-    // every table of the structure starts on 32 bytes
+    // 32-byte reads when every table of the structure starts on 32 bytes (a caller's allocator may
+    // give others); the library allocates every table to a multiple of 32 bytes
     bool wide = true;
     for (uint32_t l = 0; l <= Q.layers; ++l)
         if (Q.m[l] != 0 && ((uintptr_t)Q.z[l] & 31u) != 0) wide = false;
-    if (Q.r == 8 && vbytes == 1) {
-        if (wide) k_query_r<uint8_t, 8, true><<<grid, kQThreads, 0, st>>>(Q, keys, (uint8_t *)out, n);
-        else k_query_r<uint8_t, 8, false><<<grid, kQThreads, 0, st>>>(Q, keys, (uint8_t *)out, n);
-        return cudaGetLastError();
-    }
-    if (Q.r == 1 && vbytes == 1) {
-        k_query_r<uint8_t, 1, false><<<grid, kQThreads, 0, st>>>(Q, keys, (uint8_t *)out, n);
-        return cudaGetLastError();
-    }
-    if (Q.r == 16 && vbytes == 2) {
-        if (wide) k_query_r<uint16_t, 16, true><<<grid, kQThreads, 0, st>>>(Q, keys, (uint16_t *)out, n);
-        else k_query_r<uint16_t, 16, false><<<grid, kQThreads, 0, st>>>(Q, keys, (uint16_t *)out, n);
-        return cudaGetLastError();
-    }
+    if (wide && launch_query_r(Q, keys, out, n, grid, st)) return cudaGetLastError();
     switch (vbytes) {
     case 1: k_query<uint8_t><<<grid, kQThreads, 0, st>>>(Q, keys, (uint8_t *)out, n); break;
     case 2: k_query<uint16_t><<<grid, kQThreads, 0, st>>>(Q, keys, (uint16_t *)out, n); break;
