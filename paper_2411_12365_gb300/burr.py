@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes as C
 import operator
 import os
+import sys
 import threading
 import weakref
 from collections.abc import Sequence
@@ -93,6 +94,8 @@ def lib_path() -> str:
 def load(path: str | None = None):
     """Load libburr.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -191,19 +194,21 @@ def default_params(**kw) -> Params:
     return p
 
 
+def _current_stream(torch, x):
+    """Handle of torch's current CUDA stream on the tensor's device."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # without making a Stream object
+    return raw(x.get_device()) if raw is not None else torch.cuda.current_stream(x.device).cuda_stream
+
+
 def _ptr_and_stream(x, stream):
     """(pointer, stream handle, keepalive) for a torch tensor or numpy array."""
-    try:
-        import torch
-        if isinstance(x, torch.Tensor):
-            if not x.is_contiguous():
-                x = x.contiguous()
-            if x.is_cuda:
-                s = stream if stream is not None else torch.cuda.current_stream(x.device).cuda_stream
-                return x.data_ptr(), s, x
-            return x.data_ptr(), stream, x
-    except ImportError:
-        pass
+    torch = sys.modules.get("torch")   # a tensor's module is loaded
+    if torch is not None and isinstance(x, torch.Tensor):
+        if not x.is_contiguous():
+            x = x.contiguous()
+        if stream is None and x.is_cuda:
+            stream = _current_stream(torch, x)
+        return x.data_ptr(), stream, x
     a = np.ascontiguousarray(x)
     return a.ctypes.data, stream, a
 

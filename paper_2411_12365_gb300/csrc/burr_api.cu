@@ -387,46 +387,112 @@ constexpr int kSplitEndSlot = kBandSets + 4;
 constexpr int kCopySlot = kBandSets + 5;
 // Keys per chunk of host input copied ahead of the sort's first pass.
 constexpr uint64_t kStreamChunk = 1ull << 24;
+// Build scratch of up to so many bytes comes in one allocation.
+constexpr size_t kOneBlock = 64ull << 20;
+constexpr int kNumEvents = kBandSets + 6;
+// Streams, events and a page-locked page that a build uses beside the caller's
+// stream.  Making them took about a third of a 1,000-key build, so they are kept
+// for the next build on the device: at most kKeptSets of them per process (a set
+// given back beyond that is destroyed), and those when the library is unloaded.
+// A set belongs to one build or query at a time.  Work still queued on its
+// streams when it is given back only comes before the next user's.
+struct StreamSet {
+    int dev = 0;
+    cudaStream_t side = nullptr, band2 = nullptr, copy = nullptr;
+    cudaEvent_t ev[kNumEvents] = {};
+    void *page = nullptr;                  // kPageBytes, for results read by the host
+    cudaError_t make() {
+        cudaError_t e = cudaGetDevice(&dev);
+        for (cudaStream_t *s : {&side, &band2, &copy})
+            if (e == cudaSuccess) e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking);
+        for (int i = 0; i < kNumEvents && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+        return e == cudaSuccess ? cudaMallocHost(&page, kPageBytes) : e;
+    }
+    ~StreamSet() {
+        for (cudaStream_t s : {side, band2, copy})
+            if (s) cudaStreamDestroy(s);
+        for (cudaEvent_t e : ev)
+            if (e) cudaEventDestroy(e);
+        if (page) cudaFreeHost(page);
+    }
+    static constexpr size_t kPageBytes = 4096;
+};
+constexpr size_t kKeptSets = 8;
+std::mutex g_sets_mu;
+struct KeptSets : std::vector<std::unique_ptr<StreamSet>> {   // not in use
+    ~KeptSets() {
+        int dev;
+        if (cudaGetDevice(&dev) == cudaSuccess) return;       // (the members are destroyed)
+        for (auto &q : *this) q.release();                    // the runtime is gone, and they with it
+    }
+} g_sets;
+
+std::unique_ptr<StreamSet> take_streams(cudaError_t &e) {
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_sets_mu);
+        for (auto &q : g_sets)
+            if (q->dev == dev) {
+                std::unique_ptr<StreamSet> s = std::move(q);
+                q = std::move(g_sets.back());
+                g_sets.pop_back();
+                return s;
+            }
+    }
+    auto s = std::make_unique<StreamSet>();
+    e = s->make();
+    return e == cudaSuccess ? std::move(s) : nullptr;
+}
+
+void give_streams(std::unique_ptr<StreamSet> s) {
+    std::lock_guard<std::mutex> lk(g_sets_mu);
+    if (g_sets.size() < kKeptSets) g_sets.push_back(std::move(s));
+}
+
 struct SideStream {
     cudaStream_t main, side = nullptr, band2 = nullptr, copy = nullptr;
-    cudaEvent_t ev[kBandSets + 6] = {};
+    std::unique_ptr<StreamSet> set;
+    bool copied = false;   // the copy stream was used
+    bool idle = false;     // the host has waited for everything queued
     explicit SideStream(cudaStream_t m) : main(m) {}
     cudaError_t init() {
-        cudaError_t e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
-        if (e == cudaSuccess && kBandSplitPct) e = cudaStreamCreateWithFlags(&band2, cudaStreamNonBlocking);
-        for (int i = 0; i < kBandSets + 6 && e == cudaSuccess; ++i)
-            e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
-        return e;
+        cudaError_t e = cudaSuccess;
+        set = take_streams(e);
+        if (!set) return e;
+        side = set->side;
+        if (kBandSplitPct) band2 = set->band2;
+        return cudaSuccess;
     }
-    cudaError_t copy_init() { return copy ? cudaSuccess : cudaStreamCreateWithFlags(&copy, cudaStreamNonBlocking); }
+    void *page() const { return set->page; }
+    void copy_init() {
+        copy = set->copy;
+        copied = true;
+    }
     // `to` waits for everything enqueued so far on `from`
     cudaError_t order(cudaStream_t from, cudaStream_t to, int slot) {
-        cudaError_t e = cudaEventRecord(ev[slot], from);
-        return e == cudaSuccess ? cudaStreamWaitEvent(to, ev[slot], 0) : e;
+        cudaError_t e = cudaEventRecord(set->ev[slot], from);
+        return e == cudaSuccess ? cudaStreamWaitEvent(to, set->ev[slot], 0) : e;
     }
-    // mark the end of the back-substitution that read band set `set`
-    cudaError_t solved(int set) { return cudaEventRecord(ev[set], side); }
-    // the main stream waits until band set `set` is no longer read (no-op if never used)
-    cudaError_t reuse(int set) { return cudaStreamWaitEvent(main, ev[set], 0); }
+    // mark the end of the back-substitution that read band set `i`
+    cudaError_t solved(int i) {
+        used |= 1u << i;
+        return cudaEventRecord(set->ev[i], side);
+    }
+    // the main stream waits until band set `i` is no longer read (no-op if never used)
+    cudaError_t reuse(int i) { return used >> i & 1u ? cudaStreamWaitEvent(main, set->ev[i], 0) : cudaSuccess; }
     ~SideStream() {
-        if (copy) {
-            if (ev[kFinalSlot] && cudaEventRecord(ev[kFinalSlot], copy) == cudaSuccess)
-                cudaStreamWaitEvent(main, ev[kFinalSlot], 0);
-            cudaStreamDestroy(copy);
+        if (!set) return;
+        if (!idle) {   // an early return: later frees on the main stream come after the other streams' work
+            for (cudaStream_t s : {copied ? copy : nullptr, band2, side})
+                if (s && cudaEventRecord(set->ev[kFinalSlot], s) == cudaSuccess) cudaStreamWaitEvent(main, set->ev[kFinalSlot], 0);
+            cudaStreamSynchronize(main);   // and nothing lands in the page any more
         }
-        if (band2) {
-            if (ev[kFinalSlot] && cudaEventRecord(ev[kFinalSlot], band2) == cudaSuccess)
-                cudaStreamWaitEvent(main, ev[kFinalSlot], 0);
-            cudaStreamDestroy(band2);
-        }
-        if (side) {
-            if (ev[kFinalSlot] && cudaEventRecord(ev[kFinalSlot], side) == cudaSuccess)
-                cudaStreamWaitEvent(main, ev[kFinalSlot], 0);
-            cudaStreamDestroy(side);
-        }
-        for (auto e : ev)
-            if (e) cudaEventDestroy(e);
+        give_streams(std::move(set));
     }
+
+private:
+    uint32_t used = 0;     // band sets solved in this build (an event may hold an earlier build's record)
 };
 
 int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r, const burr_params &p,
@@ -474,23 +540,36 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
     // scratch sized for layer 0 (later layers and a normal base case are smaller)
     uint64_t cap_m = std::max<uint64_t>(m0, 64), cap_nb = num_buckets(cap_m, p.bucket_slots);
     void *sk, *sv, *bst, *ss, *cg, *yg, *bk[2], *bv[2], *ctr;
-    CK(ar.alloc(&sk, n * 8), "alloc sorted keys");
-    CK(ar.alloc(&sv, n * vb), "alloc sorted values");
-    CK(ar.alloc(&bst, (cap_nb + 1) * 4), "alloc bucket offsets");
     // the exact sort's scratch, or the fixed-capacity sort's for layer 0 if larger
     size_t ss_bytes = std::max(sort_scratch_bytes(n, cap_m, vb), slack0);
-    CK(ar.alloc(&ss, ss_bytes), "alloc sort scratch");
+    struct {
+        void **p;
+        size_t bytes;
+        const char *what;
+    } const parts[] = {{&sk, n * 8, "alloc sorted keys"},     {&sv, n * vb, "alloc sorted values"},
+                       {&bst, (cap_nb + 1) * 4, "alloc bucket offsets"}, {&ss, ss_bytes, "alloc sort scratch"},
+                       {&cg, cap_m * 8, "alloc band"},        {&yg, cap_m * vb, "alloc band values"},
+                       {&bk[0], n * 8, "alloc bumped keys"},  {&bv[0], n * vb, "alloc bumped values"},
+                       {&ctr, 64, "alloc counters"}};
+    size_t all = 0;
+    for (const auto &q : parts) all += (q.bytes + 255) & ~(size_t)255;
+    if (all <= kOneBlock) {   // one block for all of them: nine allocations are a tenth of a 1,000-key build
+        void *d;
+        CK(ar.alloc(&d, all), "alloc scratch");
+        char *at = (char *)d;
+        for (const auto &q : parts) {
+            *q.p = at;
+            at += (q.bytes + 255) & ~(size_t)255;
+        }
+    } else {
+        for (const auto &q : parts) CK(ar.alloc(q.p, q.bytes), q.what);
+    }
     void *cgs[kBandSets] = {}, *ygs[kBandSets] = {};
     uint64_t cgcap[kBandSets] = {};
-    CK(ar.alloc(&cg, cap_m * 8), "alloc band");
-    CK(ar.alloc(&yg, cap_m * vb), "alloc band values");
     cgs[0] = cg;
     ygs[0] = yg;
     cgcap[0] = cap_m;
-    CK(ar.alloc(&bk[0], n * 8), "alloc bumped keys");
-    CK(ar.alloc(&bv[0], n * vb), "alloc bumped values");
     bk[1] = bv[1] = nullptr;
-    CK(ar.alloc(&ctr, 64), "alloc counters");
     unsigned long long *bcount = (unsigned long long *)ctr;
     uint32_t *err = (uint32_t *)((char *)ctr + 8);
     // 1+-bit thresholds: exact threshold per bucket, one segment covering
@@ -598,15 +677,16 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
         const size_t slack_bytes = kSortSlack ? sort_slack_scratch_bytes(L, vb) : 0;
         bool slack = slack_bytes != 0 && slack_bytes <= ss_bytes;
         bool streamed = false;   // layer 0: the host inputs have been copied in
-        unsigned long long hc[2] = {0, 0};
-        uint32_t nflag = 0;
+        // the layer's counters, read into page-locked memory (a pageable read costs a staging copy)
+        volatile unsigned long long *hc = (volatile unsigned long long *)side.page();
+        volatile uint32_t *hflag = (volatile uint32_t *)((char *)side.page() + 16);
         for (;;) {
             tev[l][0] = tm.mark();
             if (slack) {
                 CK(launch_sort_slack_begin(L, vb, ss, st), "sort");
                 if (l == 0 && stream_in && !streamed) {
                     // host inputs: copy chunk c, then pass 1 over it, while chunk c+1 is copied
-                    CK(side.copy_init(), "copy stream");
+                    side.copy_init();
                     CK(side.order(st, side.copy, kCopySlot), "order");   // after the allocations
                     for (uint64_t lo = 0; lo < n; lo += kStreamChunk) {
                         const uint64_t hi = std::min<uint64_t>(n, lo + kStreamChunk);
@@ -671,8 +751,8 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             if (onep) CK(launch_thresh_flags(tex, dseg, blkseg, (uint32_t)nd, S.flags, tcounts, S.dir, st), "flags");
             pending = PendingBacksub{true, l, set, Lpend, S.z};
             h->launches += (slack ? 6 : sort_kernel_count(L)) + 1 + backsub_kernel_count(Lpend) + (onep ? 2 : 0);
-            CK(cudaMemcpyAsync(hc, ctr, 16, cudaMemcpyDeviceToHost, st), "read counters");
-            if (onep) CK(cudaMemcpyAsync(&nflag, S.dir + nd, 4, cudaMemcpyDeviceToHost, st), "read threshold count");
+            CK(cudaMemcpyAsync((void *)hc, ctr, 16, cudaMemcpyDeviceToHost, st), "read counters");
+            if (onep) CK(cudaMemcpyAsync((void *)hflag, S.dir + nd, 4, cudaMemcpyDeviceToHost, st), "read threshold count");
             CK(cudaStreamSynchronize(st), "layer");
             if (!(hc[1] & kErrSortSlack)) break;
             // a bin overflowed: this layer's outputs are partial; sort and band it again exactly
@@ -689,6 +769,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
         if (onep) {
             // exact thresholds of the flagged buckets (before the next layer's
             // band reuses the per-bucket array)
+            const uint32_t nflag = *hflag;
             S.nflag = nflag;
             S.tfirst = 0;
             CK(dev_alloc((void **)&S.tbytes, std::max<uint64_t>(nflag, 1), st), "alloc thresholds");
@@ -745,9 +826,9 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             CK(launch_band(L, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cgs[set], ygs[set],
                            nullptr, nullptr, nullptr, nullptr, bcount, err, st, nullptr, seg), "band");
             h->launches += sort_kernel_count(L) + band_kernel_count(L);
-            uint32_t he = 0;
-            CK(cudaMemcpyAsync(&he, err, 4, cudaMemcpyDeviceToHost, st), "read error word");
+            CK(cudaMemcpyAsync(side.page(), err, 4, cudaMemcpyDeviceToHost, st), "read error word");
             CK(cudaStreamSynchronize(st), "base case");
+            const uint32_t he = *(volatile uint32_t *)side.page();
             if (he & ~kErrUnsolvable) return fail(BURR_ERR_INTERNAL, "base case: device error 0x%x", he);
             if (he & kErrUnsolvable) continue;
             const int t2 = tm.mark();
@@ -768,6 +849,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
     CK(side.order(side.side, st, kJoinSlot), "order");
     const int t_end = tm.mark();
     CK(cudaStreamSynchronize(st), "build");
+    side.idle = true;   // (the second band and copy streams were joined where they were used)
     for (uint32_t l = 0; l <= p.layers; ++l) {
         if (tev[l][0] < 0) continue;
         h->stage_ms[l][0] = tm.ms(tev[l][0], tev[l][1]);
@@ -1267,6 +1349,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
     CK(side.order(side.side, st, kJoinSlot), "order");
     const int t_end = tm.mark();
     CK(cudaStreamSynchronize(st), "build");
+    side.idle = true;
     const float total = tm.ms(t_begin, t_end);
     for (auto *h : hs) {
         h->total_ms = total;
@@ -1468,6 +1551,7 @@ int burr_query(const burr_handle *h, const uint64_t *keys, void *out, uint64_t n
     }
     CK(side.order(side.side, st, kJoinSlot), "order");
     CK(cudaStreamSynchronize(st), "query");
+    side.idle = true;
     return BURR_OK;
 }
 
@@ -1528,6 +1612,12 @@ int burr_export(const burr_handle *h, void *host_buf, uint64_t *len) {
         return fail(BURR_ERR_INVALID, "export buffer too small (%llu bytes needed)", (unsigned long long)need);
     }
     uint8_t *q = (uint8_t *)host_buf;
+    // the copies are queued on the default stream, which cudaMemcpy uses, and waited for once
+    auto copy = [](void *dst, const void *src, size_t bytes) {
+        const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, 0);
+        if (e != cudaSuccess) cudaStreamSynchronize(0);   // nothing is written after an early return
+        return e;
+    };
     q = put32(q, 0x52525542u);
     q = put32(q, onep ? 2 : 1);
     q = put32(q, r);
@@ -1559,23 +1649,24 @@ int burr_export(const burr_handle *h, void *host_buf, uint64_t *len) {
         const uint64_t tw = (S.nb + 31) / 32, zw = (S.m / 64) * r;
         if (onep) {
             const uint64_t fw = flag_words(S.nb), padded = 8 * ((S.nflag + 7) / 8);
-            if (fw) CK(cudaMemcpy(q, S.flags, fw * 8, cudaMemcpyDeviceToHost), "export threshold flags");
+            if (fw) CK(copy(q, S.flags, fw * 8), "export threshold flags");
             q += fw * 8;
             q = put64(q, S.nflag);
             memset(q, 0, padded);
             if (S.nflag)
-                CK(cudaMemcpy(q, S.tbytes + S.tfirst, S.nflag, cudaMemcpyDeviceToHost), "export thresholds");
+                CK(copy(q, S.tbytes + S.tfirst, S.nflag), "export thresholds");
             q += padded;
         } else {
-            if (tw) CK(cudaMemcpy(q, S.thresh, tw * 8, cudaMemcpyDeviceToHost), "export thresholds");
+            if (tw) CK(copy(q, S.thresh, tw * 8), "export thresholds");
             q += tw * 8;
         }
-        if (zw) CK(cudaMemcpy(q, S.z, zw * 8, cudaMemcpyDeviceToHost), "export table");
+        if (zw) CK(copy(q, S.z, zw * 8), "export table");
         q += zw * 8;
     }
     const uint64_t zw = (F.m / 64) * r;
-    if (zw) CK(cudaMemcpy(q, F.z, zw * 8, cudaMemcpyDeviceToHost), "export base case");
+    if (zw) CK(copy(q, F.z, zw * 8), "export base case");
     q += zw * 8;
+    CK(cudaStreamSynchronize(0), "export");
     *len = (uint64_t)(q - (uint8_t *)host_buf);
     return BURR_OK;
 }

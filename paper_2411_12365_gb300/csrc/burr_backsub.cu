@@ -392,7 +392,8 @@ cudaError_t launch_backsub(const LayerDesc &L, uint32_t vbytes, uint64_t *Cg, vo
     // byte); R lanes per partition, each solving one bit plane for one-byte values, else as many
     // planes as the value has bytes
     const BatchView v = bv ? *bv : BatchView();
-    if (bs_in_blocks(bv, parts)) {
+    // (16-byte copies of the band: a caller's allocator may give less aligned blocks)
+    if (bs_in_blocks(bv, parts) && (((uintptr_t)Cg | (uintptr_t)Yg) & 15u) == 0) {
         const uint64_t lo = bv || L.part_lo == 0 ? 0 : part_own_lo(L, L.part_lo);
         const uint64_t hi = bv ? bv->slots : (part_end(L) == L.K ? L.m : part_own_hi(L, part_end(L) - 1));
         const uint32_t rmax = bv ? 8u * vbytes : L.r;

@@ -936,7 +936,7 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
         k_band<V><<<(unsigned)p.parts, 64, 0, st>>>(a);
         return cudaGetLastError();
     }
-    char *q = (char *)scratch;
+    char *q = (char *)(((uintptr_t)scratch + 255) & ~(uintptr_t)255);   // (a caller's allocator gives the block)
     a.seg = p.seg;
     a.nseg = p.nseg;
     a.omask = (uint64_t *)q;
@@ -967,7 +967,7 @@ size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv) {
     if (bv ? bv->nparts == 0 : part_end(L) <= L.part_lo) return 0;
     const SegPlan p = seg_plan(L, bv);
     if (!p.seg) return 0;
-    return align256(p.buckets * 8) + align256(p.buckets) + 2 * align256(p.parts * p.nseg * 64 * sizeof(Pivot)) +
+    return 256 + align256(p.buckets * 8) + align256(p.buckets) + 2 * align256(p.parts * p.nseg * 64 * sizeof(Pivot)) +
            2 * align256(p.parts * p.nseg * 4);
 }
 

@@ -443,12 +443,13 @@ __device__ __forceinline__ uint64_t group_out(uint64_t x, uint64_t sigma) {
     return OUT_KEYS ? key_of_h(x, sigma) : x;
 }
 // SLACK: the input of group g starts at g * cap (the bins of a SLACK pass 2),
-// and goff holds the packed offsets of the groups' counts.
+// and goff holds the packed offsets of the groups' counts.  goff == nullptr: one
+// group of n_all keys.
 template <typename V, bool RAW, bool OUT_KEYS, bool SLACK = false>
 __global__ void __launch_bounds__(kGroupThreads)
 k_group_sort(const uint64_t *__restrict__ keys, const V *__restrict__ vals, const uint32_t *__restrict__ goff,
              uint64_t sigma, uint64_t range, uint32_t log2B, uint64_t nb, uint64_t *__restrict__ keys_out,
-             V *__restrict__ vals_out, uint32_t *__restrict__ bucket_start, uint64_t cap = 0) {
+             V *__restrict__ vals_out, uint32_t *__restrict__ bucket_start, uint64_t cap, uint32_t n_all) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *skey = reinterpret_cast<uint64_t *>(smem_raw);
     V *sval = reinterpret_cast<V *>(skey + kGroupCap);
@@ -456,7 +457,7 @@ k_group_sort(const uint64_t *__restrict__ keys, const V *__restrict__ vals, cons
     const uint64_t g = blockIdx.x;
     const uint64_t b_lo = g << kGroupShift;
     const uint32_t nbk = (uint32_t)min((uint64_t)kGroupBuckets, nb - b_lo);
-    const uint32_t lo = goff[g], hi = goff[g + 1], n = hi - lo;
+    const uint32_t lo = goff ? goff[g] : 0u, hi = goff ? goff[g + 1] : n_all, n = hi - lo;
     if (SLACK) {   // index i in [lo, hi) reads input g * cap + (i - lo)
         keys += g * cap - lo;
         vals += g * cap - lo;
@@ -556,7 +557,7 @@ cudaError_t launch_group_sort(const Plan &P, const LayerDesc &L, const uint64_t 
     if (e != cudaSuccess) return e;
     if ((e = prefer_shared(k_group_sort<V, RAW, OUT_KEYS, SLACK>)) != cudaSuccess) return e;
     k_group_sort<V, RAW, OUT_KEYS, SLACK><<<(unsigned)P.ngroups, kGroupThreads, group_smem, st>>>(
-        gk, gv, goff, L.sigma, L.range, P.log2B, L.nb, keys_out, vals_out, bucket_start, cap);
+        gk, gv, goff, L.sigma, L.range, P.log2B, L.nb, keys_out, vals_out, bucket_start, cap, (uint32_t)L.n);
     return cudaGetLastError();
 }
 
@@ -605,12 +606,9 @@ cudaError_t sort_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, u
         return e;
 
     if (P.passes == 0) {
-        // one group: offsets [0, n]; the group pass reads the keys themselves
-        const uint32_t h[2] = {0, (uint32_t)n};
-        e = cudaMemcpyAsync(S.o2, h, sizeof(h), cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return e;
-        return out_keys ? launch_group_sort<V, true, true>(P, L, keys, vals, S.o2, keys_out, vals_out, bucket_start, st)
-                        : launch_group_sort<V, true, false>(P, L, keys, vals, S.o2, keys_out, vals_out, bucket_start,
+        // one group, [0, n): the group pass reads the keys themselves
+        return out_keys ? launch_group_sort<V, true, true>(P, L, keys, vals, nullptr, keys_out, vals_out, bucket_start, st)
+                        : launch_group_sort<V, true, false>(P, L, keys, vals, nullptr, keys_out, vals_out, bucket_start,
                                                             st);
     }
     const uint32_t *goff;
