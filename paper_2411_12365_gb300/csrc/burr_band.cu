@@ -33,18 +33,19 @@
 //     threshold above it is taken at once.
 //
 // What bounds it: with every warp slot taken, the ALU pipe (integer logic,
-// selects and compares at half rate: 79% busy at 10^9 keys, 43 warp
-// instructions per key); with few partitions, the chain of a step (bit test,
-// warp maximum, shuffle, XOR: ~95 cycles per slot).  Layer-0 band, ms (r = 8
+// selects and compares at half rate) and the queue of shuffles, maxima and
+// shared-memory stores, at about 37 cycles of an SM quarter per slot; with few
+// partitions, the chain of a step (bit test, warp maximum, shuffle, XOR: about 75
+// cycles per slot) and of the bookkeeping between blocks of slots.  Layer-0 band, ms (r = 8
 // unless said), against the streaming insertion that it replaces (32 lanes
 // eliminating one row each against a band in shared memory, a 128-bit
 // compare-and-swap per step, every bucket as long as its longest chain, a
 // dependent bucket inserted again):
-//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 3.2
-//   10^6 keys (16 partitions)                     6.57 -> 4.4
-//   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 7.7
-//   10^8 keys (1504 partitions)                   8.33 -> 6.9;  1+-bit 16.3 -> 10.6
-//   10^9 keys (15034 partitions)                  63.7 -> 50.5
+//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 2.9 (in segments 0.75)
+//   10^6 keys (16 partitions)                     6.57 -> 3.9 (in segments 1.27)
+//   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 6.4
+//   10^8 keys (1504 partitions)                   8.33 -> 6.3;  1+-bit 16.3 -> 9.3
+//   10^9 keys (15034 partitions)                  63.7 -> 47.4
 #include <algorithm>
 
 #include "burr_internal.cuh"
@@ -62,16 +63,14 @@ constexpr unsigned kFull = 0xffffffffu;
 // 16 slots unrolled and the sweep inlined for both halves of a bucket, the
 // warps of an SM, each at its own place in the code, waited on instruction
 // fetches (layer-0 band of 10^9 keys 104.7 ms against 60.9 with 4 slots and
-// one copy); 1, 2, 4, 8 and 16 slots in one copy: 58.7, 55.2, 54.2, 54.5, 56.6.
-#ifndef BURR_BAND_UNROLL
-#define BURR_BAND_UNROLL 8
-#endif
-constexpr uint32_t kUnrollSlots = BURR_BAND_UNROLL;
-// CTAs (partitions) per SM that the kernel's registers allow: 64 registers a
-// thread.  Layer-0 band of 10^9 keys with 16, 14 and 12: 50.5, 53.3, 55.4 ms.
-#ifndef BURR_BAND_CTAS
-#define BURR_BAND_CTAS 16
-#endif
+// one copy).  Now 4 / 8 / 16 slots: 47.4 / 47.5 / 50.4 ms, 10^6 keys 1.27 / 1.31 / 1.65.
+constexpr uint32_t kUnrollSlots = 4;
+// CTAs (partitions) per SM that the registers allow: 16 (64 registers a thread,
+// 76 bytes of spills) where partitions outnumber what fits, else 14 (72, none).
+// Layer-0 band, ms, 16 / 14: 10^9 keys 47.4 / 50.1 (12: 55.4 before other
+// changes); 10^8 6.37 / 6.33, 1+-bit 9.41 / 9.33; 10^6 1.31 / 1.27.
+constexpr int kManyCtas = 16, kFewCtas = 14;
+constexpr uint64_t kFewParts = 152 * kFewCtas;
 
 // Key of a live row: bit 30 = row of an earlier bucket, bits 22..29 = offset + 1,
 // bit 21 = which of the lane's two rows, bits 0..4 = lane (so that a key is a
@@ -360,6 +359,16 @@ __device__ __forceinline__ void drop_slots(BandSmem &S, uint32_t from, uint32_t 
 }
 
 
+// If in is not 0: (w0, w1, y) ^= (p0, p1, py).  Predicated by hand: written as
+// conditionals each XOR became a select besides.
+__device__ __forceinline__ void xor_row(uint32_t in, uint32_t &w0, uint32_t &w1, uint32_t &y, uint32_t p0, uint32_t p1,
+                                        uint32_t py) {
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p xor.b32 %0, %0, %4;\n\t@p xor.b32 %1, %1, %5;\n\t"
+        "@p xor.b32 %2, %2, %6;\n\t}"
+        : "+r"(w0), "+r"(w1), "+r"(y)
+        : "r"(in), "r"(p0), "r"(p1), "r"(py));
+}
+
 // One slot: the live row of the highest key with bit `mask` is stored at `e`
 // (place c of the block) and XORed into every other such row.  Without such a
 // row every lane writes key 0 (an empty slot) and nothing changes.
@@ -368,8 +377,9 @@ __device__ __forceinline__ void drop_slots(BandSmem &S, uint32_t from, uint32_t 
 // instruction): LOP3, SEL, ISETP 2 each, max 1, warp maximum 2, shuffle 4,
 // ballot 4, popc and find-first-bit 8, a 16-byte exchange through shared memory
 // about 20.  So the pivot's lane comes out of the maximum itself (its low
-// bits) instead of a ballot and a find-first, and the pivot travels by three
-// shuffles.
+// bits) instead of a ballot and a find-first, and the pivot travels by two
+// shuffles (three with values of more than 16 bits); the whole step takes 36.5,
+// 38.7 with the pivot stored by its own lane.
 template <bool kPacked>
 __device__ __forceinline__ void sweep_slot(Row &A, Row &B, uint32_t mask, unsigned slot, uint32_t c) {
     const uint32_t xa = A.w0 & A.gate & mask, xb = B.w0 & B.gate & mask;
@@ -377,22 +387,15 @@ __device__ __forceinline__ void sweep_slot(Row &A, Row &B, uint32_t mask, unsign
     const bool second = kb > ka;
     const uint32_t s0 = second ? B.w0 : A.w0, s1 = second ? B.w1 : A.w1, sk = max(ka, kb),
                    sy = kPacked ? 0u : (second ? B.y : A.y);
-    const uint32_t ek = kPacked || sk == 0u ? sk : sk | c << kValueBit, ey = kPacked ? c : sy;
     const uint32_t K = __reduce_max_sync(kFull, sk);
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %5, %6;\n\t@p st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}" ::"r"(slot),
-                 "r"(s0), "r"(s1), "r"(ek), "r"(ey), "r"(sk), "r"(K));
     const uint32_t p0 = __shfl_sync(kFull, s0, (int)K), p1 = __shfl_sync(kFull, s1, (int)K);
     const uint32_t py = kPacked ? K & kValueMask : __shfl_sync(kFull, sy, (int)K);
+    // every lane has the pivot now and writes the same 16 bytes: cheaper than a store by its lane
+    const uint32_t ek = kPacked || K == 0u ? K : K | c << kValueBit;
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(slot), "r"(p0), "r"(p1), "r"(ek), "r"(kPacked ? c : py));
     uint32_t &ya = kPacked ? A.key : A.y, &yb = kPacked ? B.key : B.y;
-    // predicated by hand: written as conditionals each XOR became a select besides
-    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p xor.b32 %0, %0, %4;\n\t@p xor.b32 %1, %1, %5;\n\t"
-        "@p xor.b32 %2, %2, %6;\n\t}"
-        : "+r"(A.w0), "+r"(A.w1), "+r"(ya)
-        : "r"(xa), "r"(p0), "r"(p1), "r"(py));
-    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p xor.b32 %0, %0, %4;\n\t@p xor.b32 %1, %1, %5;\n\t"
-        "@p xor.b32 %2, %2, %6;\n\t}"
-        : "+r"(B.w0), "+r"(B.w1), "+r"(yb)
-        : "r"(xb), "r"(p0), "r"(p1), "r"(py));
+    xor_row(xa, A.w0, A.w1, ya, p0, p1, py);
+    xor_row(xb, B.w0, B.w1, yb, p0, p1, py);
 }
 
 // The two warps of a partition meet.
@@ -426,13 +429,22 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         if (lane == 0) atomicOr(S.x.fail ? S.x.fail : a.err, kErrUnsolvable);
         return false;
     };
-    uint32_t nfree = W.nfree();
+    const bool test_window = L.window != 0;
+    const uint32_t total = first[128];
+    uint32_t nfree = W.nfree(), i0, up;
+    // first staged index of slot W.o, and (per lane) of the slot after W.o + lane
+    auto look = [&](uint32_t o) {
+        i0 = max(first[o], W.it);
+        up = max(first[min(o + 1u + (uint32_t)lane, lim)], i0);
+    };
+    look(W.o);
     while (W.o < lim) {
         const uint32_t o = W.o;
+        // the rows that the lanes' free registers would take, read before the block's length is known
+        const uint32_t ra = i0 + (uint32_t)__popc(W.fa & lt), rb = i0 + (uint32_t)(__popc(W.fa) + __popc(W.fb & lt));
+        const StagedRow sa = rows[min(ra, (uint32_t)kStage - 1u)], sb = rows[min(rb, (uint32_t)kStage - 1u)];
         // the longest block of slots (up to 32) whose new rows fit the free registers
-        const uint32_t i0 = max(first[o], W.it);
-        const uint32_t upto = max(first[min(o + 1u + (uint32_t)lane, lim)], i0) - i0;   // rows that start in slots o .. o + lane
-        uint32_t w = (uint32_t)__popc(__ballot_sync(kFull, upto <= nfree && o + (uint32_t)lane < lim));
+        const uint32_t w = (uint32_t)__popc(__ballot_sync(kFull, up - i0 <= nfree && o + (uint32_t)lane < lim));
         if (w == 0) {
             // more than 64 rows in 64 slots: the lowest-offset row of the bucket goes
             if (L.fallback) return unsolvable();
@@ -446,11 +458,11 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
             drop_slots(S, bB, o, W.t, lane);
             W.find_free();
             nfree = W.nfree();
+            look(o);
             continue;
         }
-        if (w > kUnrollSlots) w &= ~(kUnrollSlots - 1u);   // whole rounds of the unrolled loop
-        const uint32_t cnt = __shfl_sync(kFull, upto, (int)w - 1);
-        if (L.window && o < 64 && o + L.B >= L.window && __any_sync(kFull, max(A.key, B.key) >= kOldKey)) {
+        const uint32_t cnt = __shfl_sync(kFull, up - i0, (int)w - 1);
+        if (test_window && o < 64 && o + L.B >= L.window && __any_sync(kFull, max(A.key, B.key) >= kOldKey)) {
             // testing only: a row would be stored past the window that the test asked for
             if (lane == 0) atomicOr(a.err, kErrRingOverflow);
             return false;
@@ -458,12 +470,14 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         if (cnt == 0 && nfree == 64) {   // no live row: empty slots
             if ((uint32_t)lane < w) S.ring[(bB + o + (uint32_t)lane) & kRingMask].key = 0;
             W.o += w;
+            look(W.o);
             continue;
         }
         A.gate = B.gate = kFull;
-        const uint32_t ra = (uint32_t)__popc(W.fa & lt), rb = (uint32_t)(__popc(W.fa) + __popc(W.fb & lt));
-        if (A.key == 0 && ra < cnt) load_row<kPacked>(A, rows[i0 + ra], o, (uint32_t)lane);
-        if (B.key == 0 && rb < cnt) load_row<kPacked>(B, rows[i0 + rb], o, 1u << kRowBit | (uint32_t)lane);
+        if (A.key == 0 && ra < total && sa.o < o + w) load_row<kPacked>(A, sa, o, (uint32_t)lane);
+        if (B.key == 0 && rb < total && sb.o < o + w) load_row<kPacked>(B, sb, o, 1u << kRowBit | (uint32_t)lane);
+        W.o += w;
+        look(W.o);   // for the next block, during this one's sweep
         const Pivot *e = &S.ring[(bB + o) & kRingMask];
         const unsigned slot = (unsigned)__cvta_generic_to_shared(e);
         uint32_t c = 0;
@@ -488,7 +502,6 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         const uint32_t np = (uint32_t)__popc(__ballot_sync(kFull, K != 0));
         const uint32_t expect = nfree - cnt + np;
         nfree = W.nfree();
-        W.o += w;
         if (nfree == expect) {
             if (za) A.key = 0;
             if (zb) B.key = 0;
@@ -529,6 +542,7 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         W.it = first[W.t];
         W.find_free();
         nfree = W.nfree();
+        look(W.o);
     }
     return true;
 }
@@ -763,8 +777,8 @@ __device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &
 }
 
 // One partition per CTA, from its first bucket to its last.
-template <typename V>
-__global__ void __launch_bounds__(64, BURR_BAND_CTAS)
+template <typename V, int kCtas>
+__global__ void __launch_bounds__(64, kCtas)
 k_band(BandArgs<V> a) {
     __shared__ BandSmem S;
     if (!load_ctx(S, a, blockIdx.x)) return;
@@ -795,7 +809,7 @@ k_band(BandArgs<V> a) {
 // rows, so the result does not depend on the segments.  k_band_finish then
 // emits the bumped rows.
 template <typename V>
-__global__ void __launch_bounds__(64, BURR_BAND_CTAS)
+__global__ void __launch_bounds__(64, kFewCtas)
 k_band_seg(BandArgs<V> a, uint32_t nparts, uint32_t pass, bool last) {
     __shared__ BandSmem S;
     const uint32_t gp = last ? blockIdx.x : blockIdx.x % nparts, i = last ? 0 : blockIdx.x / nparts;
@@ -865,20 +879,21 @@ __global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t npa
 
 // Segments of a launch: buckets per segment (0: whole partitions) and segments
 // of the longest partition.  A launch of few partitions is bound by their
-// chains (8.2 us per bucket, 512 buckets in a default partition) while most of
-// the chip idles.  Segments of 32 buckets are passed 2-6 times until the last
-// one has met its stored run; measured, layer-0 band in ms, whole partitions
-// against segments: 5*10^4 keys (1 partition) 3.2 / 0.80, 10^6 (16) 4.45 / 1.44,
-// 10^7 (151) 4.6 / 2.34, 3*10^7 (451, segments of 128) 4.7 / 3.5.  Segments of
-// 16 and 24 buckets at 10^6 keys: 1.49 / 1.49.  The passes bring about 23
-// buckets' work per segment, so a launch that fills the chip as it is keeps
-// whole partitions: the segment length grows until segments and partitions fit
-// the 2432 resident CTAs (16 per SM) together (a cap of 1216 / 3700: 2.79 / 2.85
-// at 10^7 keys; 10^8 keys, 1504 partitions, in segments of 128: 7.8 against 6.8).
-// Exact thresholds keep whole partitions: right-hand sides of different
-// bumped rows survive for 58 buckets on average there, and segments gave 5.0-5.6
-// against 5.6 ms at 10^6 keys and 8.1-8.6 against 7.7 at 10^7.
-constexpr uint64_t kSegCap = 2432, kSegMin = 32;
+// chains (about 7.4 us per bucket, 512 buckets in a default partition) while most
+// of the chip idles.  Segments of 32 buckets are passed 2-6 times until the last
+// one has met its stored run; measured, layer-0 band in ms, whole partitions /
+// segments: 5*10^4 keys (1 partition) 3.2 / 0.8, 10^6 (16) 3.9 / 1.27, 10^7 (151,
+// segments of 64) 4.2 / 2.1, 3*10^7 (451, segments of 128) 4.3 / 3.3.  The passes
+// bring about 23 buckets' work per segment, so a launch that fills the chip as it
+// is keeps whole partitions: the segment length grows until segments and
+// partitions fit the resident CTAs (16 per SM) together (a cap of half / 1.5
+// times that: 2.79 / 2.85 against 2.34 ms at 10^7 keys before other changes; 10^8
+// keys, 1504 partitions, in segments of 128: 7.8 against 6.8).  With exact
+// thresholds the right-hand sides of different bumped rows survive for 58
+// buckets on average, so segments pay with fewer of them: 5*10^4 keys 4.0 / 1.5,
+// 2*10^5 5.7 / 2.0, 10^6 6.2 / 4.0, 3*10^6 6.5 / 5.3, 6*10^6 (91 partitions, segments
+// of 128; of 256: 6.7) 6.3 / 5.4, but 10^7 6.4 / 7.1.
+constexpr uint64_t kSegCap = 2432, kSegMin = 32, kSegCapExact = 460, kSegMaxExact = 128;
 constexpr uint32_t kSegPasses = 7;
 struct SegPlan {
     uint32_t seg = 0, nseg = 0;
@@ -901,10 +916,11 @@ SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
     }
     const uint32_t mode = bv ? bv->mode : L.mode;
     const bool fallback = bv ? bv->fallback : L.fallback != 0;
-    if (mode == BURR_THRESH_1PLUS && !fallback) return p;
+    const bool exact = mode == BURR_THRESH_1PLUS && !fallback;
+    const uint64_t cap = exact ? kSegCapExact : kSegCap;
     uint64_t seg = kSegMin;
-    while (p.parts + total / seg > kSegCap && seg * 2 <= longest) seg *= 2;
-    if (p.parts + total / seg > kSegCap || seg * 2 > longest) return p;
+    while (p.parts + total / seg > cap && seg * 2 <= longest) seg *= 2;
+    if (p.parts + total / seg > cap || seg * 2 > longest || (exact && seg > kSegMaxExact)) return p;
     p.seg = (uint32_t)seg;
     p.nseg = (uint32_t)((longest + seg - 1) / seg);
     return p;
@@ -931,10 +947,15 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
     a.err = err;
     const SegPlan p = seg_plan(L, bv);
     if (!scratch || !p.seg) {
-        const cudaError_t e = prefer_shared(k_band<V>);
-        if (e != cudaSuccess) return e;
-        k_band<V><<<(unsigned)p.parts, 64, 0, st>>>(a);
-        return cudaGetLastError();
+        auto go = [&](auto *kernel) -> cudaError_t {
+            const cudaError_t e = prefer_shared(kernel);
+            if (e != cudaSuccess) return e;
+            kernel<<<(unsigned)p.parts, 64, 0, st>>>(a);
+            return cudaGetLastError();
+        };
+        // (a part of a split layer runs beside the rest, at its registers)
+        const bool whole = bv ? bv->slots != 0 : L.part_lo == 0 && L.part_hi == 0;
+        return whole && p.parts <= kFewParts ? go(k_band<V, kFewCtas>) : go(k_band<V, kManyCtas>);
     }
     char *q = (char *)(((uintptr_t)scratch + 255) & ~(uintptr_t)255);   // (a caller's allocator gives the block)
     a.seg = p.seg;
