@@ -348,13 +348,36 @@ cudaError_t backsub_blocks(const LayerDesc &L, uint64_t *Cg, V *Yg, uint64_t *Z,
     return cudaGetLastError();
 }
 
-// Whether a launch reduces its blocks first (see k_bs_reduce): layer-0
-// back-substitution with / without, in us: 5*10^4 keys (1 partition) 138 / 928,
-// 10^6 (16) 196 / 1103, 10^7 (151) 323 / 1105, 3*10^7 (451) 702 / 1194 (build
-// 5.27 / 5.63 ms); at 10^8 keys (1504) the reduction took 1.96 ms beside layer
-// 1 against 1.16 (build 11.0 / 10.25 ms).
-constexpr uint64_t kBlockParts = 608;   // four per SM
-bool bs_in_blocks(const BatchView *bv, uint64_t parts) { return parts <= kBlockParts && (!bv || bv->slots); }
+// Slots of a launch, and whether it reduces its blocks first (see k_bs_reduce).
+// Without the reduction a launch takes about 1.1 us per block of its longest
+// partition while the chip has room; with it 0.19 us and about 10 us per 10^6
+// slots.  Layer-0 back-substitution with / without, in us: 5*10^4 keys (1
+// partition) 138 / 928, 10^6 (16) 196 / 1103, 10^7 (151) 323 / 1105, 3*10^7 (451)
+// 702 / 1194 (build 5.27 / 5.63 ms); at 10^8 keys (1504) the reduction took 1.96 ms
+// beside layer 1 against 1.16 (build 11.0 / 10.25 ms).  The line lies between the
+// last two for default partitions (1,024 blocks), and in proportion for others.
+constexpr uint64_t kReduceSlotsPerBlock = 50000;
+struct BsPlan {
+    uint64_t parts, first, slots;
+    bool blocks;
+};
+BsPlan bs_plan(const LayerDesc &L, const BatchView *bv) {
+    BsPlan p{0, 0, 0, false};
+    uint64_t longest;   // in blocks
+    if (bv) {
+        p.parts = bv->nparts;
+        p.slots = bv->slots;                // 0: only some of the layer's partitions
+        longest = (uint64_t)bv->max_len * 2;
+    } else {
+        if (part_end(L) <= L.part_lo) return p;
+        p.parts = part_end(L) - L.part_lo;
+        p.first = L.part_lo == 0 ? 0 : part_own_lo(L, L.part_lo);
+        p.slots = (part_end(L) == L.K ? L.m : part_own_hi(L, part_end(L) - 1)) - p.first;
+        longest = (L.K <= 1 ? L.m : L.P) / 64;
+    }
+    p.blocks = p.slots != 0 && p.slots <= longest * kReduceSlotsPerBlock;
+    return p;
+}
 
 template <typename V, int kG, int kPL>
 cudaError_t backsub_launch(const LayerDesc &L, const uint64_t *Cg, const V *Yg, uint64_t *Z, cudaStream_t st,
@@ -386,21 +409,17 @@ cudaError_t backsub_impl(const LayerDesc &L, const uint64_t *Cg, const V *Yg, ui
 
 cudaError_t launch_backsub(const LayerDesc &L, uint32_t vbytes, uint64_t *Cg, void *Yg,
                            uint64_t *Z, cudaStream_t st, const BatchView *bv, uint32_t max_ctas_per_sm) {
-    const uint64_t parts = bv ? bv->nparts : (part_end(L) > L.part_lo ? part_end(L) - L.part_lo : 0);
+    const BsPlan p = bs_plan(L, bv);
+    const uint64_t parts = p.parts;
     if (parts == 0) return cudaSuccess;
-    // several partitions per warp; a batch's structures may differ in r (up to 8 bits per value
-    // byte); R lanes per partition, each solving one bit plane for one-byte values, else as many
-    // planes as the value has bytes
     const BatchView v = bv ? *bv : BatchView();
     // (16-byte copies of the band: a caller's allocator may give less aligned blocks)
-    if (bs_in_blocks(bv, parts) && (((uintptr_t)Cg | (uintptr_t)Yg) & 15u) == 0) {
-        const uint64_t lo = bv || L.part_lo == 0 ? 0 : part_own_lo(L, L.part_lo);
-        const uint64_t hi = bv ? bv->slots : (part_end(L) == L.K ? L.m : part_own_hi(L, part_end(L) - 1));
+    if (p.blocks && (((uintptr_t)Cg | (uintptr_t)Yg) & 15u) == 0) {
         const uint32_t rmax = bv ? 8u * vbytes : L.r;
         switch (vbytes) {
-        case 1: return backsub_blocks<uint8_t>(L, Cg, (uint8_t *)Yg, Z, st, v, rmax, parts, lo, hi - lo);
-        case 2: return backsub_blocks<uint16_t>(L, Cg, (uint16_t *)Yg, Z, st, v, rmax, parts, lo, hi - lo);
-        default: return backsub_blocks<uint32_t>(L, Cg, (uint32_t *)Yg, Z, st, v, rmax, parts, lo, hi - lo);
+        case 1: return backsub_blocks<uint8_t>(L, Cg, (uint8_t *)Yg, Z, st, v, rmax, parts, p.first, p.slots);
+        case 2: return backsub_blocks<uint16_t>(L, Cg, (uint16_t *)Yg, Z, st, v, rmax, parts, p.first, p.slots);
+        default: return backsub_blocks<uint32_t>(L, Cg, (uint32_t *)Yg, Z, st, v, rmax, parts, p.first, p.slots);
         }
     }
     const uint32_t pl = vbytes == 1 ? 1u : vbytes;
@@ -422,8 +441,7 @@ cudaError_t launch_backsub(const LayerDesc &L, uint32_t vbytes, uint64_t *Cg, vo
 }
 
 uint32_t backsub_kernel_count(const LayerDesc &L, const BatchView *bv) {
-    const uint64_t parts = bv ? bv->nparts : (part_end(L) > L.part_lo ? part_end(L) - L.part_lo : 0);
-    return bs_in_blocks(bv, parts) ? 2u : 1u;
+    return bs_plan(L, bv).blocks ? 2u : 1u;
 }
 
 }  // namespace burr
