@@ -708,7 +708,9 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
                     CK(launch_sort_slack_pass1(L, vb, cur_k, cur_v, 0, cur_n, ss, err, st), "sort");
                 }
                 CK(launch_sort_slack_end(L, vb, (uint64_t *)sk, sv, (uint32_t *)bst, ss, err, st), "sort");
+                sort_slack_packing(L, vb, ss);   // what the cut search and the band read
             } else {
+                L.hbase = nullptr;
                 CK(launch_sort(L, vb, cur_k, cur_v, (uint64_t *)sk, sv, (uint32_t *)bst, ss, err, st), "sort");
             }
             CK(start_backsub(), "backsub");   // the previous layer's, now that this layer's sort is queued
@@ -750,7 +752,7 @@ int build_impl(const uint64_t *keys, const void *values, uint64_t n, uint32_t r,
             tev[l][2] = tm.mark();
             if (onep) CK(launch_thresh_flags(tex, dseg, blkseg, (uint32_t)nd, S.flags, tcounts, S.dir, st), "flags");
             pending = PendingBacksub{true, l, set, Lpend, S.z};
-            h->launches += (slack ? 6 : sort_kernel_count(L)) + 1 + backsub_kernel_count(Lpend) + (onep ? 2 : 0);
+            h->launches += (slack ? 7 : sort_kernel_count(L)) + 1 + backsub_kernel_count(Lpend) + (onep ? 2 : 0);
             CK(cudaMemcpyAsync((void *)hc, ctr, 16, cudaMemcpyDeviceToHost, st), "read counters");
             if (onep) CK(cudaMemcpyAsync((void *)hflag, S.dir + nd, 4, cudaMemcpyDeviceToHost, st), "read threshold count");
             CK(cudaStreamSynchronize(st), "layer");

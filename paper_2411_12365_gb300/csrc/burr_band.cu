@@ -138,7 +138,7 @@ struct BandSmem {
 template <typename V>
 struct BandArgs {
     LayerDesc L;
-    const uint64_t *keys;    // bucket-sorted records h = mix64(key ^ sigma) of the layer's keys
+    const uint64_t *keys;    // bucket-sorted records h = mix64(key ^ sigma) of the layer's keys (or packed)
     const V *vals;
     const uint32_t *bstart;
     uint64_t *Cg;
@@ -197,6 +197,19 @@ __device__ __forceinline__ void scan_first(uint32_t *first, int lane) {
     __syncwarp();
 }
 
+// Record h and value of equation i (base: the bucket's entry of L.hbase if packed).
+template <typename V>
+__device__ __forceinline__ uint64_t record(const uint64_t *keys, const V *vals, uint32_t i, bool packed, uint64_t base,
+                                           uint32_t &v) {
+    const uint64_t k = keys[i];
+    if (sizeof(V) == 1 && packed) {
+        v = packed_value(k);
+        return packed_h(k, base);
+    }
+    v = (uint32_t)vals[i];
+    return k;
+}
+
 // Stage the rows of bucket [rs, re) (start slot bB) at offsets >= the returned
 // threshold, in ascending offset order; first[o] = first index with offset
 // >= o.  The rows at offsets >= o span 63 + B - o slots, so where there are
@@ -208,6 +221,8 @@ template <typename V>
 __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, const BandArgs<V> &a, const LayerDesc &L,
                                             uint32_t rs, uint32_t re, uint32_t bB, uint32_t forced, int lane) {
     const uint32_t cnt = re - rs;
+    const bool packed = sizeof(V) == 1 && L.hbase;
+    const uint64_t base = packed ? L.hbase[(bB / L.B) >> L.hshift] : 0ull;
     for (int i = lane; i < 132; i += 32) first[i] = 0;
     __syncwarp();
     if (cnt <= (uint32_t)kStage) {
@@ -217,10 +232,10 @@ __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, co
         for (int j = 0; j < kStagePerLane; ++j) {
             const uint32_t i = (uint32_t)lane + 32u * j;
             if (i < cnt) {
-                const uint64_t h = a.keys[rs + i];     // the record h of the key
+                const uint64_t h = record(a.keys, a.vals, rs + i, packed, base, y[j]);
                 c[j] = coeff_of_h(h, L.sigma);
                 const uint32_t o = start_of_h(h, L.range) - bB;
-                y[j] = (uint32_t)a.vals[rs + i] & L.vmask;
+                y[j] &= L.vmask;
                 at[j] = o | atomicAdd(&first[o], 1u) << 8;
             }
         }
@@ -238,7 +253,9 @@ __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, co
         return forced;
     }
     // more rows than can be kept: count, find the threshold, stage the rows above it
-    for (uint32_t i = rs + lane; i < re; i += 32) atomicAdd(&first[start_of_h(a.keys[i], L.range) - bB], 1u);
+    uint32_t v = 0;
+    for (uint32_t i = rs + lane; i < re; i += 32)
+        atomicAdd(&first[start_of_h(record(a.keys, a.vals, i, packed, base, v), L.range) - bB], 1u);
     __syncwarp();
     scan_first(first, lane);
     uint32_t over = 0;   // one above the largest offset o with more than 63 + B - o rows at offsets >= o
@@ -250,7 +267,7 @@ __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, co
     for (int i = lane; i < 132; i += 32) first[i] = 0;
     __syncwarp();
     for (uint32_t i = rs + lane; i < re; i += 32) {
-        const uint32_t o = start_of_h(a.keys[i], L.range) - bB;
+        const uint32_t o = start_of_h(record(a.keys, a.vals, i, packed, base, v), L.range) - bB;
         if (o >= t) atomicAdd(&first[o], 1u);
     }
     __syncwarp();
@@ -258,21 +275,21 @@ __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, co
     // place the rows: the cursor of offset o is first[o] itself, which then ends where offset
     // o + 1 starts
     for (uint32_t i = rs + lane; i < re; i += 32) {
-        const uint64_t h = a.keys[i];
+        const uint64_t h = record(a.keys, a.vals, i, packed, base, v);
         const uint32_t o = start_of_h(h, L.range) - bB;
         if (o >= t) {
             const uint64_t c = coeff_of_h(h, L.sigma);
             const uint32_t p = atomicAdd(&first[o], 1u);
-            rows[p] = StagedRow{(uint32_t)c, (uint32_t)(c >> 32), (uint32_t)a.vals[i] & L.vmask, o};
+            rows[p] = StagedRow{(uint32_t)c, (uint32_t)(c >> 32), v & L.vmask, o};
         }
     }
     __syncwarp();
-    uint32_t v[4];
+    uint32_t f[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = first[4 * lane + k];
+    for (int k = 0; k < 4; ++k) f[k] = first[4 * lane + k];
     __syncwarp();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) first[4 * lane + k + 1] = v[k];
+    for (int k = 0; k < 4; ++k) first[4 * lane + k + 1] = f[k];
     if (lane == 0) first[0] = 0;
     __syncwarp();
     return t;
@@ -283,17 +300,18 @@ __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, co
 template <typename V>
 __device__ __noinline__ void emit_bumped(const BandArgs<V> &a, const Ctx &x, uint32_t rs, uint32_t re, uint32_t bB,
                                          uint32_t t, int lane) {
+    const bool packed = sizeof(V) == 1 && x.L.hbase;
+    const uint64_t hb = packed ? x.L.hbase[(bB / x.L.B) >> x.L.hshift] : 0ull;
     for (uint32_t base = rs; base < re; base += 32) {
         const uint32_t idx = base + lane;
         bool bump = false;
         uint64_t key = 0;
-        V val = 0;
+        uint32_t val = 0;
         if (idx < re) {
-            const uint64_t h = a.keys[idx];
+            const uint64_t h = record(a.keys, a.vals, idx, packed, hb, val);
             bump = (start_of_h(h, x.L.range) - bB) < t;
             if (bump) {
                 key = key_of_h(h, x.L.sigma);
-                val = a.vals[idx];
             }
         }
         const uint32_t mask = __ballot_sync(kFull, bump);
@@ -304,7 +322,7 @@ __device__ __noinline__ void emit_bumped(const BandArgs<V> &a, const Ctx &x, uin
         if (bump) {
             const unsigned long long o = x.out_base + ob + __popc(mask & ((1u << lane) - 1u));
             a.bkeys[o] = key;
-            a.bvals[o] = val;
+            a.bvals[o] = (V)val;
         }
     }
 }
@@ -721,7 +739,7 @@ __device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &
         if (lane < 16) {
             const uint32_t k = re + (uint32_t)lane * (128u / sizeof(uint64_t));
             if (k < x.pend) prefetch_l2(a.keys + k);
-        } else if (lane < 24) {
+        } else if (lane < 24 && !(sizeof(V) == 1 && L.hbase)) {
             const uint32_t k = re + (uint32_t)(lane - 16) * (128u / sizeof(V));
             if (k < x.pend) prefetch_l2(a.vals + k);
         }

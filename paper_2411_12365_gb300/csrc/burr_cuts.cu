@@ -23,8 +23,10 @@ __device__ __forceinline__ uint32_t count_offsets(const uint64_t *__restrict__ k
                                                   uint64_t g, uint64_t b, uint32_t lo, uint32_t hi, int lane) {
     uint32_t c = 0;
     const uint32_t e = bstart[g + 1];
+    const uint64_t base = L.hbase ? L.hbase[b >> L.hshift] : 0ull;
     for (uint32_t i = bstart[g] + (uint32_t)lane; i < e; i += 32) {
-        const uint32_t o = start_of_h(keys[i], L.range) - (uint32_t)(b * L.B);   // keys[] holds records h
+        const uint64_t h = L.hbase ? packed_h(keys[i], base) : keys[i];   // keys[] holds records
+        const uint32_t o = start_of_h(h, L.range) - (uint32_t)(b * L.B);
         c += (o >= lo && o < hi) ? 1u : 0u;
     }
     for (int d = 16; d; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);

@@ -100,8 +100,18 @@ struct LayerDesc {
     uint32_t test_slack; // 1: the fixed-capacity sort bins get half their expected size (testing the exact redo)
     uint32_t part_lo;    // band and back-substitution launches cover partitions [part_lo, part_hi)
     uint32_t part_hi;    // (0: up to K); a shard of a sharded build owns such a range
+    const uint64_t *hbase; // device: the sorted records are packed (see packed_h); nullptr: plain records
+    uint32_t hshift;       // log2 of the buckets that share an entry of hbase
     const uint32_t *cuts;  // device: first bucket of each partition, [K] = nb; nullptr: partition j at j*P
 };
+
+// Packed records.  The keys of a bin of consecutive buckets have their h in
+// [base, base + 2^56) where a layer has more than 256 such bins, so h - base and a
+// one-byte value share 8 bytes: the passes after the first and the band then
+// move no values of their own.  The bin of bucket b is b >> hshift.
+constexpr uint64_t kPackedMask = (1ull << 56) - 1;
+__host__ __device__ __forceinline__ uint64_t packed_h(uint64_t x, uint64_t base) { return base + (x & kPackedMask); }
+__host__ __device__ __forceinline__ uint32_t packed_value(uint64_t x) { return (uint32_t)(x >> 56); }
 
 // End of the partition range a launch covers.
 __host__ __device__ inline uint64_t part_end(const LayerDesc &L) { return L.part_hi ? L.part_hi : L.K; }
@@ -172,6 +182,9 @@ cudaError_t launch_sort(const LayerDesc &L, uint32_t vbytes, const uint64_t *key
 // kErrSortSlack and the output holds only part of the keys (each in its right
 // place): the caller sorts again with launch_sort.
 size_t sort_slack_scratch_bytes(const LayerDesc &L, uint32_t vbytes);
+// Sets L.hbase and L.hshift if the sort's output is packed records (values of
+// one byte, then vals_out is not written); the table lies in the scratch.
+void sort_slack_packing(LayerDesc &L, uint32_t vbytes, void *scratch);
 cudaError_t launch_sort_slack_begin(const LayerDesc &L, uint32_t vbytes, void *scratch, cudaStream_t st);
 cudaError_t launch_sort_slack_pass1(const LayerDesc &L, uint32_t vbytes, const uint64_t *keys, const void *vals,
                                     uint64_t lo, uint64_t hi, void *scratch, uint32_t *err, cudaStream_t st);

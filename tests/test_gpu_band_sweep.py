@@ -48,3 +48,20 @@ def test_sweep_matches_oracle(n, r, alpha, kw, mode):
     assert ref.ok
     want = ref.export()
     assert got == want, describe_difference(got, want)
+
+
+@pytest.mark.parametrize("r,mode,cut,alpha", [(8, burr.THRESH_2BIT, burr.CUT_NONE, 1.015),
+                                              (3, burr.THRESH_1PLUS, burr.CUT_DIFF, 1.015),
+                                              (1, burr.THRESH_2BIT, burr.CUT_MINBUMP, 1.6)])
+def test_packed_records_match_oracle(r, mode, cut, alpha):
+    """Layers sorted in two passes with one-byte values: records and values travel
+    packed; just past the smallest such layer, whole exports against the oracle."""
+    n = int(8_400_000 * alpha) + 101
+    keys = I.keys_torch(n, "cuda", seed=r)
+    vals = I.values_torch(keys, r)
+    got = burr.build(keys, vals, r, threshold_mode=mode, cut_search=cut, load_factor=alpha).export()
+    ref = O.build(keys.cpu().numpy().view(np.uint64), vals.cpu().numpy().astype(np.uint32), threads=16, r=r,
+                  threshold_mode=mode, cut_search=cut, alpha=alpha)
+    assert ref.ok
+    want = ref.export()
+    assert got == want, describe_difference(got, want)
