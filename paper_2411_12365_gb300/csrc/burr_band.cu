@@ -132,6 +132,7 @@ struct BandSmem {
     uint32_t sweeper;              // the warp that sweeps
     uint32_t failed;               // the build has failed already
     Pivot snap[2][32];             // live rows at the bucket's start
+    alignas(4) uint8_t stored[64]; // rows (lane, and 32 + lane) that a block of slots stored
     Ctx x;
 };
 
@@ -219,10 +220,9 @@ __device__ __forceinline__ uint64_t record(const uint64_t *keys, const V *vals, 
 // its registers would stay live across the sweep.
 template <typename V>
 __device__ __noinline__ uint32_t stage_rows(StagedRow *rows, uint32_t *first, const BandArgs<V> &a, const LayerDesc &L,
-                                            uint32_t rs, uint32_t re, uint32_t bB, uint32_t forced, int lane) {
+                                            uint32_t rs, uint32_t re, uint32_t bB, uint32_t forced,
+                                            bool packed, uint64_t base, int lane) {
     const uint32_t cnt = re - rs;
-    const bool packed = sizeof(V) == 1 && L.hbase;
-    const uint64_t base = packed ? L.hbase[(bB / L.B) >> L.hshift] : 0ull;
     for (int i = lane; i < 132; i += 32) first[i] = 0;
     __syncwarp();
     if (cnt <= (uint32_t)kStage) {
@@ -525,11 +525,14 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
             if (zb) B.key = 0;
             continue;
         }
-        for (uint32_t k = 0; k < w; ++k) {   // the rows that were stored are free
-            const uint32_t x = __shfl_sync(kFull, K, (int)k);
-            if (x && ((x ^ A.key) & ~kValueMask) == 0u) A.key = 0;
-            if (x && ((x ^ B.key) & ~kValueMask) == 0u) B.key = 0;
-        }
+        // the rows that were stored are free, which the block's keys tell the lanes (a shuffle per
+        // slot instead took 1,000 cycles)
+        if (lane < 16) reinterpret_cast<uint32_t *>(S.stored)[lane] = 0;
+        __syncwarp();
+        if (K) S.stored[(K & 31u) | (K >> kRowBit & 1u) << 5] = 1;
+        __syncwarp();
+        if (S.stored[lane]) A.key = 0;
+        if (S.stored[32 + lane]) B.key = 0;
         const uint32_t D = __reduce_max_sync(kFull, max(za ? A.key : 0u, zb ? B.key : 0u));
         if (L.fallback) return unsolvable();
         if (D == 0 || (D >= kOldKey && o >= 64)) {   // not expected
@@ -730,7 +733,15 @@ __device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &
     const uint64_t own_hi = b1 == x.b1 ? x.own_hi : (uint64_t)b1 * Bs;
     uint64_t tword = 0;
     uint32_t rs = a.bstart[x.bucket_base + b0];   // first equation of the next bucket to stage
+    // packed records: the entry of hbase holds for 2^hshift buckets
+    const bool packed = sizeof(V) == 1 && L.hbase;
+    uint32_t bin = ~0u;
+    uint64_t base = 0;
     auto stage = [&](uint32_t b) {
+        if (packed && b >> L.hshift != bin) {
+            bin = b >> L.hshift;
+            base = L.hbase[bin];
+        }
         const uint32_t q = b & 1u, re = a.bstart[x.bucket_base + b + 1];
         uint32_t t = 0;
         if (x.part > 0 && b == x.b0 && !L.fallback)
@@ -739,11 +750,11 @@ __device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &
         if (lane < 16) {
             const uint32_t k = re + (uint32_t)lane * (128u / sizeof(uint64_t));
             if (k < x.pend) prefetch_l2(a.keys + k);
-        } else if (lane < 24 && !(sizeof(V) == 1 && L.hbase)) {
+        } else if (lane < 24 && !packed) {
             const uint32_t k = re + (uint32_t)(lane - 16) * (128u / sizeof(V));
             if (k < x.pend) prefetch_l2(a.vals + k);
         }
-        const uint32_t ts = stage_rows(S.rows[q], S.first[q], a, L, rs, re, b * Bs, t, lane);
+        const uint32_t ts = stage_rows(S.rows[q], S.first[q], a, L, rs, re, b * Bs, t, packed, base, lane);
         if (lane == 0) S.tstage[q] = ts;
         rs = re;
         if (ts > t && L.fallback) {
@@ -912,7 +923,8 @@ __global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t npa
 // 2*10^5 5.7 / 2.0, 10^6 6.2 / 4.0, 3*10^6 6.5 / 5.3, 6*10^6 (91 partitions, segments
 // of 128; of 256: 6.7) 6.3 / 5.4, but 10^7 6.4 / 7.1.
 constexpr uint64_t kSegCap = 2432, kSegMin = 32, kSegCapExact = 460, kSegMaxExact = 128;
-constexpr uint32_t kSegPasses = 7;
+// Passes before the last one: enough for runs that meet after 190 buckets.
+inline uint32_t seg_passes(uint32_t seg) { return 1 + (190 + seg - 1) / seg; }
 struct SegPlan {
     uint32_t seg = 0, nseg = 0;
     uint64_t parts = 0, buckets = 0;
@@ -993,8 +1005,9 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
     const bool fallback = bv ? bv->fallback : L.fallback != 0;
     cudaError_t e;
     if ((e = prefer_shared(k_band_seg<V>)) != cudaSuccess || (e = prefer_shared(k_band_finish<V>)) != cudaSuccess) return e;
-    for (uint32_t pass = 0; pass < kSegPasses; ++pass) k_band_seg<V><<<parts * p.nseg, 64, 0, st>>>(a, parts, pass, false);
-    k_band_seg<V><<<parts, 64, 0, st>>>(a, parts, kSegPasses, true);
+    const uint32_t passes = seg_passes(p.seg);
+    for (uint32_t pass = 0; pass < passes; ++pass) k_band_seg<V><<<parts * p.nseg, 64, 0, st>>>(a, parts, pass, false);
+    k_band_seg<V><<<parts, 64, 0, st>>>(a, parts, passes, true);
     // a partition's buckets may start inside a code word
     if (!fallback) k_band_finish<V><<<parts * (p.nseg * p.seg / 32 + 2), 128, 0, st>>>(a, parts);
     return cudaGetLastError();
@@ -1011,7 +1024,8 @@ size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv) {
 }
 
 uint32_t band_kernel_count(const LayerDesc &L, const BatchView *bv) {
-    return band_scratch_bytes(L, bv) == 0 ? 1u : kSegPasses + ((bv ? bv->fallback : L.fallback != 0) ? 1u : 2u);
+    if (band_scratch_bytes(L, bv) == 0) return 1u;
+    return seg_passes(seg_plan(L, bv).seg) + ((bv ? bv->fallback : L.fallback != 0) ? 1u : 2u);
 }
 
 cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *keys, const void *vals,
