@@ -41,10 +41,10 @@
 // eliminating one row each against a band in shared memory, a 128-bit
 // compare-and-swap per step, every bucket as long as its longest chain, a
 // dependent bucket inserted again):
-//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 2.9 (in segments 0.75)
-//   10^6 keys (16 partitions)                     6.57 -> 3.9 (in segments 1.27)
-//   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 6.4
-//   10^8 keys (1504 partitions)                   8.33 -> 6.3;  1+-bit 16.3 -> 9.3
+//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 2.9 (in segments 0.79)
+//   10^6 keys (16 partitions)                     6.57 -> 3.9 (in segments 1.23)
+//   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 6.1
+//   10^8 keys (1504 partitions)                   8.33 -> 6.2;  1+-bit 16.3 -> 9.0
 //   10^9 keys (15034 partitions)                  63.7 -> 47.4
 #include <algorithm>
 
@@ -448,12 +448,14 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         return false;
     };
     const bool test_window = L.window != 0;
-    const uint32_t total = first[128];
     uint32_t nfree = W.nfree(), i0, up;
-    // first staged index of slot W.o, and (per lane) of the slot after W.o + lane
+    // first staged index of slot W.o, and (per lane) of the slot after W.o + lane.  The bookkeeping
+    // between blocks (about ten per bucket) is kept short: i0 advances by the rows taken, and a row's
+    // place among them tells whether it is taken (10^7 keys, 1+-bit: 6.46 -> 6.05 ms; 10^8 6.36 -> 6.22)
+    auto look_ahead = [&](uint32_t o) { up = max(first[min(o + 1u + (uint32_t)lane, lim)], W.it); };
     auto look = [&](uint32_t o) {
         i0 = max(first[o], W.it);
-        up = max(first[min(o + 1u + (uint32_t)lane, lim)], i0);
+        look_ahead(o);
     };
     look(W.o);
     while (W.o < lim) {
@@ -461,8 +463,11 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         // the rows that the lanes' free registers would take, read before the block's length is known
         const uint32_t ra = i0 + (uint32_t)__popc(W.fa & lt), rb = i0 + (uint32_t)(__popc(W.fa) + __popc(W.fb & lt));
         const StagedRow sa = rows[min(ra, (uint32_t)kStage - 1u)], sb = rows[min(rb, (uint32_t)kStage - 1u)];
-        // the longest block of slots (up to 32) whose new rows fit the free registers
+        // the longest block of slots (up to 32) whose new rows fit the free registers, and their number
         const uint32_t w = (uint32_t)__popc(__ballot_sync(kFull, up - i0 <= nfree && o + (uint32_t)lane < lim));
+        const uint32_t cnt = w ? __shfl_sync(kFull, up - i0, (int)w - 1) : 0u;
+        // (one maximum over both, and the empty slots from the least key stored instead of the block's
+        // keys: 6.46 -> 6.18 as well alone, but 10^8 keys 6.36 -> 6.47 and 10^9 47.7 -> 48.9 ms)
         if (w == 0) {
             // more than 64 rows in 64 slots: the lowest-offset row of the bucket goes
             if (L.fallback) return unsolvable();
@@ -479,7 +484,6 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
             look(o);
             continue;
         }
-        const uint32_t cnt = __shfl_sync(kFull, up - i0, (int)w - 1);
         if (test_window && o < 64 && o + L.B >= L.window && __any_sync(kFull, max(A.key, B.key) >= kOldKey)) {
             // testing only: a row would be stored past the window that the test asked for
             if (lane == 0) atomicOr(a.err, kErrRingOverflow);
@@ -488,14 +492,15 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         if (cnt == 0 && nfree == 64) {   // no live row: empty slots
             if ((uint32_t)lane < w) S.ring[(bB + o + (uint32_t)lane) & kRingMask].key = 0;
             W.o += w;
-            look(W.o);
+            look_ahead(W.o);
             continue;
         }
         A.gate = B.gate = kFull;
-        if (A.key == 0 && ra < total && sa.o < o + w) load_row<kPacked>(A, sa, o, (uint32_t)lane);
-        if (B.key == 0 && rb < total && sb.o < o + w) load_row<kPacked>(B, sb, o, 1u << kRowBit | (uint32_t)lane);
+        if (A.key == 0 && ra - i0 < cnt) load_row<kPacked>(A, sa, o, (uint32_t)lane);
+        if (B.key == 0 && rb - i0 < cnt) load_row<kPacked>(B, sb, o, 1u << kRowBit | (uint32_t)lane);
         W.o += w;
-        look(W.o);   // for the next block, during this one's sweep
+        i0 += cnt;
+        look_ahead(W.o);   // for the next block, during this one's sweep
         const Pivot *e = &S.ring[(bB + o) & kRingMask];
         const unsigned slot = (unsigned)__cvta_generic_to_shared(e);
         uint32_t c = 0;
@@ -514,10 +519,9 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         __syncwarp();
         // free registers: a live row that is zero was stored in this block, or it is dependent
         const bool za = (A.w0 | A.w1) == 0u, zb = (B.w0 | B.w1) == 0u;
-        const uint32_t K = (uint32_t)lane < w ? e[lane].key : 0u;
         W.fa = __ballot_sync(kFull, za);
         W.fb = __ballot_sync(kFull, zb);
-        const uint32_t np = (uint32_t)__popc(__ballot_sync(kFull, K != 0));
+        const uint32_t np = (uint32_t)__popc(__ballot_sync(kFull, (uint32_t)lane < w && e[lane].key != 0));
         const uint32_t expect = nfree - cnt + np;
         nfree = W.nfree();
         if (nfree == expect) {
@@ -527,6 +531,7 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         }
         // the rows that were stored are free, which the block's keys tell the lanes (a shuffle per
         // slot instead took 1,000 cycles)
+        const uint32_t K = (uint32_t)lane < w ? e[lane].key : 0u;
         if (lane < 16) reinterpret_cast<uint32_t *>(S.stored)[lane] = 0;
         __syncwarp();
         if (K) S.stored[(K & 31u) | (K >> kRowBit & 1u) << 5] = 1;
