@@ -770,7 +770,7 @@ def run_plain(a, ws, rank, local, pg):
                      "algorithmic_bytes": band_bytes,
                      "algorithmic_model": "read n0 sorted (key, value) records, write the bumped ones, "
                                           "write the 2-bit thresholds",
-                     "note": "band+bump is latency-bound (dependent GF(2) elimination chains); see issue"},
+                     "note": "band+bump is bound by the integer work of the GF(2) elimination; see issue"},
         "gpu_launches": launches[0],
     }
     line["clocks"] = clk.summary()
