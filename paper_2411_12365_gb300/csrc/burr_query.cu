@@ -102,6 +102,30 @@ __device__ __forceinline__ void load_window(const uint64_t *__restrict__ z, uint
     }
 }
 
+// The same words by loads of 16 bytes (R even) or 8, which need not be moved.
+template <int R>
+__device__ __forceinline__ void load_narrow(const uint64_t *__restrict__ z, uint32_t s, Window<R> &w) {
+    const uint64_t *p = z + (uint64_t)(s >> 6) * R;
+    const bool two = (s & 63u) != 0u;
+    if (R % 2 == 0) {
+        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(p);
+#pragma unroll
+        for (int k = 0; k < R; k += 2) {
+            const ulonglong2 x = __ldg(q + k / 2), y = two ? __ldg(q + (R + k) / 2) : ulonglong2{0ull, 0ull};
+            w.w[k] = x.x;
+            w.w[k + 1] = x.y;
+            w.w[R + k] = y.x;
+            w.w[R + k + 1] = y.y;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            w.w[k] = __ldg(p + k);
+            w.w[R + k] = two ? __ldg(p + R + k) : 0ull;
+        }
+    }
+}
+
 template <int R>
 __device__ __forceinline__ uint32_t eval_loaded(const Window<R> &w, uint32_t s, uint64_t c) {
     uint64_t cA, cB;
@@ -162,7 +186,10 @@ __device__ __forceinline__ uint32_t threshold_of(const QueryDesc &Q, uint32_t l,
 // Two keys per thread (their layer-0 reads in flight together, 98 registers)
 // gave 70.7 ms against 72.5 at 10^9 keys (r = 8) but 4.69 against 4.20 and 0.89
 // against 0.79 at 10^8 (r = 16, r = 1).
-template <typename V, int R, bool kKeep, bool kExact>
+//
+// kLoad: how the window is read (see query_r).
+enum { kWide = 0, kWideKeep = 1, kNarrow = 2 };   // 32-byte loads, kept in L1 or not; 16 or 8 bytes
+template <typename V, int R, int kLoad, bool kExact>
 __global__ void __launch_bounds__(kQThreads)
 k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -180,12 +207,14 @@ k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, u
             const uint32_t s = (uint32_t)__umul64hi(h, m - kW + 1);
             if constexpr (R <= 16) {
                 Window<R> w;
-                load_window<R, kKeep>(Q.z[l], s, w);
+                if (kLoad != kNarrow) load_window<R, kLoad == kWideKeep>(Q.z[l], s, w);
                 if (l < Q.layers && (s & (Q.B - 1)) < threshold_of<kExact>(Q, l, s >> log2B)) continue;   // bumped: next layer
+                // (read before the threshold is known they are slower: r = 7 in 100 KB 77 against 71 us, r = 15 167 / 144)
+                if (kLoad == kNarrow) load_narrow<R>(Q.z[l], s, w);
                 v = eval_loaded<R>(w, s, mix64(h + Q.sigma[l]) | 1ull);
             } else {
                 if (l < Q.layers && (s & (Q.B - 1)) < threshold_of<kExact>(Q, l, s >> log2B)) continue;
-                v = eval_planes<R, kKeep>(Q.z[l], s, mix64(h + Q.sigma[l]) | 1ull);
+                v = eval_planes<R, kLoad == kWideKeep>(Q.z[l], s, mix64(h + Q.sigma[l]) | 1ull);
             }
             break;
         }
@@ -203,7 +232,7 @@ k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, u
 // r = 8, 10^8 keys of a 100 MB table 1.71 -> 1.58 ms, 2*10^7 of a 1 MB table 445 ->
 // 290 us (1+-bit); r = 16, 5*10^6 of 20 MB 182 -> 118 us, 1+-bit 261 -> 130; r = 32,
 // 2*10^7 of 40 MB 1070 -> 717 us.
-template <typename V, int R, bool kExact>
+template <typename V, int R, bool kKeep, bool kExact>
 __global__ void __launch_bounds__(kQThreads)
 k_query_group(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
     constexpr int G = R / 4, kAtOnce = G < 4 ? G : 4;   // keys of the group whose reads are in flight together
@@ -231,9 +260,9 @@ k_query_group(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ ou
             for (int t = 0; t < kAtOnce; ++t) {
                 st[t] = __shfl_sync(0xffffffffu, s, first + t0 + t);
                 const uint64_t *p = z0 + (uint64_t)(st[t] >> 6) * R;
-                ldg_v4<false>(p, a[t][0], a[t][1], a[t][2], a[t][3]);
+                ldg_v4<kKeep>(p, a[t][0], a[t][1], a[t][2], a[t][3]);
                 b[t][0] = b[t][1] = b[t][2] = b[t][3] = 0;
-                if (st[t] & 63u) ldg_v4<false>(p + R, b[t][0], b[t][1], b[t][2], b[t][3]);
+                if (st[t] & 63u) ldg_v4<kKeep>(p + R, b[t][0], b[t][1], b[t][2], b[t][3]);
             }
 #pragma unroll
             for (int t = 0; t < kAtOnce; ++t) {
@@ -267,7 +296,9 @@ k_query_group(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ ou
     }
 }
 
-template <typename V>
+// kCodes: 2-bit thresholds only.  The other instance takes either mode: with the
+// mode fixed to 1+-bit it is slower (r = 3, 4*10^6 queries of 7 KB: 70 us against 54).
+template <typename V, bool kCodes>
 __global__ void __launch_bounds__(kQThreads)
 k_query(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -283,7 +314,8 @@ k_query(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uin
             const uint32_t s = (uint32_t)__umul64hi(h, m - kW + 1);
             const uint32_t b = s >> log2B;
             const uint32_t off = s & (Q.B - 1);
-            const uint32_t t = Q.mode == BURR_THRESH_1PLUS ? threshold_of<true>(Q, l, b) : threshold_of<false>(Q, l, b);
+            const uint32_t t = !kCodes && Q.mode == BURR_THRESH_1PLUS ? threshold_of<true>(Q, l, b)
+                                                                      : threshold_of<false>(Q, l, b);
             if (off < t) continue;                             // bumped: next layer
             v = eval_window(Q.z[l], Q.r, s, mix64(h + Q.sigma[l]) | 1ull);
             break;
@@ -313,29 +345,62 @@ __global__ void k_hash(const uint64_t *__restrict__ keys, uint64_t n, uint64_t s
 
 namespace {
 
-// The kernel of width Q.r, if there is one; false otherwise (wider values of
-// which the planes don't come in fours).
+// The kernel of width Q.r, if there is one for its table's size; false otherwise,
+// also for wider values of which the planes don't come in fours.
+//
+// Times in us for 4*10^6 queries, 2-bit thresholds unless said.  A table that
+// mostly stays in L1 or is met again there is read through it: groups up to
+// 128 KB (r = 8, 2 KB 62 against 393 without: few lines, all of them in
+// L2's way; 20 KB 55 / 104; r = 16, 200 KB 91 / 95, 800 KB 100 / 95), single keys up to 1 MB.
+// Below 8 KB groups only add work (r = 8: 62, one lane per key 56).
+// Widths that are no multiple of 4 pay for moving a window read by wide loads
+// (odd ones most).  Against narrow loads / any width's kernel, which reads plane
+// by plane in a loop, wide loads take:
+//   r = 2    20 KB..5 MB  39..40 / 34..36;   1+-bit 60..65 / 52..56
+//   r = 3    7 KB 48 / 36;  375 KB 52 / 50 (general 48);  1.5 MB 52 / 53;  7 MB 52 / 54
+//   r = 5    60 KB 64 / 52;  250 KB 66 (general 60);  625 KB 68 / 76 (general 70)
+//   r = 6    75 KB 57 / 46;  750 KB 64 / 64;  3 MB 64 / 67
+//   r = 10, 14   125, 175 KB 85, 109 / 60, 82;  1.3, 1.8 MB 97, 127 / 99, 141
+//   r = 13, 15   160, 190 KB 134, 157 / 126, 144;  1.6, 1.9 MB 152, 177 / 167, 199
+// and with 1+-bit thresholds, whose loads take the registers, even widths are best
+// narrow (r = 6, 10, 14 in 12 to 35 MB: 101, 175, 195 / 83, 124, 162), odd ones up to
+// 11 in the general kernel (r = 5 in 625 KB: 99 / 98 / 81), 13 and 15 narrow (1.6, 1.9 MB:
+// 204, 220 / 196, 226).
 template <int R>
-void query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
+bool query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
     using V = std::conditional_t<(R <= 8), uint8_t, std::conditional_t<(R <= 16), uint16_t, uint32_t>>;
-    // a table of at most 1 MB (layer 0 holds nearly all of it) mostly stays in L1 or is met again there
-    const bool keep = (Q.m[0] / 64) * R * 8 <= (1ull << 20), exact = Q.mode == BURR_THRESH_1PLUS;
+    const uint64_t kb = (Q.m[0] / 64) * R * 8 >> 10;   // layer 0 holds nearly all of the table
+    const bool exact = Q.mode == BURR_THRESH_1PLUS;
+    auto go = [&](auto *kernel) {
+        kernel<<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n);
+        return true;
+    };
     if constexpr (R == 8 || R == 16 || R == 32) {
-        if (Q.layers > 0 && Q.m[0] != 0) {   // (without bumping layers there is no layer 0 with thresholds)
-            if (exact) k_query_group<V, R, true><<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n);
-            else k_query_group<V, R, false><<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n);
-            return;
+        // (without bumping layers there is no layer 0 with thresholds)
+        if (Q.layers > 0 && Q.m[0] != 0 && (R != 8 || kb >= 8)) {
+            if (kb < 128) return exact ? go(k_query_group<V, R, true, true>) : go(k_query_group<V, R, true, false>);
+            return exact ? go(k_query_group<V, R, false, true>) : go(k_query_group<V, R, false, false>);
         }
     }
-    auto go = [&](auto *kernel) { kernel<<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n); };
-    if (exact) keep ? go(k_query_r<V, R, true, true>) : go(k_query_r<V, R, false, true>);
-    else keep ? go(k_query_r<V, R, true, false>) : go(k_query_r<V, R, false, false>);
+    if constexpr (R % 4 != 0 && R != 1) {
+        if (exact) return R % 2 == 0 || R >= 13 ? go(k_query_r<V, R, kNarrow, true>) : false;
+        constexpr uint64_t kNarrowKb = R == 2 ? ~0ull : R % 2 == 0 ? 512 : R >= 7 ? 256 : 64;
+        constexpr uint64_t kGeneralKb = R == 3 ? 1536 : R == 5 ? 512 : 0;
+        if (kb < kNarrowKb) return go(k_query_r<V, R, kNarrow, false>);
+        if constexpr (kGeneralKb != 0) {
+            if (kb < kGeneralKb) return false;
+        }
+        return kb < 1024 ? go(k_query_r<V, R, kWideKeep, false>) : go(k_query_r<V, R, kWide, false>);
+    } else {
+        if (kb < 1024) return exact ? go(k_query_r<V, R, kWideKeep, true>) : go(k_query_r<V, R, kWideKeep, false>);
+        return exact ? go(k_query_r<V, R, kWide, true>) : go(k_query_r<V, R, kWide, false>);
+    }
 }
 
 bool launch_query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
     switch (Q.r) {
 #define BURR_QUERY_R(R) \
-    case R: query_r<R>(Q, keys, out, n, grid, st); return true;
+    case R: return query_r<R>(Q, keys, out, n, grid, st);
         BURR_QUERY_R(1) BURR_QUERY_R(2) BURR_QUERY_R(3) BURR_QUERY_R(4) BURR_QUERY_R(5) BURR_QUERY_R(6)
         BURR_QUERY_R(7) BURR_QUERY_R(8) BURR_QUERY_R(9) BURR_QUERY_R(10) BURR_QUERY_R(11) BURR_QUERY_R(12)
         BURR_QUERY_R(13) BURR_QUERY_R(14) BURR_QUERY_R(15) BURR_QUERY_R(16) BURR_QUERY_R(20) BURR_QUERY_R(24)
@@ -357,10 +422,13 @@ cudaError_t launch_query(const QueryDesc &Q, uint32_t vbytes, const uint64_t *ke
     for (uint32_t l = 0; l <= Q.layers; ++l)
         if (Q.m[l] != 0 && ((uintptr_t)Q.z[l] & 31u) != 0) wide = false;
     if (wide && launch_query_r(Q, keys, out, n, grid, st)) return cudaGetLastError();
+    auto go = [&](auto *any, auto *codes, auto *v) {
+        (Q.mode == BURR_THRESH_1PLUS ? any : codes)<<<grid, kQThreads, 0, st>>>(Q, keys, v, n);
+    };
     switch (vbytes) {
-    case 1: k_query<uint8_t><<<grid, kQThreads, 0, st>>>(Q, keys, (uint8_t *)out, n); break;
-    case 2: k_query<uint16_t><<<grid, kQThreads, 0, st>>>(Q, keys, (uint16_t *)out, n); break;
-    default: k_query<uint32_t><<<grid, kQThreads, 0, st>>>(Q, keys, (uint32_t *)out, n); break;
+    case 1: go(k_query<uint8_t, false>, k_query<uint8_t, true>, (uint8_t *)out); break;
+    case 2: go(k_query<uint16_t, false>, k_query<uint16_t, true>, (uint16_t *)out); break;
+    default: go(k_query<uint32_t, false>, k_query<uint32_t, true>, (uint32_t *)out); break;
     }
     return cudaGetLastError();
 }

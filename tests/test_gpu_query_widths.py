@@ -44,3 +44,16 @@ def test_no_bumping_layers():
         vals = I.values_torch(keys, r)
         h = burr.build(keys, vals, r, layers=0)
         assert torch.equal(h.query(keys[:1_001]), vals[:1_001])
+
+
+@pytest.mark.parametrize("r,n", [(3, 300_000), (3, 4_400_000), (5, 150_000), (5, 900_000), (6, 800_000), (7, 320_000),
+                                 (8, 9_001), (13, 180_000), (14, 320_000), (15, 150_000), (16, 80_000), (32, 40_000)])
+def test_larger_tables_are_read_otherwise_and_equal(r, n):
+    """Tables past the sizes at which a width changes its loads or leaves L1."""
+    keys = I.keys_torch(n, "cuda", seed=r)
+    vals = I.values_torch(keys, r)
+    h = burr.build(keys, vals, r)
+    ref = O.build(keys.cpu().numpy().view(np.uint64), _u32(vals), r=r)
+    assert torch.equal(h.query(keys), vals)
+    others = I.keys_torch(20_011, "cuda", offset=1 << 40)
+    assert np.array_equal(_u32(h.query(others)), ref.query(others.cpu().numpy().view(np.uint64)))
