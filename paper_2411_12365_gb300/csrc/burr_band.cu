@@ -714,9 +714,16 @@ __device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &
                         const uint32_t k0 = S.ring[(bB + lane) & kRingMask].key, k1 = S.ring[(bB + 32 + lane) & kRingMask].key;
                         const uint64_t mine = (uint64_t)__ballot_sync(kFull, k1 >= kOldKey) << 32 |
                                               __ballot_sync(kFull, k0 >= kOldKey);
+                        // one lane reads the stored mask and replaces it, so the store follows the
+                        // read (other lanes' reads would have to be ordered before it)
                         uint64_t *om = a.omask + x.bucket_base + b;
-                        if (R.compare && same_space(S, a, x.slot_base + (uint64_t)b * Bs, bB, mine, *om, lane)) why = kRunCoupled;
-                        else if (lane == 0) *om = mine;
+                        if (R.compare) {
+                            uint64_t theirs = 0;
+                            if (lane == 0) theirs = *om;
+                            theirs = __shfl_sync(kFull, theirs, 0);
+                            if (same_space(S, a, x.slot_base + (uint64_t)b * Bs, bB, mine, theirs, lane)) why = kRunCoupled;
+                        }
+                        if (lane == 0 && why == kRunDone) *om = mine;
                     } else if (R.out) {
                         R.out[lane] = S.snap[0][lane];
                         R.out[32 + lane] = S.snap[1][lane];
