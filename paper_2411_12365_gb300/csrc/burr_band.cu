@@ -491,6 +491,7 @@ __device__ __forceinline__ bool sweep_to(BandSmem &S, const BandArgs<V> &a, Swee
         }
         if (cnt == 0 && nfree == 64) {   // no live row: empty slots
             if ((uint32_t)lane < w) S.ring[(bB + o + (uint32_t)lane) & kRingMask].key = 0;
+            __syncwarp();   // the caller's lanes read other lanes' slots
             W.o += w;
             look_ahead(W.o);
             continue;

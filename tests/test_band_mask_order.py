@@ -1,15 +1,19 @@
-"""The stored mask of a bucket in the segmented band is read and replaced by one
-lane.  A race between the lanes of a warp seldom shows in results, so the source
-is checked: every access to the mask stands under `lane == 0`."""
+"""Order of the band's accesses to memory that lanes and warps share.  A race
+between them seldom shows in results, so the source is checked."""
 import os
 import re
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def test_one_lane_reads_and_replaces_the_stored_mask():
+def _source():
     src = open(os.path.join(ROOT, "paper_2411_12365_gb300", "csrc", "burr_band.cu")).read()
-    src = re.sub(r"//[^\n]*", "", src)
+    return re.sub(r"//[^\n]*", "", src)
+
+
+def test_one_lane_reads_and_replaces_the_stored_mask():
+    """Every access to the stored mask of a bucket stands under `lane == 0`."""
+    src = _source()
     decl = re.search(r"uint64_t \*om\s*=\s*a\.omask[^;]*;", src)
     assert decl
     body = src[decl.end():src.index("S.tdone", decl.end())]
@@ -19,3 +23,11 @@ def test_one_lane_reads_and_replaces_the_stored_mask():
         statement = body[max(body.rfind(c, 0, u) for c in ";{}") + 1:u]
         assert re.match(r"\s*if \(lane == 0\b", statement), statement
     assert len(re.findall(r"\bomask\b", src)) == 3   # declared, used above, and set by the launch
+
+
+def test_stores_of_empty_slots_are_followed_by_a_warp_barrier():
+    """Lanes read slots that others emptied (the masks of a bucket's first slots)."""
+    src = _source()
+    store = re.search(r"S\.ring\[\(bB \+ o \+ \(uint32_t\)lane\) & kRingMask\]\.key = 0;", src)
+    assert store
+    assert "__syncwarp();" in src[store.end():src.index("continue;", store.end())]
