@@ -731,8 +731,10 @@ __device__ __forceinline__ uint32_t run_buckets(BandSmem &S, const BandArgs<V> &
                     }
                 }
                 if (lane == 0) {
-                    S.tdone = W.tprev;
-                    S.at = b;
+                    if (half == 0) {   // (final then; the other warp reads it during the second half)
+                        S.tdone = W.tprev;
+                        S.at = b;
+                    }
                     if (why) S.stop[half] = why;
                 }
                 pair_sync();

@@ -31,3 +31,11 @@ def test_stores_of_empty_slots_are_followed_by_a_warp_barrier():
     store = re.search(r"S\.ring\[\(bB \+ o \+ \(uint32_t\)lane\) & kRingMask\]\.key = 0;", src)
     assert store
     assert "__syncwarp();" in src[store.end():src.index("continue;", store.end())]
+
+
+def test_final_threshold_is_written_before_the_second_half_only():
+    """The staging warp reads it while the sweeping warp is in the second half."""
+    src = _source()
+    writes = [m.start() for m in re.finditer(r"S\.tdone = ", src)]
+    assert len(writes) == 1
+    assert re.search(r"if \(half == 0\) \{\s*$", src[:writes[0]])
