@@ -13,10 +13,13 @@
 #include <memory>
 #include <string>
 #include <mutex>
+#include <new>
 #include <set>
 #include <tuple>
 #include <type_traits>
 #include <vector>
+
+#include <cuda.h>
 
 #include "burr_internal.cuh"
 
@@ -392,17 +395,22 @@ constexpr size_t kOneBlock = 64ull << 20;
 constexpr int kNumEvents = kBandSets + 6;
 // Streams, events and a page-locked page that a build uses beside the caller's
 // stream.  Making them took about a third of a 1,000-key build, so they are kept
-// for the next build on the device: at most kKeptSets of them per process (a set
-// given back beyond that is destroyed), and those when the library is unloaded.
+// for the next build in the same context: at most kKeptSets of them per process (a
+// set given back beyond that is destroyed), and those when the library is
+// unloaded.  They belong to the context that they were made in, so a set is known
+// by that context's id, which no later context of the process has again (a device's
+// primary context made anew after cudaDeviceReset, or another context on the
+// device, gets sets of its own).
 // A set belongs to one build or query at a time.  Work still queued on its
 // streams when it is given back only comes before the next user's.
 struct StreamSet {
-    int dev = 0;
+    unsigned long long ctx = 0;            // id of its context; 0: not known (never kept)
     cudaStream_t side = nullptr, band2 = nullptr, copy = nullptr;
     cudaEvent_t ev[kNumEvents] = {};
     void *page = nullptr;                  // kPageBytes, for results read by the host
-    cudaError_t make() {
-        cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t make(unsigned long long context) {
+        ctx = context;
+        cudaError_t e = cudaSuccess;
         for (cudaStream_t *s : {&side, &band2, &copy})
             if (e == cudaSuccess) e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking);
         for (int i = 0; i < kNumEvents && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
@@ -417,37 +425,73 @@ struct StreamSet {
     }
     static constexpr size_t kPageBytes = 4096;
 };
+
+// Id of the calling thread's current context; 0 if there is none or the driver does not tell.
+unsigned long long current_context() {
+    struct Driver {
+        CUresult (*get)(CUcontext *) = nullptr;
+        CUresult (*id)(CUcontext, unsigned long long *) = nullptr;
+        Driver() {
+            cudaDriverEntryPointQueryResult q;
+            void *f = nullptr;
+            if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 4000, cudaEnableDefault, &q) == cudaSuccess &&
+                q == cudaDriverEntryPointSuccess)
+                get = (CUresult (*)(CUcontext *))f;
+            if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                q == cudaDriverEntryPointSuccess)
+                id = (CUresult (*)(CUcontext, unsigned long long *))f;
+        }
+    };
+    static const Driver d;
+    CUcontext c = nullptr;
+    unsigned long long id = 0;
+    if (!d.get || !d.id || d.get(&c) != CUDA_SUCCESS || !c || d.id(c, &id) != CUDA_SUCCESS) return 0;
+    return id;
+}
+
 constexpr size_t kKeptSets = 8;
 std::mutex g_sets_mu;
-struct KeptSets : std::vector<std::unique_ptr<StreamSet>> {   // not in use
+struct KeptSets {
+    std::unique_ptr<StreamSet> q[kKeptSets];   // not in use
     ~KeptSets() {
-        int dev;
-        if (cudaGetDevice(&dev) == cudaSuccess) return;       // (the members are destroyed)
-        for (auto &q : *this) q.release();                    // the runtime is gone, and they with it
+        // those of another context, or of one that is gone, end with it
+        const unsigned long long ctx = current_context();
+        for (auto &s : q)
+            if (s && s->ctx != ctx) s.release();
     }
 } g_sets;
 
 std::unique_ptr<StreamSet> take_streams(cudaError_t &e) {
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return nullptr;
-    {
-        std::lock_guard<std::mutex> lk(g_sets_mu);
-        for (auto &q : g_sets)
-            if (q->dev == dev) {
-                std::unique_ptr<StreamSet> s = std::move(q);
-                q = std::move(g_sets.back());
-                g_sets.pop_back();
-                return s;
-            }
+    unsigned long long ctx = current_context();
+    if (!ctx) {   // a thread's first call: its device's primary context, as any runtime call would make current
+        int dev = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaSetDevice(dev)) != cudaSuccess) return nullptr;
+        ctx = current_context();
     }
-    auto s = std::make_unique<StreamSet>();
-    e = s->make();
+    if (ctx) {
+        std::lock_guard<std::mutex> lk(g_sets_mu);
+        for (auto &q : g_sets.q)
+            if (q && q->ctx == ctx) return std::move(q);
+    }
+    std::unique_ptr<StreamSet> s(new (std::nothrow) StreamSet());
+    e = s ? s->make(ctx) : cudaErrorMemoryAllocation;
     return e == cudaSuccess ? std::move(s) : nullptr;
 }
 
 void give_streams(std::unique_ptr<StreamSet> s) {
+    if (!s->ctx) return;
     std::lock_guard<std::mutex> lk(g_sets_mu);
-    if (g_sets.size() < kKeptSets) g_sets.push_back(std::move(s));
+    std::unique_ptr<StreamSet> *at = nullptr;
+    for (auto &q : g_sets.q) {
+        if (!q) {
+            at = &q;
+            break;
+        }
+        if (q->ctx != s->ctx) at = &q;
+    }
+    if (!at) return;              // all of this context: s is destroyed
+    (void)at->release();          // (nothing, or another context's, which may be gone)
+    *at = std::move(s);
 }
 
 struct SideStream {
