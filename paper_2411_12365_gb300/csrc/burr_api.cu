@@ -939,7 +939,9 @@ struct BatchTables {
     std::vector<uint32_t> part_order;   // partitions by decreasing length (the band's launch order)
     std::vector<uint64_t> tile_lo;
     std::vector<uint32_t> who;   // active index -> structure index
-    uint32_t max_len = 0;        // buckets of the longest partition
+    uint32_t max_len = 0;        // buckets of the longest partition, at most (cuts may be searched)
+    std::vector<uint32_t> part_len;   // buckets of each partition before cuts are searched
+    uint32_t moved = 0;          // buckets that a searched cut moves by, at most
     bool fallback = false;
     uint64_t nbuckets = 0, ngroups = 0, nparts = 0, slots = 0, tw = 0, zw = 0, nkeys = 0;
 };
@@ -1013,20 +1015,21 @@ int batch_tables(const burr_params &p, const std::vector<uint32_t> &r, const std
     // sort it replaces: most partitions share a handful of lengths.)
     std::vector<uint32_t> len(T.nparts);
     uint32_t lmax = 0;
+    T.moved = p.cut_search != BURR_CUT_NONE && !fb ? (uint32_t)(Pl / p.bucket_slots) : 0u;
     for (uint32_t i = 0; i < T.sd.size(); ++i)
         for (uint64_t k = 0; k < T.sd[i].L.K; ++k) {
             const uint32_t x = (uint32_t)(part_bucket(T.sd[i].L, k + 1) - part_bucket(T.sd[i].L, k));
             len[T.sd[i].part_base + k] = x;
             lmax = std::max(lmax, x);
+            T.max_len = std::max(T.max_len, x + (T.sd[i].L.K > 1 ? T.moved : 0u));
         }
-    // (cut search moves a cut by less than a partition)
-    T.max_len = lmax + (p.cut_search != BURR_CUT_NONE && !fb ? (uint32_t)(Pl / p.bucket_slots) : 0u);
     T.fallback = fb;
     std::vector<uint32_t> at(lmax + 2, 0);
     for (const uint32_t x : len) ++at[lmax - x + 1];   // decreasing length
     for (uint32_t x = 1; x <= lmax + 1; ++x) at[x] += at[x - 1];
     T.part_order.resize(T.nparts);
     for (uint32_t j = 0; j < T.nparts; ++j) T.part_order[at[lmax - len[j]]++] = j;
+    T.part_len = std::move(len);
     return BURR_OK;
 }
 
@@ -1161,6 +1164,20 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         v.max_len = T.max_len;
         v.mode = p.threshold_mode;
         v.fallback = T.fallback;
+        if (const uint32_t seg_len = band_segment(v)) {
+            std::vector<uint32_t> table(T.nparts + 1);   // first segment of each partition, then the partition of each
+            for (uint32_t q = 0; q < T.nparts; ++q) {
+                const uint32_t j = T.part_order[q],
+                               len = T.part_len[j] + (T.sd[T.part_struct[j]].L.K > 1 ? T.moved : 0u);
+                table[q + 1] = table[q] + (len + seg_len - 1) / seg_len;
+                table.resize(T.nparts + 1 + table[q + 1], q);
+            }
+            uint32_t *d;
+            CK(upload(ar, table, &d, st), "upload segments");
+            v.nsegs = table[T.nparts];
+            v.seg_first = d;
+            v.seg_part = d + T.nparts + 1;
+        }
         const size_t need = band_scratch_bytes(LayerDesc(), &v);
         if (need > seg_bytes) {
             if (seg) ar.release(seg);

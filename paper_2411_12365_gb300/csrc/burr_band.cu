@@ -856,8 +856,11 @@ template <typename V>
 __global__ void __launch_bounds__(64, kFewCtas)
 k_band_seg(BandArgs<V> a, uint32_t nparts, uint32_t pass, bool last) {
     __shared__ BandSmem S;
-    const uint32_t gp = last ? blockIdx.x : blockIdx.x % nparts, i = last ? 0 : blockIdx.x / nparts;
-    const uint64_t base = (uint64_t)gp * a.nseg;      // the partition's first segment
+    // the partition, its first segment, and the place of this one in it
+    const bool table = a.bv.seg_first != nullptr;
+    const uint32_t gp = last ? blockIdx.x : (table ? a.bv.seg_part[blockIdx.x] : blockIdx.x % nparts);
+    const uint64_t base = table ? (uint64_t)a.bv.seg_first[gp] : (uint64_t)gp * a.nseg;
+    const uint32_t i = last ? 0 : (table ? blockIdx.x - (uint32_t)base : blockIdx.x / nparts);
     const uint64_t g = base + i;
     const uint32_t now = pass & 1u, then = now ^ 1u;
     // (a partition's first segment starts from true rows; what a segment behind a partition's end
@@ -899,11 +902,17 @@ k_band_seg(BandArgs<V> a, uint32_t nparts, uint32_t pass, bool last) {
 template <typename V>
 __global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t nparts) {
     __shared__ BandSmem S;
-    if (!load_ctx(S, a, blockIdx.x % nparts) || S.failed) return;
+    uint32_t gp = blockIdx.x % nparts, i = blockIdx.x / nparts;   // the partition and a word of its
+    if (a.bv.seg_first) {   // those of its segments, and one more: its buckets may start inside a word
+        const uint32_t per = a.seg / 32, words = a.bv.nsegs * per;
+        gp = blockIdx.x < words ? a.bv.seg_part[blockIdx.x / per] : blockIdx.x - words;
+        i = blockIdx.x < words ? blockIdx.x - a.bv.seg_first[gp] * per : (a.bv.seg_first[gp + 1] - a.bv.seg_first[gp]) * per;
+    }
+    if (!load_ctx(S, a, gp) || S.failed) return;
     const Ctx &x = S.x;
     const int lane = (int)(threadIdx.x & 31);
     const uint32_t warp = threadIdx.x >> 5;
-    const uint32_t w = (x.b0 >> 5) + blockIdx.x / nparts, b = w * 32u + (uint32_t)lane;
+    const uint32_t w = (x.b0 >> 5) + i, b = w * 32u + (uint32_t)lane;
     if (w * 32u >= x.b1) return;
     const uint32_t t = b >= x.b0 && b < x.b1 ? a.texact[x.bucket_base + b] : 0u;
     if (warp == 0 && x.L.mode != BURR_THRESH_1PLUS) {
@@ -940,9 +949,14 @@ __global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t npa
 constexpr uint64_t kSegCap = 2432, kSegMin = 32, kSegCapExact = 460, kSegMaxExact = 128;
 // Passes before the last one: enough for runs that meet after 190 buckets.
 inline uint32_t seg_passes(uint32_t seg) { return 1 + (190 + seg - 1) / seg; }
+// A layer's partitions have nearly the same length, and each has as many segments
+// in the launch's arrays as the longest.  Those of a batch may be one long and many
+// short ones, so a batched launch has a table of segments: their number is at most
+// partitions + buckets / segment length then, which kSegCap bounds (a product with
+// the longest partition's took 2 GB for one structure of 4*10^6 keys among 1,000 of 100).
 struct SegPlan {
     uint32_t seg = 0, nseg = 0;
-    uint64_t parts = 0, buckets = 0;
+    uint64_t parts = 0, buckets = 0, nsegs = 0;   // nsegs: of the launch
 };
 SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
     SegPlan p;
@@ -968,6 +982,7 @@ SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
     if (p.parts + total / seg > cap || seg * 2 > longest || (exact && seg > kSegMaxExact)) return p;
     p.seg = (uint32_t)seg;
     p.nseg = (uint32_t)((longest + seg - 1) / seg);
+    p.nsegs = bv ? bv->nsegs : p.parts * p.nseg;
     return p;
 }
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -1009,33 +1024,35 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
     q += align256(p.buckets * 8);
     for (int i = 0; i < 2; ++i) {
         a.state[i] = (Pivot *)q;
-        q += align256(p.parts * p.nseg * 64 * sizeof(Pivot));
+        q += align256(p.nsegs * 64 * sizeof(Pivot));
     }
     for (int i = 0; i < 2; ++i) {
         a.moved[i] = (uint32_t *)q;
-        q += align256(p.parts * p.nseg * 4);
+        q += align256(p.nsegs * 4);
     }
     if (!a.texact) a.texact = (uint8_t *)q;
     const uint32_t parts = (uint32_t)p.parts;
     const bool fallback = bv ? bv->fallback : L.fallback != 0;
     cudaError_t e;
     if ((e = prefer_shared(k_band_seg<V>)) != cudaSuccess || (e = prefer_shared(k_band_finish<V>)) != cudaSuccess) return e;
-    const uint32_t passes = seg_passes(p.seg);
-    for (uint32_t pass = 0; pass < passes; ++pass) k_band_seg<V><<<parts * p.nseg, 64, 0, st>>>(a, parts, pass, false);
+    const uint32_t passes = seg_passes(p.seg), segs = (uint32_t)p.nsegs;
+    for (uint32_t pass = 0; pass < passes; ++pass) k_band_seg<V><<<segs, 64, 0, st>>>(a, parts, pass, false);
     k_band_seg<V><<<parts, 64, 0, st>>>(a, parts, passes, true);
-    // a partition's buckets may start inside a code word
-    if (!fallback) k_band_finish<V><<<parts * (p.nseg * p.seg / 32 + 2), 128, 0, st>>>(a, parts);
+    // (a partition's buckets may start inside a code word)
+    if (!fallback) k_band_finish<V><<<segs * (p.seg / 32) + parts * (bv ? 1u : 2u), 128, 0, st>>>(a, parts);
     return cudaGetLastError();
 }
 
 }  // namespace
 
+uint32_t band_segment(const BatchView &bv) { return bv.nparts ? seg_plan(LayerDesc(), &bv).seg : 0u; }
+
 size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv) {
     if (bv ? bv->nparts == 0 : part_end(L) <= L.part_lo) return 0;
     const SegPlan p = seg_plan(L, bv);
     if (!p.seg) return 0;
-    return 256 + align256(p.buckets * 8) + align256(p.buckets) + 2 * align256(p.parts * p.nseg * 64 * sizeof(Pivot)) +
-           2 * align256(p.parts * p.nseg * 4);
+    return 256 + align256(p.buckets * 8) + align256(p.buckets) + 2 * align256(p.nsegs * 64 * sizeof(Pivot)) +
+           2 * align256(p.nsegs * 4);
 }
 
 uint32_t band_kernel_count(const LayerDesc &L, const BatchView *bv) {

@@ -159,6 +159,10 @@ struct BatchView {
     uint32_t max_len = 0;                   // buckets of the longest partition
     uint32_t mode = 0;                      // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
     bool fallback = false;                  // a base case
+    // segments of the launch's partitions (band_segment): first segment of each partition in launch
+    // order, [nparts] = nsegs, and the partition of each segment
+    uint32_t nsegs = 0;
+    const uint32_t *seg_first = nullptr, *seg_part = nullptr;
 };
 
 // Scratch bytes of launch_sort for n keys in a layer of m slots.
@@ -198,6 +202,9 @@ cudaError_t launch_sort_slack_end(const LayerDesc &L, uint32_t vbytes, uint64_t 
 // 0 (launches of few partitions, banded in segments); without it every
 // partition is banded from end to end by one CTA.
 size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv = nullptr);
+// Buckets per segment of a batched launch, 0 if it bands whole partitions.  Otherwise the view
+// needs its table of segments before band_scratch_bytes and the launch.
+uint32_t band_segment(const BatchView &bv);
 // Kernels that launch enqueues with its scratch.
 uint32_t band_kernel_count(const LayerDesc &L, const BatchView *bv = nullptr);
 cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *keys, const void *vals,
