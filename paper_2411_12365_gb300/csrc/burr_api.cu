@@ -1380,7 +1380,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         CK(launch_band(none, vb, (const uint64_t *)sk, sv, (const uint32_t *)bst, (uint64_t *)cg, yg, nullptr, nullptr,
                        (uint64_t *)bk[wfb], bv2[wfb], bcount, err, st, &v, seg), "band");
         CK(launch_backsub(none, vb, (uint64_t *)cg, yg, z, st, &v), "backsub");
-        for (auto *h : hs) h->launches += 5 + backsub_kernel_count(none, &v);
+        for (auto *h : hs) h->launches += 4 + band_kernel_count(none, &v) + backsub_kernel_count(none, &v);
         std::vector<uint32_t> f(left.size());
         uint32_t e = 0;
         CK(cudaMemcpyAsync(f.data(), ffail, f.size() * 4, cudaMemcpyDeviceToHost, st), "read flags");

@@ -76,3 +76,14 @@ def test_mixed_lengths_equal_single_builds(r, kw, mode):
         a, b = int(offs[s]), int(offs[s + 1])
         got, want = h.export(), burr.build(keys[a:b], vals[a:b], r, threshold_mode=mode, **kw).export()
         assert got == want, (s, describe_difference(got, want))
+
+
+def test_launches_of_a_segmented_base_case_are_counted():
+    # 32-bucket segments: 1 + ceil(190 / 32) passes and the last one, instead of one launch
+    def launches(n):
+        keys, vals, offs = _inputs([n], 8)
+        st = burr.build_batch(keys, vals, offs, [8], layers=0)[0].stats()
+        assert st["fallback_attempt"] == 0
+        return st["kernel_launches"]
+
+    assert launches(200_000) - launches(5_000) == 1 + -(-190 // 32) + 1 - 1
