@@ -942,6 +942,7 @@ struct BatchTables {
     uint32_t max_len = 0;        // buckets of the longest partition, at most (cuts may be searched)
     std::vector<uint32_t> part_len;   // buckets of each partition before cuts are searched
     uint32_t moved = 0;          // buckets that a searched cut moves by, at most
+    uint64_t max_slots = 0;      // slots of the longest partition before cuts are searched
     bool fallback = false;
     uint64_t nbuckets = 0, ngroups = 0, nparts = 0, slots = 0, tw = 0, zw = 0, nkeys = 0;
 };
@@ -1023,6 +1024,7 @@ int batch_tables(const burr_params &p, const std::vector<uint32_t> &r, const std
             lmax = std::max(lmax, x);
             T.max_len = std::max(T.max_len, x + (T.sd[i].L.K > 1 ? T.moved : 0u));
         }
+    T.max_slots = (uint64_t)lmax * p.bucket_slots;
     T.fallback = fb;
     std::vector<uint32_t> at(lmax + 2, 0);
     for (const uint32_t x : len) ++at[lmax - x + 1];   // decreasing length
@@ -1162,6 +1164,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         v.nkeys = T.nkeys;
         v.slots = T.slots;
         v.max_len = T.max_len;
+        v.max_slots = T.max_slots;
         v.mode = p.threshold_mode;
         v.fallback = T.fallback;
         if (const uint32_t seg_len = band_segment(v)) {

@@ -367,7 +367,7 @@ BsPlan bs_plan(const LayerDesc &L, const BatchView *bv) {
     if (bv) {
         p.parts = bv->nparts;
         p.slots = bv->slots;                // 0: only some of the layer's partitions
-        longest = (uint64_t)bv->max_len * 2;
+        longest = bv->max_slots / 64;
     } else {
         if (part_end(L) <= L.part_lo) return p;
         p.parts = part_end(L) - L.part_lo;

@@ -156,7 +156,8 @@ struct BatchView {
     uint64_t nbuckets = 0;                  // global buckets
     uint64_t nkeys = 0;                     // keys of the layer (sum over structures)
     uint64_t slots = 0;                     // slots of the layer (sum over structures; 0: only some of its partitions)
-    uint32_t max_len = 0;                   // buckets of the longest partition
+    uint32_t max_len = 0;                   // buckets of the longest partition, at most (cuts may be searched)
+    uint64_t max_slots = 0;                 // slots of the longest partition before cuts are searched
     uint32_t mode = 0;                      // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
     bool fallback = false;                  // a base case
     // segments of the launch's partitions (band_segment): first segment of each partition in launch

@@ -87,3 +87,17 @@ def test_launches_of_a_segmented_base_case_are_counted():
         return st["kernel_launches"]
 
     assert launches(200_000) - launches(5_000) == 1 + -(-190 // 32) + 1 - 1
+
+
+def test_searched_cuts_choose_the_back_substitution_of_plain_ones():
+    # partitions of 32 to 47 blocks (the last ones): past the size up to which blocks are reduced first
+    # (50,000 slots per block of the longest), but within that of partitions 32 blocks longer
+    keys, vals, offs = _inputs([1_500_000, 1_500_000], 8)
+
+    def stats(cut):
+        st = burr.build_batch(keys, vals, offs, [8, 8], cut_search=cut, layers=1, partition_slots=2_048,
+                              min_partition_slots=2_048)[0].stats()
+        assert st["fallback_attempt"] == 0
+        return st["kernel_launches"]
+
+    assert stats(burr.CUT_DIFF) - stats(burr.CUT_NONE) == 1   # the search
