@@ -318,6 +318,7 @@ LayerDesc make_desc(const burr_params &p, uint32_t r, uint64_t n, uint64_t m, ui
     L.forced_code = (uint32_t)forced_code(p.levels);
     L.vmask = r >= 32 ? 0xffffffffu : ((1u << r) - 1u);
     L.mode = p.threshold_mode;
+    L.load = (float)(fallback ? 1.0 / (1.0 + p.fallback_slack) : p.load_factor);
     L.window = (p.flags & BURR_FLAG_TEST_WINDOW) ? kTestWindow : 0u;
     L.test_slack = (p.flags & BURR_FLAG_TEST_SLACK) ? 1u : 0u;
     return L;
@@ -1167,6 +1168,7 @@ int build_batch_impl(const uint64_t *keys, const void *values, const std::vector
         v.max_slots = T.max_slots;
         v.mode = p.threshold_mode;
         v.fallback = T.fallback;
+        v.load = T.sd[0].L.load;
         if (const uint32_t seg_len = band_segment(v)) {
             std::vector<uint32_t> table(T.nparts + 1);   // first segment of each partition, then the partition of each
             for (uint32_t q = 0; q < T.nparts; ++q) {

@@ -47,6 +47,7 @@
 //   10^8 keys (1504 partitions)                   8.33 -> 6.2;  1+-bit 16.3 -> 9.0
 //   10^9 keys (15034 partitions)                  63.7 -> 47.4
 #include <algorithm>
+#include <cmath>
 
 #include "burr_internal.cuh"
 
@@ -830,6 +831,8 @@ k_band(BandArgs<V> a) {
     run_buckets<V, false>(S, a, R, (int)(threadIdx.x & 31));
 }
 
+#include "burr_band_stream.cuh"
+
 // Few partitions: each is banded in segments of a.seg buckets at the same time.
 //
 // A bucket's result depends on the buckets before it only through the rows
@@ -954,13 +957,35 @@ inline uint32_t seg_passes(uint32_t seg) { return 1 + (190 + seg - 1) / seg; }
 // short ones, so a batched launch has a table of segments: their number is at most
 // partitions + buckets / segment length then, which kSegCap bounds (a product with
 // the longest partition's took 2 GB for one structure of 4*10^6 keys among 1,000 of 100).
-struct SegPlan {
+struct BandPlan {
     uint32_t seg = 0, nseg = 0;
     uint64_t parts = 0, buckets = 0, nsegs = 0;   // nsegs: of the launch
+    bool sparse = false, stream = false;          // the stream beats the sweep of whole partitions, and segments too
 };
-SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
-    SegPlan p;
-    uint64_t total, longest;
+
+// Which launches of sparse layers are streamed (burr_band_stream.cuh): estimates of
+// a launch in us from the chain over its longest partition and the chip's
+// throughput, in buckets of 128 slots.  Measured, r = 2, 2-bit thresholds, at loads
+// 0.25 / 0.5 / 0.7 / 0.85 / 0.9 / 0.95:
+//   stream   one warp alone 2.5 / 3.5 / 4.7 / 6.1 / 7.1 / 8.8 us per bucket, the chip full 1.4 / 1.9 / 2.6 / 3.8 / 4.4 / 5.7 ns
+//   sweep    6.6 us, 5.5 to 5.9 ns; in segments 8.5 us per bucket of one segment, at any of these loads
+// so the line lies at 0.87 (few partitions) to 0.95 (many).  Layer-0 band, ms, sweep / stream:
+//   6*10^7 keys, partitions of 4,096 slots   - , 5.15 / 1.80, 3.76 / 1.74, 3.16 / 2.10, 3.01 / 2.29, 2.90 / 2.80
+//   6*10^7 keys, default (964 to 1,832)      - , 7.24 / 2.17, 5.54 / 2.64, 4.32 / 3.37, 4.32 / 3.91, 4.38 / 4.93
+//   2*10^7 keys, default, from 0.5 on in segments   5.43 / 1.38, 2.82 / 1.79, 1.51 / 2.24, 1.48 / 3.05, 1.52 / 3.55, 1.62 / 4.53
+// Above kStreamLoad nothing is streamed: there many buckets are dependent.
+constexpr double kStreamLoad = 1.0;
+inline double band_us(double bucket_us, double longest, double bucket_ns, double buckets) {
+    return std::hypot(bucket_us * longest, bucket_ns * 1e-3 * buckets);
+}
+inline double stream_us(double longest, double buckets, double load) {
+    const double x = 1.0 / (1.1 - load);
+    return band_us(1.1 + 1.27 * x, longest, 0.44 + 0.81 * x, buckets);
+}
+
+BandPlan band_plan(const LayerDesc &L, const BatchView *bv) {
+    BandPlan p;
+    uint64_t total, longest, moved = 0;   // moved: buckets by which searched cuts may lengthen a partition
     if (bv) {
         p.parts = bv->nparts;
         total = bv->nbuckets;
@@ -969,7 +994,8 @@ SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
     } else {
         p.parts = part_end(L) - L.part_lo;
         // partitions of P slots, the last one with the remainder; searched cuts move by less than P
-        longest = L.K <= 1 ? L.nb : std::max<uint64_t>(L.P / L.B, L.nb - (L.K - 1) * (L.P / L.B)) + (L.cuts ? L.P / L.B : 0);
+        moved = L.K > 1 && L.cuts ? L.P / L.B : 0;
+        longest = L.K <= 1 ? L.nb : std::max<uint64_t>(L.P / L.B, L.nb - (L.K - 1) * (L.P / L.B)) + moved;
         total = std::min<uint64_t>(L.nb, p.parts * longest);
         p.buckets = L.nb;
     }
@@ -979,7 +1005,16 @@ SegPlan seg_plan(const LayerDesc &L, const BatchView *bv) {
     const uint64_t cap = exact ? kSegCapExact : kSegCap;
     uint64_t seg = kSegMin;
     while (p.parts + total / seg > cap && seg * 2 <= longest) seg *= 2;
-    if (p.parts + total / seg > cap || seg * 2 > longest || (exact && seg > kSegMaxExact)) return p;
+    if (p.parts + total / seg > cap || seg * 2 > longest || (exact && seg > kSegMaxExact)) seg = 0;
+    const double load = bv ? bv->load : L.load;
+    if (load <= kStreamLoad) {
+        const double len = (bv ? (double)bv->max_slots : (double)(longest - moved) * L.B) / 128.0;
+        const double all = bv ? (double)total : (double)total * L.B / 128.0;
+        const double us = stream_us(len, all, load);
+        p.sparse = us < band_us(6.6, len, 5.7, all + 0.5 * (double)p.parts);   // (64 slots past each end)
+        p.stream = seg ? us < band_us(8.5, (double)seg, 6.6, all) : p.sparse;
+    }
+    if (seg == 0 || p.stream) return p;
     p.seg = (uint32_t)seg;
     p.nseg = (uint32_t)((longest + seg - 1) / seg);
     p.nsegs = bv ? bv->nsegs : p.parts * p.nseg;
@@ -1005,7 +1040,17 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
     a.bvals = bvals;
     a.bcount = bcount;
     a.err = err;
-    const SegPlan p = seg_plan(L, bv);
+    const BandPlan p = band_plan(L, bv);
+    if (p.stream || (p.sparse && !scratch)) {
+        const bool exact = (bv ? bv->mode : L.mode) == BURR_THRESH_1PLUS;
+        auto go = [&](auto *kernel) -> cudaError_t {
+            const cudaError_t e = prefer_shared(kernel);
+            if (e != cudaSuccess) return e;
+            kernel<<<(unsigned)((p.parts + kStreamWarps - 1) / kStreamWarps), 32 * kStreamWarps, 0, st>>>(a);
+            return cudaGetLastError();
+        };
+        return exact ? go(k_band_stream<V, true>) : go(k_band_stream<V, false>);
+    }
     if (!scratch || !p.seg) {
         auto go = [&](auto *kernel) -> cudaError_t {
             const cudaError_t e = prefer_shared(kernel);
@@ -1045,11 +1090,11 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
 
 }  // namespace
 
-uint32_t band_segment(const BatchView &bv) { return bv.nparts ? seg_plan(LayerDesc(), &bv).seg : 0u; }
+uint32_t band_segment(const BatchView &bv) { return bv.nparts ? band_plan(LayerDesc(), &bv).seg : 0u; }
 
 size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv) {
     if (bv ? bv->nparts == 0 : part_end(L) <= L.part_lo) return 0;
-    const SegPlan p = seg_plan(L, bv);
+    const BandPlan p = band_plan(L, bv);
     if (!p.seg) return 0;
     return 256 + align256(p.buckets * 8) + align256(p.buckets) + 2 * align256(p.nsegs * 64 * sizeof(Pivot)) +
            2 * align256(p.nsegs * 4);
@@ -1057,7 +1102,7 @@ size_t band_scratch_bytes(const LayerDesc &L, const BatchView *bv) {
 
 uint32_t band_kernel_count(const LayerDesc &L, const BatchView *bv) {
     if (band_scratch_bytes(L, bv) == 0) return 1u;
-    return seg_passes(seg_plan(L, bv).seg) + ((bv ? bv->fallback : L.fallback != 0) ? 1u : 2u);
+    return seg_passes(band_plan(L, bv).seg) + ((bv ? bv->fallback : L.fallback != 0) ? 1u : 2u);
 }
 
 cudaError_t launch_band(const LayerDesc &L, uint32_t vbytes, const uint64_t *keys, const void *vals,

@@ -96,6 +96,7 @@ struct LayerDesc {
     uint32_t forced_code;
     uint32_t vmask;      // (1 << r) - 1
     uint32_t mode;       // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
+    float load;          // keys per slot that the layer is sized for
     uint32_t window;     // testing: live rows this many slots past their bucket's start are an error (0 = no check)
     uint32_t test_slack; // 1: the fixed-capacity sort bins get half their expected size (testing the exact redo)
     uint32_t part_lo;    // band and back-substitution launches cover partitions [part_lo, part_hi)
@@ -160,6 +161,7 @@ struct BatchView {
     uint64_t max_slots = 0;                 // slots of the longest partition before cuts are searched
     uint32_t mode = 0;                      // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
     bool fallback = false;                  // a base case
+    float load = 0;                         // keys per slot that the structures' layers are sized for
     // segments of the launch's partitions (band_segment): first segment of each partition in launch
     // order, [nparts] = nsegs, and the partition of each segment
     uint32_t nsegs = 0;
