@@ -1555,6 +1555,7 @@ int burr_query(const burr_handle *h, const uint64_t *keys, void *out, uint64_t n
     Q.B = h->p.bucket_slots;
     Q.layers = h->p.layers;
     Q.mode = h->p.threshold_mode;
+    Q.load = (float)h->p.load_factor;
     for (int i = 0; i < 4; ++i) Q.levels[i] = h->p.levels[i];
     for (uint32_t l = 0; l <= h->p.layers; ++l) {
         Q.m[l] = h->L[l].m;

@@ -241,6 +241,7 @@ struct QueryDesc {
     uint32_t layers;          // bumping layers
     uint32_t levels[4];
     uint32_t mode;            // BURR_THRESH_2BIT or BURR_THRESH_1PLUS
+    float load;               // keys per slot that the bumping layers are sized for
     uint64_t m[BURR_MAX_LAYERS + 1];
     uint64_t sigma[BURR_MAX_LAYERS + 1];
     const uint64_t *thresh[BURR_MAX_LAYERS];   // 2-bit codes

@@ -77,12 +77,6 @@ struct Window {
 
 template <int R, bool kKeep>
 __device__ __forceinline__ void load_window(const uint64_t *__restrict__ z, uint32_t s, Window<R> &w) {
-    if (R == 1) {   // two words: narrow reads of the same sector are cheaper than the move
-        const bool two = (s & 63u) != 0u;
-        w.w[0] = __ldg(z + (s >> 6));
-        w.w[1] = two ? __ldg(z + (s >> 6) + 1) : 0ull;
-        return;
-    }
     const uint64_t at = (uint64_t)(s >> 6) * R;
     const uint32_t shift = (uint32_t)at & 3u & (uint32_t)Window<R>::kMaxShift;
     const uint32_t need = shift + ((s & 63u) ? 2u * R : (uint32_t)R);
@@ -102,12 +96,12 @@ __device__ __forceinline__ void load_window(const uint64_t *__restrict__ z, uint
     }
 }
 
-// The same words by loads of 16 bytes (R even) or 8, which need not be moved.
-template <int R>
+// The same words by loads of 16 bytes (kPairs, R even) or 8, which need not be moved.
+template <int R, bool kPairs>
 __device__ __forceinline__ void load_narrow(const uint64_t *__restrict__ z, uint32_t s, Window<R> &w) {
     const uint64_t *p = z + (uint64_t)(s >> 6) * R;
     const bool two = (s & 63u) != 0u;
-    if (R % 2 == 0) {
+    if (kPairs) {
         const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(p);
 #pragma unroll
         for (int k = 0; k < R; k += 2) {
@@ -180,6 +174,26 @@ __device__ __forceinline__ uint32_t threshold_of(const QueryDesc &Q, uint32_t l,
     return Q.levels[(uint32_t)(__ldg(Q.thresh[l] + (b >> 5)) >> (2 * (b & 31))) & 3u];
 }
 
+// The same in either mode, the flag words of a block one by one: less work where
+// there is one flag word, or for keys that go through several layers.
+__device__ __forceinline__ uint32_t threshold_any(const QueryDesc &Q, uint32_t l, uint32_t b) {
+    if (Q.mode != BURR_THRESH_1PLUS) return threshold_of<false>(Q, l, b);
+    const uint64_t *fl = Q.flags[l];
+    const uint64_t w = __ldg(fl + (b >> 6));
+    if (!((w >> (b & 63u)) & 1ull)) return 0;
+    uint32_t rank = __ldg(Q.dir[l] + (b >> 9));
+    for (uint32_t k = (b >> 9) << 3; k < (b >> 6); ++k) rank += (uint32_t)__popcll(__ldg(fl + k));
+    rank += (uint32_t)__popcll(w & ((1ull << (b & 63u)) - 1ull));
+    return __ldg(Q.tbytes[l] + rank);
+}
+
+// How a kernel finds thresholds.
+enum { kCodes = 0, kFlags = 1, kEither = 2 };   // of 2-bit codes, of flags, threshold_any
+template <int kHow>
+__device__ __forceinline__ uint32_t threshold(const QueryDesc &Q, uint32_t l, uint32_t b) {
+    return kHow == kEither ? threshold_any(Q, l, b) : threshold_of<kHow == kFlags>(Q, l, b);
+}
+
 // Query kernel for a value width R known at compile time: the table window
 // of a layer is loaded together with its threshold (values of up to 16 bits),
 // and the thread's next key is read while this key's table reads are in flight.
@@ -187,9 +201,10 @@ __device__ __forceinline__ uint32_t threshold_of(const QueryDesc &Q, uint32_t l,
 // gave 70.7 ms against 72.5 at 10^9 keys (r = 8) but 4.69 against 4.20 and 0.89
 // against 0.79 at 10^8 (r = 16, r = 1).
 //
-// kLoad: how the window is read (see query_r).
-enum { kWide = 0, kWideKeep = 1, kNarrow = 2 };   // 32-byte loads, kept in L1 or not; 16 or 8 bytes
-template <typename V, int R, int kLoad, bool kExact>
+// kLoad: how the window is read (see query_r): by 32-byte loads, kept in L1 or not,
+// by loads of 16 or 8 bytes after the threshold, or by 8-byte ones before it.
+enum { kWide = 0, kWideKeep = 1, kNarrow = 2, kWords = 3 };
+template <typename V, int R, int kLoad, int kHow>
 __global__ void __launch_bounds__(kQThreads)
 k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -207,13 +222,14 @@ k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, u
             const uint32_t s = (uint32_t)__umul64hi(h, m - kW + 1);
             if constexpr (R <= 16) {
                 Window<R> w;
-                if (kLoad != kNarrow) load_window<R, kLoad == kWideKeep>(Q.z[l], s, w);
-                if (l < Q.layers && (s & (Q.B - 1)) < threshold_of<kExact>(Q, l, s >> log2B)) continue;   // bumped: next layer
+                if (kLoad == kWords) load_narrow<R, false>(Q.z[l], s, w);
+                else if (kLoad != kNarrow) load_window<R, kLoad == kWideKeep>(Q.z[l], s, w);
+                if (l < Q.layers && (s & (Q.B - 1)) < threshold<kHow>(Q, l, s >> log2B)) continue;   // bumped: next layer
                 // (read before the threshold is known they are slower: r = 7 in 100 KB 77 against 71 us, r = 15 167 / 144)
-                if (kLoad == kNarrow) load_narrow<R>(Q.z[l], s, w);
+                if (kLoad == kNarrow) load_narrow<R, R % 2 == 0>(Q.z[l], s, w);
                 v = eval_loaded<R>(w, s, mix64(h + Q.sigma[l]) | 1ull);
             } else {
-                if (l < Q.layers && (s & (Q.B - 1)) < threshold_of<kExact>(Q, l, s >> log2B)) continue;
+                if (l < Q.layers && (s & (Q.B - 1)) < threshold<kHow>(Q, l, s >> log2B)) continue;
                 v = eval_planes<R, kLoad == kWideKeep>(Q.z[l], s, mix64(h + Q.sigma[l]) | 1ull);
             }
             break;
@@ -296,9 +312,9 @@ k_query_group(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ ou
     }
 }
 
-// kCodes: 2-bit thresholds only.  The other instance takes either mode: with the
-// mode fixed to 1+-bit it is slower (r = 3, 4*10^6 queries of 7 KB: 70 us against 54).
-template <typename V, bool kCodes>
+// Any width, plane by plane.  (kFlags with the mode fixed is slower: r = 3, 4*10^6
+// queries of 7 KB 70 us against 54.)
+template <typename V, int kHow>
 __global__ void __launch_bounds__(kQThreads)
 k_query(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uint64_t n) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -314,8 +330,7 @@ k_query(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, uin
             const uint32_t s = (uint32_t)__umul64hi(h, m - kW + 1);
             const uint32_t b = s >> log2B;
             const uint32_t off = s & (Q.B - 1);
-            const uint32_t t = !kCodes && Q.mode == BURR_THRESH_1PLUS ? threshold_of<true>(Q, l, b)
-                                                                      : threshold_of<false>(Q, l, b);
+            const uint32_t t = kHow == kFlags && Q.mode != BURR_THRESH_1PLUS ? threshold<kCodes>(Q, l, b) : threshold<kHow>(Q, l, b);
             if (off < t) continue;                             // bumped: next layer
             v = eval_window(Q.z[l], Q.r, s, mix64(h + Q.sigma[l]) | 1ull);
             break;
@@ -345,62 +360,107 @@ __global__ void k_hash(const uint64_t *__restrict__ keys, uint64_t n, uint64_t s
 
 namespace {
 
-// The kernel of width Q.r, if there is one for its table's size; false otherwise,
-// also for wider values of which the planes don't come in fours.
+// The kernel of width Q.r, if there is one for the case; false: any width's kernel
+// (launch_query), which reads plane by plane.  Times in us for 4*10^6 queries, 2-bit
+// thresholds, unless said.
 //
-// Times in us for 4*10^6 queries, 2-bit thresholds unless said.  A table that
-// mostly stays in L1 or is met again there is read through it: groups up to
-// 128 KB (r = 8, 2 KB 62 against 393 without: few lines, all of them in
-// L2's way; 20 KB 55 / 104; r = 16, 200 KB 91 / 95, 800 KB 100 / 95), single keys up to 1 MB.
-// Below 8 KB groups only add work (r = 8: 62, one lane per key 56).
-// Widths that are no multiple of 4 pay for moving a window read by wide loads
-// (odd ones most).  Against narrow loads / any width's kernel, which reads plane
-// by plane in a loop, wide loads take:
+// Groups of lanes (r = 8 from 8 KB on, 16, 32; both sides at k_query_group; r = 8 in 2 KB 62, one lane per
+// key 56) exchange results, which few keys don't pay for: r = 8 in 50 KB / 1 MB, 10,007 keys 3.4 / 4.1, one
+// lane per key 3.2 / 3.6; 10^5 keys 4.4 / 4.8 and 5.0 / 5.3; r = 16, 20 keys 2.5 / 3.3 and 2.1 / 2.7.
+//
+// Kept in L1, where a table mostly fits it: groups up to 128 KB (kept / not: r = 8, 2 KB 62 / 393,
+// 20 KB 55 / 104; r = 16, 200 KB 91 / 95, 800 KB 100 / 95), single keys up to 1 MB.
+//
+// Widths that are no multiple of 4 pay for moving a window read by wide loads (odd ones most).
+// Wide loads / narrow ones:
 //   r = 2    20 KB..5 MB  39..40 / 34..36;   1+-bit 60..65 / 52..56
-//   r = 3    7 KB 48 / 36;  375 KB 52 / 50 (general 48);  1.5 MB 52 / 53;  7 MB 52 / 54
-//   r = 5    60 KB 64 / 52;  250 KB 66 (general 60);  625 KB 68 / 76 (general 70)
+//   r = 3    7 KB 48 / 36;  375 KB 52 / 50 (any width's 48);  1.5 MB 52 / 53;  7 MB 52 / 54
+//   r = 5    60 KB 64 / 52;  250 KB 66 (any width's 60);  625 KB 68 / 76 (any width's 70)
 //   r = 6    75 KB 57 / 46;  750 KB 64 / 64;  3 MB 64 / 67
 //   r = 10, 14   125, 175 KB 85, 109 / 60, 82;  1.3, 1.8 MB 97, 127 / 99, 141
 //   r = 13, 15   160, 190 KB 134, 157 / 126, 144;  1.6, 1.9 MB 152, 177 / 167, 199
-// and with 1+-bit thresholds, whose loads take the registers, even widths are best
-// narrow (r = 6, 10, 14 in 12 to 35 MB: 101, 175, 195 / 83, 124, 162), odd ones up to
-// 11 in the general kernel (r = 5 in 625 KB: 99 / 98 / 81), 13 and 15 narrow (1.6, 1.9 MB:
-// 204, 220 / 196, 226).
+// and with 1+-bit thresholds, whose loads take the registers, even widths are best narrow (r = 6, 10, 14 in
+// 12 to 35 MB: 101, 175, 195 / 83, 124, 162), odd ones up to 11 in any width's kernel (r = 5 in 625 KB: 99 / 98 / 81),
+// 13 and 15 narrow (1.6, 1.9 MB: 204, 220 / 196, 226).  With one flag word (a few thousand keys) r = 1 and 8 look
+// the words up one by one (r = 8, 10^6 queries of 3,000 keys 19.8 / 21.8).
+//
+// These lines hold near the default load of 1.015.  Far from it other keys are met in other layers (at 1.3 a
+// quarter are bumped and the wide loads of their windows are wasted: r = 15 in 560 KB takes 1.46 times as long as
+// plane by plane; at 0.8 hardly a bucket is flagged).  There, and for tables off 32-byte boundaries (of a
+// caller's allocator), the widths that lost keep to kernels of either mode.  Over 1,824 combinations of width,
+// mode and sizes at each of the loads 0.8, 0.97, 1.05, 1.1, 1.3, by the lines alone 80, 27, 30, 87, 223 are more
+// than 4% slower than plane by plane (r = 1, 8, 16: than one lane per key), with the exception 8, -, 7, 12, 7;
+// at 1.0, 1.015, 1.03 6, 6, 8 are.
+inline bool usual_load(const QueryDesc &Q) { return Q.load >= 0.99f && Q.load <= 1.04f; }
+constexpr uint64_t kGroupKeys = 1 << 15, kGroupKeys16 = 256;
 template <int R>
-bool query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
+bool query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, bool aligned, cudaStream_t st) {
     using V = std::conditional_t<(R <= 8), uint8_t, std::conditional_t<(R <= 16), uint16_t, uint32_t>>;
     const uint64_t kb = (Q.m[0] / 64) * R * 8 >> 10;   // layer 0 holds nearly all of the table
-    const bool exact = Q.mode == BURR_THRESH_1PLUS;
+    const bool exact = Q.mode == BURR_THRESH_1PLUS, other = !usual_load(Q);
+    const bool one_word = exact && Q.m[0] <= 64ull * Q.B;   // of flags
     auto go = [&](auto *kernel) {
         kernel<<<grid, kQThreads, 0, st>>>(Q, keys, (V *)out, n);
         return true;
     };
-    if constexpr (R == 8 || R == 16 || R == 32) {
-        // (without bumping layers there is no layer 0 with thresholds)
-        if (Q.layers > 0 && Q.m[0] != 0 && (R != 8 || kb >= 8)) {
+    // without bumping layers there is no layer 0 with thresholds, in either mode
+    const bool layers = Q.layers > 0 && Q.m[0] != 0;
+    if constexpr (R == 1) {   // two words: narrow reads of the same sector are cheaper than the move
+        if (one_word || other) return go(k_query_r<V, 1, kWords, kEither>);
+        return exact ? go(k_query_r<V, 1, kWords, kFlags>) : go(k_query_r<V, 1, kWords, kCodes>);
+    } else if constexpr (R == 8 || R == 16 || R == 32) {
+        auto group = [&]() {
             if (kb < 128) return exact ? go(k_query_group<V, R, true, true>) : go(k_query_group<V, R, true, false>);
             return exact ? go(k_query_group<V, R, false, true>) : go(k_query_group<V, R, false, false>);
+        };
+        if (!aligned) {
+            // (4*10^6 keys: r = 8 151 us, plane by plane 147; r = 16 452, 427; 1,000 keys: 3.1 / 4.4, 4.3 / 7.3)
+            if constexpr (R != 32) {
+                if (n < kGroupKeys) return go(k_query_r<V, R, kWords, kEither>);
+            }
+            return false;
         }
-    }
-    if constexpr (R % 4 != 0 && R != 1) {
-        if (exact) return R % 2 == 0 || R >= 13 ? go(k_query_r<V, R, kNarrow, true>) : false;
-        constexpr uint64_t kNarrowKb = R == 2 ? ~0ull : R % 2 == 0 ? 512 : R >= 7 ? 256 : 64;
-        constexpr uint64_t kGeneralKb = R == 3 ? 1536 : R == 5 ? 512 : 0;
-        if (kb < kNarrowKb) return go(k_query_r<V, R, kNarrow, false>);
-        if constexpr (kGeneralKb != 0) {
-            if (kb < kGeneralKb) return false;
+        if (!layers) return kb < 1024 ? go(k_query_r<V, R, kWideKeep, kCodes>) : go(k_query_r<V, R, kWide, kCodes>);
+        if constexpr (R == 8) {
+            if (kb >= 8 && (exact || n >= kGroupKeys)) return group();
+            if (one_word || other) return go(k_query_r<V, R, kWideKeep, kEither>);
+            return exact ? go(k_query_r<V, R, kWideKeep, kFlags>) : go(k_query_r<V, R, kWideKeep, kCodes>);
+        } else {
+            if constexpr (R == 16) {
+                if (n < kGroupKeys16 || (other && kb < 16)) return go(k_query_r<V, R, kWideKeep, kEither>);
+            }
+            return group();
         }
-        return kb < 1024 ? go(k_query_r<V, R, kWideKeep, false>) : go(k_query_r<V, R, kWide, false>);
+    } else if constexpr (R % 4 != 0) {
+        if (!aligned || (other && R % 2 != 0)) return false;
+        if (exact) {
+            if constexpr (R % 2 == 0 || R >= 13) return go(k_query_r<V, R, kNarrow, kFlags>);
+            return false;
+        }
+        if constexpr (R == 2) {
+            return go(k_query_r<V, R, kNarrow, kCodes>);
+        } else {
+            constexpr uint64_t kNarrowKb = R % 2 == 0 ? 512 : R >= 7 ? 256 : 64;
+            constexpr uint64_t kGeneralKb = R == 3 ? 1536 : R == 5 ? 512 : kNarrowKb;
+            if (kb < kNarrowKb) return go(k_query_r<V, R, kNarrow, kCodes>);
+            if (kb < kGeneralKb || other) return false;
+            if constexpr (kGeneralKb < 1024) {
+                if (kb < 1024) return go(k_query_r<V, R, kWideKeep, kCodes>);
+            }
+            return go(k_query_r<V, R, kWide, kCodes>);
+        }
     } else {
-        if (kb < 1024) return exact ? go(k_query_r<V, R, kWideKeep, true>) : go(k_query_r<V, R, kWideKeep, false>);
-        return exact ? go(k_query_r<V, R, kWide, true>) : go(k_query_r<V, R, kWide, false>);
+        if (!aligned || (other && exact && R <= 12)) return false;
+        if (kb < 1024) return exact ? go(k_query_r<V, R, kWideKeep, kFlags>) : go(k_query_r<V, R, kWideKeep, kCodes>);
+        return exact ? go(k_query_r<V, R, kWide, kFlags>) : go(k_query_r<V, R, kWide, kCodes>);
     }
 }
 
-bool launch_query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, cudaStream_t st) {
+bool launch_query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, bool aligned,
+                    cudaStream_t st) {
     switch (Q.r) {
 #define BURR_QUERY_R(R) \
-    case R: return query_r<R>(Q, keys, out, n, grid, st);
+    case R: return query_r<R>(Q, keys, out, n, grid, aligned, st);
         BURR_QUERY_R(1) BURR_QUERY_R(2) BURR_QUERY_R(3) BURR_QUERY_R(4) BURR_QUERY_R(5) BURR_QUERY_R(6)
         BURR_QUERY_R(7) BURR_QUERY_R(8) BURR_QUERY_R(9) BURR_QUERY_R(10) BURR_QUERY_R(11) BURR_QUERY_R(12)
         BURR_QUERY_R(13) BURR_QUERY_R(14) BURR_QUERY_R(15) BURR_QUERY_R(16) BURR_QUERY_R(20) BURR_QUERY_R(24)
@@ -418,17 +478,24 @@ cudaError_t launch_query(const QueryDesc &Q, uint32_t vbytes, const uint64_t *ke
     const unsigned grid = grid_for(n, kQThreads, 152u * 64u);
     // 32-byte reads when every table of the structure starts on 32 bytes (a caller's allocator may
     // give others); the library allocates every table to a multiple of 32 bytes
-    bool wide = true;
+    bool aligned = true;
     for (uint32_t l = 0; l <= Q.layers; ++l)
-        if (Q.m[l] != 0 && ((uintptr_t)Q.z[l] & 31u) != 0) wide = false;
-    if (wide && launch_query_r(Q, keys, out, n, grid, st)) return cudaGetLastError();
-    auto go = [&](auto *any, auto *codes, auto *v) {
-        (Q.mode == BURR_THRESH_1PLUS ? any : codes)<<<grid, kQThreads, 0, st>>>(Q, keys, v, n);
+        if (Q.m[l] != 0 && ((uintptr_t)Q.z[l] & 31u) != 0) aligned = false;
+    if (launch_query_r(Q, keys, out, n, grid, aligned, st)) return cudaGetLastError();
+    // any width, plane by plane.  Fixed to a mode: r = 3, 4*10^6 keys of 1 MB 71 / 82 us, r = 9 with 1+-bit
+    // thresholds 109 / 124; but r = 5 of 1.9 MB 5.2 / 4.5 us for 10,007 keys, r = 31 15.2 / 10.8, r = 9 with
+    // 1+-bit thresholds 9.6 / 9.0 for 10^5 keys of 5.6 MB
+    const bool exact = Q.mode == BURR_THRESH_1PLUS;
+    const bool few = n < kGroupKeys && Q.m[0] <= 64ull * Q.B;   // keys, and flag words
+    const bool either = (!aligned && Q.r != 8 && Q.r != 16) || Q.r > 16 || !usual_load(Q) ||
+                        (exact ? few || (Q.m[0] / 64) * Q.r * 8 >= 1 << 20 : Q.r == 5);
+    auto go = [&](auto *codes, auto *flags, auto *any, auto *v) {
+        (either ? any : exact ? flags : codes)<<<grid, kQThreads, 0, st>>>(Q, keys, v, n);
     };
     switch (vbytes) {
-    case 1: go(k_query<uint8_t, false>, k_query<uint8_t, true>, (uint8_t *)out); break;
-    case 2: go(k_query<uint16_t, false>, k_query<uint16_t, true>, (uint16_t *)out); break;
-    default: go(k_query<uint32_t, false>, k_query<uint32_t, true>, (uint32_t *)out); break;
+    case 1: go(k_query<uint8_t, kCodes>, k_query<uint8_t, kFlags>, k_query<uint8_t, kEither>, (uint8_t *)out); break;
+    case 2: go(k_query<uint16_t, kCodes>, k_query<uint16_t, kFlags>, k_query<uint16_t, kEither>, (uint16_t *)out); break;
+    default: k_query<uint32_t, kEither><<<grid, kQThreads, 0, st>>>(Q, keys, (uint32_t *)out, n); break;
     }
     return cudaGetLastError();
 }
