@@ -368,10 +368,9 @@ constexpr uint32_t kBacksubCtasPerSm = BURR_BACKSUB_CTAS_PER_SM;
 // launch (0: one launch).  The rest go in a second launch on a stream of its
 // own, started together with the first, and the first launch's
 // back-substitution starts as soon as the first launch ends, in the SMs that
-// the band's last partitions leave idle.  Measured at 10^9 keys (r = 8): one
-// launch 96.1 ms per build; 70 / 80 / 90 / 95 percent 95.3 / 95.0 / 94.2 /
-// 94.3 ms (the layer-0 band takes 1.2 ms longer, the back-substitution after
-// it 3.1 ms less).
+// the band's last partitions leave idle.  Builds, ms, one launch / 90 percent: 10^9 keys
+// 69.8 / 68.6; 3*10^8 r = 8 23.8 / 22.9, 1+-bit r = 16 31.8 / 30.8, r = 32 29.4 / 30.5, 1+-bit 38.9 / 35.7 (the
+// layer-0 band takes 1 to 2% longer, what follows it less).
 #ifndef BURR_BAND_SPLIT
 #define BURR_BAND_SPLIT 90
 #endif

@@ -32,20 +32,25 @@
 //     dependency: the lowest-offset row of the bucket cannot be kept, and the
 //     threshold above it is taken at once.
 //
-// What bounds it: with every warp slot taken, the ALU pipe (integer logic,
-// selects and compares at half rate) and the queue of shuffles, maxima and
-// shared-memory stores, at about 37 cycles of an SM quarter per slot; with few
-// partitions, the chain of a step (bit test, warp maximum, shuffle, XOR: about 75
-// cycles per slot) and of the bookkeeping between blocks of slots.  Layer-0 band, ms (r = 8
-// unless said), against the streaming insertion that it replaces (32 lanes
-// eliminating one row each against a band in shared memory, a 128-bit
-// compare-and-swap per step, every bucket as long as its longest chain, a
-// dependent bucket inserted again):
-//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 2.9 (in segments 0.79)
-//   10^6 keys (16 partitions)                     6.57 -> 3.9 (in segments 1.23)
+// What bounds it: with every CTA slot taken, the ALU pipe (integer logic, selects
+// and compares at half rate): 77% of its peak and 66% of the issue slots (3*10^7 keys
+// in 3,608 partitions), 43 warp instructions and about 61 cycles of an SM quarter per
+// slot (10^9 keys).  A step is 37 of these cycles; the rest is the bookkeeping
+// between blocks of slots, staging, writing out, and waits at the pair's barrier.
+// With few partitions, the chain of a warp alone: about 6.6 us per bucket, 107
+// cycles per slot, of which the step (bit test, warp maximum, shuffle, XOR) is about
+// 75.  Layer-0 band, ms (r = 8 unless said), against the streaming insertion
+// that it replaces (32 lanes eliminating one row each against a band in shared
+// memory, a 128-bit compare-and-swap per step, every bucket as long as its longest
+// chain, a dependent bucket inserted again; sparse layers still take it, see
+// burr_band_stream.cuh):
+//   5*10^4 keys, r = 3 (1 partition)              4.59 -> 2.9 (in segments 0.71)
+//   10^6 keys (16 partitions)                     6.57 -> 3.9 (in segments 1.24)
 //   10^7 keys, r = 16, 1+-bit, searched cuts      13.7 -> 6.1
 //   10^8 keys (1504 partitions)                   8.33 -> 6.2;  1+-bit 16.3 -> 9.0
-//   10^9 keys (15034 partitions)                  63.7 -> 47.4
+//   10^9 keys (15034 partitions)                  63.7 -> 47.5
+//   10^8 keys, r = 17..32                         8.4 -> 6.9;  1+-bit 16.2 -> 9.6
+//   10^8 keys at load 1.3                         13.7 -> 6.9;  1+-bit 50.2 -> 22.3
 #include <algorithm>
 #include <cmath>
 
@@ -66,10 +71,11 @@ constexpr unsigned kFull = 0xffffffffu;
 // fetches (layer-0 band of 10^9 keys 104.7 ms against 60.9 with 4 slots and
 // one copy).  Now 4 / 8 / 16 slots: 47.4 / 47.5 / 50.4 ms, 10^6 keys 1.27 / 1.31 / 1.65.
 constexpr uint32_t kUnrollSlots = 4;
-// CTAs (partitions) per SM that the registers allow: 16 (64 registers a thread,
-// 76 bytes of spills) where partitions outnumber what fits, else 14 (72, none).
-// Layer-0 band, ms, 16 / 14: 10^9 keys 47.4 / 50.1 (12: 55.4 before other
-// changes); 10^8 6.37 / 6.33, 1+-bit 9.41 / 9.33; 10^6 1.31 / 1.27.
+// CTAs (partitions) per SM that the registers allow: 16 (64 registers a thread, 92
+// bytes of spill loads with one-byte values, 48 with wider ones) where partitions
+// outnumber what fits, else 14 (72, 56 and 20).  Builds, ms, 16 / 14: 10^9 keys 68.6 / 70.4; 3*10^8
+// r = 8 22.9 / 22.9, r = 16 25.2 / 25.5, 1+-bit 30.8 / 31.8, r = 32 30.5 / 29.6, 1+-bit 35.7 / 35.5.  Layer-0 band with all
+// partitions resident: 10^8 keys 6.37 / 6.33, 1+-bit 9.41 / 9.33, 10^6 1.31 / 1.27.
 constexpr int kManyCtas = 16, kFewCtas = 14;
 constexpr uint64_t kFewParts = 152 * kFewCtas;
 
@@ -934,21 +940,18 @@ __global__ void __launch_bounds__(128) k_band_finish(BandArgs<V> a, uint32_t npa
 }
 
 // Segments of a launch: buckets per segment (0: whole partitions) and segments
-// of the longest partition.  A launch of few partitions is bound by their
-// chains (about 7.4 us per bucket, 512 buckets in a default partition) while most
-// of the chip idles.  Segments of 32 buckets are passed 2-6 times until the last
-// one has met its stored run; measured, layer-0 band in ms, whole partitions /
-// segments: 5*10^4 keys (1 partition) 3.2 / 0.8, 10^6 (16) 3.9 / 1.27, 10^7 (151,
-// segments of 64) 4.2 / 2.1, 3*10^7 (451, segments of 128) 4.3 / 3.3.  The passes
-// bring about 23 buckets' work per segment, so a launch that fills the chip as it
-// is keeps whole partitions: the segment length grows until segments and
-// partitions fit the resident CTAs (16 per SM) together (a cap of half / 1.5
-// times that: 2.79 / 2.85 against 2.34 ms at 10^7 keys before other changes; 10^8
-// keys, 1504 partitions, in segments of 128: 7.8 against 6.8).  With exact
-// thresholds the right-hand sides of different bumped rows survive for 58
-// buckets on average, so segments pay with fewer of them: 5*10^4 keys 4.0 / 1.5,
-// 2*10^5 5.7 / 2.0, 10^6 6.2 / 4.0, 3*10^6 6.5 / 5.3, 6*10^6 (91 partitions, segments
-// of 128; of 256: 6.7) 6.3 / 5.4, but 10^7 6.4 / 7.1.
+// of the longest partition.  A launch of few partitions is bound by their chains
+// (512 buckets in a default partition) while most of the chip idles.  Segments of 32
+// buckets are passed 2 to 6 times until the last one has met its stored run.  Layer-0
+// band, ms, whole partitions / segments: 5*10^4 keys (1 partition) 3.2 / 0.71, 10^6 (16) 3.9 / 1.24,
+// 10^7 (151, segments of 64) 4.2 / 1.88, 3*10^7 (451, segments of 128) 4.3 / 3.15.
+// The passes bring about 23 buckets' work per segment, so a launch that fills the
+// chip as it is keeps whole partitions: the segment length grows until segments and
+// partitions together are at most kSegCap (2,128 CTAs are resident; caps of 1,216 / 2,128 / 2,432 / 3,648: 10^7 keys
+// 1.85 / 1.88 / 1.88 / 2.39, 3*10^7 3.95 / 3.55 / 3.15 / 3.15).  With exact thresholds the right-hand
+// sides of different bumped rows survive for 58 buckets on average, so segments pay
+// with fewer of them: 5*10^4 keys 4.0 / 1.5, 10^6 6.2 / 4.0, 6*10^6 (91 partitions, segments of 128) 6.3 /
+// 5.4, but 10^7 6.4 / 7.1.
 constexpr uint64_t kSegCap = 2432, kSegMin = 32, kSegCapExact = 460, kSegMaxExact = 128;
 // Passes before the last one: enough for runs that meet after 190 buckets.
 inline uint32_t seg_passes(uint32_t seg) { return 1 + (190 + seg - 1) / seg; }
@@ -1058,7 +1061,7 @@ cudaError_t band_impl(const LayerDesc &L, const uint64_t *keys, const V *vals, c
             kernel<<<(unsigned)p.parts, 64, 0, st>>>(a);
             return cudaGetLastError();
         };
-        // (a part of a split layer runs beside the rest, at its registers)
+        // (a part of a split layer runs beside the rest, at its registers; a shard's range does as well)
         const bool whole = bv ? bv->slots != 0 : L.part_lo == 0 && L.part_hi == 0;
         return whole && p.parts <= kFewParts ? go(k_band<V, kFewCtas>) : go(k_band<V, kManyCtas>);
     }

@@ -242,8 +242,9 @@ k_query_r(QueryDesc Q, const uint64_t *__restrict__ keys, V *__restrict__ out, u
 // G = R / 4 neighbouring lanes read together, for the keys of the group in turn;
 // each lane evaluates four planes of all G keys, and the group exchanges the
 // results.  A load is then one request per key and block instead of one per
-// sector: the requests of an SM to L2 bound the kernel (84% of their peak, 22%
-// of the returning sectors', 10^8 keys of r = 8).  The bumped keys (2 in 100)
+// sector: those requests of an SM to L2 bound the kernel of one lane per key.
+// Now they are at 58% of their peak, the sectors returned at 26%, L1's data pipe at 76% and the ALU
+// at 75% (1.6*10^7 keys of a 30 MB table, r = 8).  The bumped keys (2 in 100)
 // go on lane by lane in the deeper layers.  Measured against one lane per key:
 // r = 8, 10^8 keys of a 100 MB table 1.71 -> 1.58 ms, 2*10^7 of a 1 MB table 445 ->
 // 290 us (1+-bit); r = 16, 5*10^6 of 20 MB 182 -> 118 us, 1+-bit 261 -> 130; r = 32,
