@@ -389,10 +389,10 @@ namespace {
 // quarter are bumped and the wide loads of their windows are wasted: r = 15 in 560 KB takes 1.46 times as long as
 // plane by plane; at 0.8 hardly a bucket is flagged).  There, and for tables off 32-byte boundaries (of a
 // caller's allocator), the widths that lost keep to kernels of either mode.  Over 1,824 combinations of width,
-// mode and sizes at each of the loads 0.8, 0.97, 1.05, 1.1, 1.3, by the lines alone 80, 27, 30, 87, 223 are more
-// than 4% slower than plane by plane (r = 1, 8, 16: than one lane per key), with the exception 8, -, 7, 12, 7;
-// at 1.0, 1.015, 1.03 6, 6, 8 are.
-inline bool usual_load(const QueryDesc &Q) { return Q.load >= 0.99f && Q.load <= 1.04f; }
+// mode and sizes at each of the loads 0.8, 0.97, 1.04, 1.05, 1.1, 1.3, by the lines alone 80, 27, 28, 30, 87, 223
+// are more than 4% slower than plane by plane (r = 1, 8, 16: than one lane per key), with the exception at
+// 0.8, 0.97, 1.05, 1.1, 1.3 8, 12, 7, 12, 7; at 1.0, 1.015, 1.03, by the lines, 6, 6, 8 are.
+inline bool usual_load(const QueryDesc &Q) { return Q.load >= 0.995f && Q.load <= 1.03f; }
 constexpr uint64_t kGroupKeys = 1 << 15, kGroupKeys16 = 256;
 template <int R>
 bool query_r(const QueryDesc &Q, const uint64_t *keys, void *out, uint64_t n, unsigned grid, bool aligned, cudaStream_t st) {

@@ -50,7 +50,8 @@ uint64_t first_layer_slots(uint64_t n, double alpha) {
 
 // Device bytes a build of n keys holds at its peak: the input copies, the
 // sorted copies and the sort's scratch, the band of every partition, the
-// bumped lists and the tables (a conservative model of the build's arena).
+// bumped lists and the tables (a conservative model of the build's arena: the
+// band's segments, about 2 KB per 4,096 slots or more, lie within it).
 uint64_t build_estimate(uint64_t n, uint32_t r, double alpha) {
     const uint64_t vb = vbytes_of(r);
     const uint64_t m = first_layer_slots(n, alpha);
